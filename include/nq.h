@@ -106,14 +106,14 @@ typedef struct nq_queen {
                              integer multiply-adds, balancing the FMA and ALU pipes */
 #define NQ_LAYOUT_REGM 7  /* REG with the same multiply-add arithmetic, the control tail as
                              one predicated block */
-#define NQ_LAYOUT_REGP 8  /* REGM without the last-row rule: the row N-1 child is pushed and
-                             a solution is the step that fills every column (one compare
-                             instead of a population count; one more frame per thread).
-                             The default. */
+#define NQ_LAYOUT_REGP 8  /* REG with a one-row look-ahead: a child is entered only if its
+                             own row and the row after it have a free column. The default.
+                             (Its diagnostic build takes every step, as REGM without the
+                             last-row rule: a solution is the step that fills every column.) */
 #define NQ_LAYOUT_REGZ 9  /* REGM with each frame saved and restored as four 32-bit words
                              in four arrays, every word in its lane's own bank: zero bank
                              conflicts for any set of active lanes (256-thread blocks) */
-#define NQ_LAYOUT_REGPZ 10 /* REGP with REGZ's split-word frames */
+#define NQ_LAYOUT_REGPZ 10 /* REGZ with the row N-1 child pushed instead of the last-row rule */
 #define NQ_LAYOUT_AVAIL 11 /* the avail-only stack: one 32-bit word per level (the level's
                               candidates), the parent state restored by undoing the
                               placement; 4 bytes of shared memory per level, every access
@@ -446,8 +446,8 @@ int nq_probe_smem(int kind, uint32_t lane_mask, int density, int iters, int slot
 /*
  * Byte offset, within a block's dynamic shared memory, of 32-bit field `field`
  * (0 cols, 1 ld, 2 rd, 3 avail) of stack slot `slot` (slot 0 holds a sentinel
- * frame; the production builds of REGM, REGP, REGZ and REGPZ keep a second one
- * in slot 1) of thread `thread`, for a block of `block` threads with `slots`
+ * frame; the production builds of REGM, REGZ and REGPZ keep a second one in
+ * slot 1) of thread `thread`, for a block of `block` threads with `slots`
  * slots per thread, in layout `layout` (0: the default) -- the addresses the
  * search kernel computes (the kernel and this call share one definition).
  * Whole-frame layouts (PAPER, REG, REGM, REGP, WT, WTM) put slot k of thread t

@@ -1,0 +1,285 @@
+// lookahead.cu -- the default search form's production kernel (layout REGP):
+// Algorithm 2 with a one-row look-ahead.
+//
+// A child is entered only if its own row has a free column AND the row after
+// that would still have one under the child's state. Both tests are NORs of
+// the same masks, and the second one's shifted masks are the ones that the
+// child's frame needs anyway, so the look-ahead costs one logic instruction
+// and no state. It removes a fifth of the steps and a quarter of the stack
+// traffic at N = 18 (counted on a sampled tree: 14.8 M steps, 9.4 M entered
+// frames -> 11.9 M, 7.3 M).
+//
+// What bounds it (N = 18, d = 7, 7.4 M subproblems in one launch, 20.0 ms
+// against 26.2 ms for the same search without look-ahead): issue slots 85 %, the ALU pipe 84 % and the shared
+// memory data path 86 % at once, so a step has to lose instructions, ALU work
+// and stack traffic together to get faster. Tried and slower, all on that
+// workload: high-half multiplies in place of the right shifts (22.6 ms), a
+// compare for the last column in place of the population count (22.4 ms),
+// dropping the candidates that a forced next row rules out (25.7 ms: five more
+// instructions for 16 % fewer steps).
+#include "nq_internal.h"
+
+namespace nqi {
+namespace {
+
+constexpr int kLookSteps = 31;  // steps between bookkeeping points
+
+// The sentinel frame, in slot 0 of every stack: whatever candidate bit p is
+// taken, cols + p, L + 2p and R + p/2 together cover all 32 bits (each of the
+// three patterns keeps one bit of every pair of columns, also where p's carry
+// moves it), so a child is never live. All 32 bits are candidates, which holds
+// 32 idle steps: one frame lasts a whole round.
+constexpr uint32_t kSentC = 0x55555555u, kSentL = 0xAAAAAAAAu, kSentR = 0x55555555u;
+constexpr uint32_t kSentAv = 0xFFFFFFFFu;
+static_assert(kLookSteps < 32, "an idle lane must not use up the sentinel's candidates");
+
+extern __shared__ __align__(16) unsigned char look_smem[];
+
+__device__ __forceinline__ void look_error(int *status, int code) {
+    if (status) atomicCAS(status, 0, code);
+}
+
+// One step. The top frame is in registers: c = columns taken (columns >= N
+// pre-set), L and R = the diagonals as they reach the NEXT row before this
+// row's queen is placed (kept shifted, so that placing p adds 2p and p/2 to
+// them and nothing else), av = candidates left. (c, L, R, av) of a frame with
+// candidates left is saved in 16 bytes of the lane's stack.
+//   p          the lowest candidate, ar the others
+//   c2 l2 r2   the child's masks, a2 its free columns
+//   L2 R2      the same masks one row on, b2 that row's free columns
+// Every sum is of disjoint bits, so the integer multiply-adds by the run-time
+// multipliers m1 = 1, m2 = 2, mneg = 2^32 - 1 are exact; they issue on the FMA
+// pipe, which this integer loop would otherwise leave idle.
+// A solution is counted when the child has one free column left (rows 0..N-2
+// hold queens) and its row has it free; such a child may be entered too (its
+// look-ahead row does not exist), which costs a step and finds nothing.
+__device__ __forceinline__ void look_step(uint32_t &c, uint32_t &L, uint32_t &R, uint32_t &av,
+                                          uint32_t &top, const uint32_t stride, uint32_t &s32,
+                                          const uint32_t m1, const uint32_t m2,
+                                          const uint32_t mneg) {
+    const uint32_t p = av & (av * mneg);
+    const uint32_t ar = p * mneg + av;
+    const uint32_t c2 = p * m1 + c;
+    const uint32_t l2 = L + 2u * p;
+    const uint32_t r2 = (p >> 1) + R;
+    const uint32_t L2 = l2 * m2;
+    const uint32_t R2 = r2 >> 1;
+    const uint32_t pc = (uint32_t)__popc(c2);
+    // %0..%5 c, L, R, av, top, s32; %6 l2, %7 pc, %8 ar, %9 c2, %10 r2,
+    // %11 stride, %12 L2, %13 R2. lop3 table 0x01: NOR of its three inputs;
+    // the predicate beside the result says that it is not zero (and-ed with
+    // the last operand).
+    asm volatile(
+        "{\n\t"
+        ".reg .pred ptrue, plive, ppush, pcnt, psave, ppop;\n\t"
+        ".reg .b32 a2, b2;\n\t"
+        "setp.eq.u32 ptrue, 0, 0;\n\t"
+        "lop3.and.b32 a2|plive, %9, %6, %10, 0x01, ptrue;\n\t"    // the child's row has a column
+        "lop3.and.b32 b2|ppush, %9, %12, %13, 0x01, plive;\n\t"   // ... and so has the row after
+        "setp.eq.and.u32 pcnt, %7, 31, plive;\n\t"                // one column left, and free: a solution
+        "@pcnt add.u32 %5, %5, 1;\n\t"
+        "setp.ne.and.u32 psave, %8, 0, ppush;\n\t"                // entered with candidates left: save
+        "setp.eq.and.u32 ppop, %8, 0, !ppush;\n\t"                // nothing left, nothing entered: pop
+        "@psave st.shared.v4.u32 [%4], {%0, %1, %2, %8};\n\t"
+        "@psave add.u32 %4, %4, %11;\n\t"
+        "@ppop sub.u32 %4, %4, %11;\n\t"
+        "selp.b32 %3, a2, %8, ppush;\n\t"
+        "@ppush mov.b32 %0, %9;\n\t"
+        "@ppush mov.b32 %1, %12;\n\t"
+        "@ppush mov.b32 %2, %13;\n\t"
+        "@ppop ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n\t"
+        "}"
+        : "+r"(c), "+r"(L), "+r"(R), "+r"(av), "+r"(top), "+r"(s32)
+        : "r"(l2), "r"(pc), "r"(ar), "r"(c2), "r"(r2), "r"(stride), "r"(L2), "r"(R2)
+        : "memory");
+}
+
+// The persistent search: every warp takes ranges of `kRange x claim` record
+// indices (the first one by its number, the others from the work cursor) and
+// hands them to its lanes as they become idle. One atomic serves a whole
+// range, and a launch whose records fit the first ranges needs no cursor.
+// Consecutive ranges go to different blocks first, so that few records spread
+// over the SMs.
+template <bool STREAM>
+__device__ __forceinline__ void look_body(const SearchArgs &a) {
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(look_smem);
+    const uint32_t stride = stack_slot_offset(blockDim.x, 0u, 1u, 16u);
+    const uint32_t base = sbase + stack_slot_offset(blockDim.x, threadIdx.x, 0u, 16u);
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const uint32_t m1 = a.mul[0], m2 = a.mul[1], mneg = a.mul[2];
+    const uint32_t range = kLookRange * (a.claim > 0 ? (uint32_t)a.claim : 1u);
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+
+    uint32_t c = kSentC, L = kSentL, R = kSentR, av = kSentAv, top = base;
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
+                 :
+                 : "r"(base), "r"(c), "r"(L), "r"(R), "r"(av)
+                 : "memory");
+
+    bool busy = false;          // a subproblem is being searched
+    uint64_t idx = 0;           // its record
+    uint32_t wn = 0;            // its weight | N << 2
+    uint64_t sol = 0;
+    uint64_t wsum = 0;          // weighted solutions not yet in totals[wsum_n]
+    uint32_t wsum_n = 0;
+    // the warp's range (the same in every lane)
+    uint64_t next = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * range;
+    uint32_t rem = next < a.n ? (uint32_t)(a.n - next < range ? a.n - next : range) : 0u;
+    bool exhausted = a.cursor == nullptr;
+    uint32_t waits = 0;
+
+    auto finish = [&](uint64_t i, uint64_t s, uint32_t w_n) {
+        if (a.by_tag) {  // split subproblems: the count goes to the parent named by the tag
+            const uint64_t parent = __ldg(reinterpret_cast<const uint32_t *>(a.pre + i) + 3) >> 12;
+            if (parent >= a.n_tags)
+                look_error(a.status, NQ_EINVAL);
+            else if (a.counts && s)
+                atomicAdd(reinterpret_cast<unsigned long long *>(&a.counts[parent]),
+                          (unsigned long long)s);
+        } else if (a.counts) {
+            a.counts[i] = s;
+        }
+        if (a.totals && s) {
+            const uint32_t n = w_n >> 2;
+            if (n != wsum_n && wsum != 0) {
+                atomicAdd(reinterpret_cast<unsigned long long *>(&a.totals[wsum_n]),
+                          (unsigned long long)wsum);
+                wsum = 0;
+            }
+            wsum_n = n;
+            wsum += (uint64_t)(w_n & 3u) * s;
+        }
+    };
+
+    for (;;) {
+        const bool idle = top == base;  // on the sentinel
+        if (idle) {
+            if (busy) finish(idx, sol, wn);
+            busy = false;
+            c = kSentC;
+            L = kSentL;
+            R = kSentR;
+            av = kSentAv;
+        }
+        bool need = idle;
+        unsigned need_mask = __ballot_sync(~0u, need);
+        while (need_mask) {
+            if (rem == 0u) {
+                if (exhausted) break;
+                unsigned long long f = 0;
+                if (lane == 0) f = atomicAdd(a.cursor, (unsigned long long)range);
+                next = __shfl_sync(~0u, f, 0) + warps * range;
+                if (next >= a.n) {
+                    exhausted = true;
+                    break;
+                }
+                rem = a.n - next < range ? (uint32_t)(a.n - next) : range;
+            }
+            uint32_t ready = rem;
+            if (STREAM) {  // streamed input: only what has been published may be read
+                unsigned long long v = 0;
+                if (lane == 0)
+                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v)
+                                 : "l"(a.published) : "memory");
+                v = __shfl_sync(~0u, v, 0);
+                ready = v <= next ? 0u : v - next < rem ? (uint32_t)(v - next) : rem;
+                if (ready == 0u) break;
+            }
+            const uint32_t rank = __popc(need_mask & lt_mask);
+            if (need && rank < ready) {
+                const uint64_t pi = a.order ? a.n - 1 - (next + rank) : next + rank;
+                uint4 P;
+                if (STREAM)  // (a line may have been cached before its copy arrived)
+                    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(P.x), "=r"(P.y), "=r"(P.z), "=r"(P.w)
+                                 : "l"(a.pre + pi)
+                                 : "memory");
+                else
+                    P = __ldg(reinterpret_cast<const uint4 *>(a.pre) + pi);
+                const uint32_t n = (P.w >> 2) & 31u, d = (P.w >> 7) & 31u, w = P.w & 3u;
+                const uint32_t last = (n >= 1u) ? (0xFFFFFFFFu >> (32u - n)) : 0u;
+                const bool ok = n >= 1u && (a.expect_n == 0 || (int)n == a.expect_n) &&
+                                (w == 1u || w == 2u) && d <= n && (P.x & ~last) == 0u &&
+                                (uint32_t)__popc(P.x) == d;
+                // the stack: the sentinel and the ancestors of rows d..N-2
+                if (!ok) {
+                    look_error(a.status, NQ_EINVAL);
+                    finish(pi, 0, 0);
+                } else if (d + 1u < n && (int)(n - d) > a.slots) {
+                    look_error(a.status, NQ_ESTACK);
+                    finish(pi, 0, 0);
+                } else {
+                    const uint32_t c0 = P.x | ~last;
+                    const uint32_t l0 = P.y, r0 = P.z & last;
+                    const uint32_t a0 = ~(c0 | l0 | r0);
+                    if (d == n) {
+                        finish(pi, 1, w | (n << 2));  // the prefix is a solution
+                    } else if (d + 1u == n || a0 == 0u) {
+                        finish(pi, (uint64_t)__popc(a0), w | (n << 2));  // last row or dead end
+                    } else {
+                        idx = pi;
+                        wn = w | (n << 2);
+                        sol = 0;
+                        busy = true;
+                        c = c0;
+                        L = l0 << 1;
+                        R = r0 >> 1;
+                        av = a0;
+                        top = base + stride;
+                        need = false;
+                    }
+                }
+            }
+            const uint32_t asked = __popc(need_mask);
+            const uint32_t taken = asked < ready ? asked : ready;
+            next += taken;
+            rem -= taken;
+            need_mask = __ballot_sync(~0u, need);
+        }
+        if (need_mask == ~0u) {  // the whole warp is idle
+            if (!STREAM || (exhausted && rem == 0u)) break;
+            // bounded wait for the host to publish more
+            if (++waits > kMaxPublishWaits) {
+                look_error(a.status, NQ_ETIMEOUT);
+                break;
+            }
+            __nanosleep(256);
+            continue;
+        }
+
+        uint32_t s32 = 0;
+#pragma unroll
+        for (int j = 0; j < kLookSteps; ++j) look_step(c, L, R, av, top, stride, s32, m1, m2, mneg);
+        sol += s32;
+    }
+
+    if (a.totals) {
+        const unsigned has = __ballot_sync(~0u, wsum != 0);
+        if (has) {
+            const uint32_t n0 = __shfl_sync(~0u, wsum_n, __ffs(has) - 1);
+            if (__all_sync(~0u, wsum == 0 || wsum_n == n0)) {
+                uint64_t v = wsum;
+                for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(~0u, v, o);
+                if (lane == 0)
+                    atomicAdd(reinterpret_cast<unsigned long long *>(&a.totals[n0]),
+                              (unsigned long long)v);
+            } else if (wsum) {
+                atomicAdd(reinterpret_cast<unsigned long long *>(&a.totals[wsum_n]),
+                          (unsigned long long)wsum);
+            }
+        }
+    }
+}
+
+__global__ void __maxnreg__(48) look_kernel(const SearchArgs a) { look_body<false>(a); }
+__global__ void __maxnreg__(48) look_kernel_stream(const SearchArgs a) { look_body<true>(a); }
+
+}  // namespace
+
+void *look_kernel_ptr(bool stream) {
+    return stream ? reinterpret_cast<void *>(&look_kernel_stream)
+                  : reinterpret_cast<void *>(&look_kernel);
+}
+
+}  // namespace nqi

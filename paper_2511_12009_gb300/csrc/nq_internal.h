@@ -103,8 +103,9 @@ __host__ __device__ constexpr uint32_t stack_word_offset(bool split, uint32_t bl
     return split ? ((4u * slot + field) * block + thread) * 4u
                  : stack_slot_offset(block, thread, slot, 16u) + 4u * field;
 }
-// The search form the library uses when none is configured: REGM with the
-// last row pushed (measured 7 % faster than REGM at N = 18 on GB300).
+// The search form the library uses when none is configured: REGP, whose
+// production kernel looks one row ahead (lookahead.cu; N = 18, d = 7 on GB300:
+// 20 ms, REGM 28.9 ms).
 constexpr int NQ_LAYOUT_DEFAULT_SEARCH = NQ_LAYOUT_REGP;
 // The split-word kernels are built for this block size (their word stride is
 // an immediate offset).
@@ -181,6 +182,11 @@ struct ServeArgs {
     unsigned int *closing;
     int *status;                     // the server's error word (device)
 };
+
+// The production kernel of layout REGP (lookahead.cu), plain or for streamed input.
+void *look_kernel_ptr(bool stream);
+// Records a warp of it takes at once (times SearchArgs::claim).
+constexpr uint32_t kLookRange = 32;
 
 int launch_serve(const ServeArgs &a, int grid, int block, size_t smem, cudaStream_t s);
 int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *smem,

@@ -250,7 +250,7 @@ __device__ __forceinline__ void step_reg(uint32_t &c, uint32_t &l, uint32_t &r, 
 // s32 (updated); %6..%12 = popc(c2) (unused with PUSHLAST), a2, ar, c2, l2,
 // r2, stride.
 //
-// PUSHLAST (layouts REGP, REGPZ): Algorithm 2 without Algorithm 3's last-row
+// PUSHLAST (layout REGPZ): Algorithm 2 without Algorithm 3's last-row
 // rule: the row N-1 child is pushed like any other, and the step that places
 // the last queen is recognised by cols == ~0 (the columns >= N are pre-set),
 // one compare instead of a population count and two predicates. It costs one
@@ -306,6 +306,7 @@ __device__ __forceinline__ void step_regm(uint32_t &c, uint32_t &l, uint32_t &r,
                                           const uint32_t m1, const uint32_t m2,
                                           const uint32_t mneg, const uint32_t mhalf) {
     static_assert(!SPLIT || kZWord == 1024u, "the PTX offsets assume 256-thread blocks");
+    static_assert(SPLIT || !PUSHLAST, "REGP's production build is look_kernel");
     const uint32_t p = av & (av * mneg);
     const uint32_t ar = p * mneg + av;
     const uint32_t c2 = p * m1 + c;
@@ -319,8 +320,6 @@ __device__ __forceinline__ void step_regm(uint32_t &c, uint32_t &l, uint32_t &r,
     : "memory"
     if constexpr (!PUSHLAST && !SPLIT)
         asm volatile(NQ_TAIL(NQ_PRED_LASTROW, NQ_SAVE4, NQ_LOAD4) NQ_OPERANDS);
-    else if constexpr (PUSHLAST && !SPLIT)
-        asm volatile(NQ_TAIL(NQ_PRED_PUSHLAST, NQ_SAVE4, NQ_LOAD4) NQ_OPERANDS);
     else if constexpr (!PUSHLAST && SPLIT)
         asm volatile(NQ_TAIL(NQ_PRED_LASTROW, NQ_SAVEZ, NQ_LOADZ) NQ_OPERANDS);
     else
@@ -1058,26 +1057,26 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
         uint32_t s32 = 0, n32 = 0;
 #pragma unroll
         for (int j = 0; j < kSteps; ++j) {
-            if (kAvail)
+            if constexpr (kAvail)
                 step_avail<DIAG>(c, l, r, av, top, k, s32, n32, m1, m2, mneg, mhalf);
-            else if (kRegm && CONSTR && DIAG)
+            else if constexpr (kRegm && CONSTR && DIAG)
                 step_reg<DIAG, true, true>(c, l, r, av, top, k, s32, n32, m1, m2, mneg, mhalf);
-            else if (kRegm && CONSTR)
+            else if constexpr (kRegm && CONSTR)
                 step_regm_constr(c, l, r, av, top, k.stride, k.table, k.thr, s32, m1, m2, mneg,
                                  mhalf);
-            else if (kRegm && DIAG)
+            else if constexpr (kRegm && DIAG)
                 step_reg<DIAG, false, true, kPushLast, kSplit>(c, l, r, av, top, k, s32, n32, m1,
                                                                m2, mneg, mhalf);
-            else if (kRegm)
+            else if constexpr (kRegm)
                 step_regm<kPushLast, kSplit>(c, l, r, av, top, k.stride, s32, m1, m2, mneg,
                                              mhalf);
-            else if (kReg)
+            else if constexpr (kReg)
                 step_reg<DIAG, CONSTR>(c, l, r, av, top, k, s32, n32);
-            else if (kWt)
+            else if constexpr (kWt)
                 step_wt<DIAG>(c, l, r, av, top, k, s32, n32);
-            else if (kWt32)
+            else if constexpr (kWt32)
                 step_wt32<DIAG, kArith>(c, l, r, av, top, k, s32, n32);
-            else if (kWtm)
+            else if constexpr (kWtm)
                 step_wtm<DIAG>(c, l, r, av, top, k, m1, m2, mneg, mhalf, s32, n32);
             else
                 step_paper<DIAG>(top, k, s32, n32);
@@ -1365,10 +1364,13 @@ void *kernel_ptr() {
         return reinterpret_cast<void *>(&search_kernel<LAYOUT, DIAG, CONSTR>);
 }
 
+template <int LAYOUT, bool DIAG>
+void *stream_ptr() {
+    return reinterpret_cast<void *>(&search_kernel_stream<LAYOUT, DIAG>);
+}
 template <int LAYOUT>
 void *stream_ptr(bool diag) {
-    return diag ? reinterpret_cast<void *>(&search_kernel_stream<LAYOUT, true>)
-                : reinterpret_cast<void *>(&search_kernel_stream<LAYOUT, false>);
+    return diag ? stream_ptr<LAYOUT, true>() : stream_ptr<LAYOUT, false>();
 }
 template <int LAYOUT>
 void *plain_ptr(bool diag) {
@@ -1380,7 +1382,8 @@ void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
     if (stream) {
         switch (layout) {
             case NQ_LAYOUT_REGM: return stream_ptr<NQ_LAYOUT_REGM>(diag);
-            case NQ_LAYOUT_REGP: return stream_ptr<NQ_LAYOUT_REGP>(diag);
+            case NQ_LAYOUT_REGP:
+                return diag ? stream_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(true);
             case NQ_LAYOUT_REGZ: return stream_ptr<NQ_LAYOUT_REGZ>(diag);
             case NQ_LAYOUT_REGPZ: return stream_ptr<NQ_LAYOUT_REGPZ>(diag);
             default: return stream_ptr<NQ_LAYOUT_REG>(diag);
@@ -1402,7 +1405,8 @@ void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
         case NQ_LAYOUT_WT32A: return plain_ptr<NQ_LAYOUT_WT32A>(diag);
         case NQ_LAYOUT_WTM: return plain_ptr<NQ_LAYOUT_WTM>(diag);
         case NQ_LAYOUT_REGM: return plain_ptr<NQ_LAYOUT_REGM>(diag);
-        case NQ_LAYOUT_REGP: return plain_ptr<NQ_LAYOUT_REGP>(diag);
+        case NQ_LAYOUT_REGP:
+            return diag ? kernel_ptr<NQ_LAYOUT_REGP, true, false>() : look_kernel_ptr(false);
         case NQ_LAYOUT_REGZ: return plain_ptr<NQ_LAYOUT_REGZ>(diag);
         case NQ_LAYOUT_REGPZ: return plain_ptr<NQ_LAYOUT_REGPZ>(diag);
         case NQ_LAYOUT_AVAIL: return plain_ptr<NQ_LAYOUT_AVAIL>(diag);
@@ -1419,7 +1423,8 @@ int slots_needed(int layout, int max_n, int min_d) {
     int s = reg ? max_n - 1 - min_d : max_n - min_d;
     if (layout == NQ_LAYOUT_REGP || layout == NQ_LAYOUT_REGPZ) s += 1;
     if (layout == NQ_LAYOUT_AVAIL) s = max_n - 2 - min_d;  // one word per level d..N-3
-    if (layout_regm_family(layout)) s = (s < 1 ? 1 : s) + 1;  // the second sentinel frame
+    // the second sentinel frame (REGP's production kernel needs one only)
+    if (layout_regm_family(layout) && layout != NQ_LAYOUT_REGP) s = (s < 1 ? 1 : s) + 1;
     return s < 1 ? 1 : s;
 }
 

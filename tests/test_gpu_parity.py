@@ -435,3 +435,17 @@ def test_avail_only_stack_limits():
     with pytest.raises(nq.NQError) as e:
         nq.count_ex(dp, 2, 31, cnt, None, None, nq.make_config("avail"))
     assert e.value.code == nq.NQ_EINVAL
+
+
+@pytest.mark.parametrize("n,d,m", [(12, 4, 1), (12, 4, 31), (12, 4, 33), (13, 6, 9999), (15, 7, 0)])
+@pytest.mark.parametrize("claim,order,shape", [(1, 0, {}), (3, 1, {}), (64, 2, {}),
+                                               (1, 0, {"block": 32, "blocks_per_sm": 1})])
+def test_default_form_record_ranges(orc, n, d, m, claim, order, shape):
+    """The default form takes records in ranges of 32 x claim per warp (the first
+    by the warp's number): every record exactly once, at ragged set sizes, for
+    fewer records than one range and for many ranges per warp."""
+    pre = nq.enumerate_prefixes(n, d)
+    want = run(pre, d, n, "reg")[0]
+    m = m or len(pre)
+    got, _, tot = run(pre[:m], d, n, "regp", claim=claim, order=order, **shape)
+    assert np.array_equal(got, want[:m]) and int(tot[n]) == weighted(pre[:m], want[:m])

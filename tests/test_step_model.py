@@ -313,3 +313,73 @@ def test_avail_only_model_equals_oracle(orc, n, d):
     for i, rec in enumerate(pre):
         sol, nodes, _ = search_avail(rec, words)
         assert (sol, nodes) == (int(want[i]), int(want_nodes[i])), (n, d, i)
+
+
+# --- the look-ahead step (layout REGP's production kernel) -------------------------
+
+LOOK_SENTINEL = (0x55555555, 0xAAAAAAAA, 0x55555555, 0xFFFFFFFF)
+
+
+def step_look(state, stack, top):
+    """One look-ahead step: L and R are the diagonals as they reach the next row,
+    a child is entered only if its row and the row after it have a free column,
+    and a solution is a child with one column left that its row has free."""
+    c, L, R, av = state
+    p = av & ((av * M) & M)
+    ar = (p * M + av) & M
+    c2 = (p + c) & M
+    l2 = (L + 2 * p) & M
+    r2 = ((p >> 1) + R) & M
+    L2, R2 = (l2 * 2) & M, r2 >> 1
+    a2 = ~(c2 | l2 | r2) & M
+    b2 = ~(c2 | L2 | R2) & M
+    pcnt = a2 != 0 and popc(c2) == 31
+    ppush = a2 != 0 and b2 != 0
+    if ar != 0 and ppush:
+        stack[top] = (c, L, R, ar)
+        top += 1
+    if ar == 0 and not ppush:
+        top -= 1
+        assert top >= 0, "popped below the stack"
+        c, L, R, av = stack[top]
+    elif ppush:
+        c, L, R, av = c2, L2, R2, a2
+    else:
+        av = ar
+    return (c, L, R, av), top, 1 if pcnt else 0
+
+
+@pytest.mark.parametrize("n,d", [(6, 2), (8, 3), (9, 4), (10, 3), (10, 6), (11, 5), (7, 7),
+                                 (9, 8), (8, 6), (13, 4), (9, 1)])
+def test_look_ahead_model_equals_oracle(orc, n, d):
+    """The oracle's counts, within N - d slots (the sentinel frame and the
+    ancestors of rows d..N-2)."""
+    pre = nq.enumerate_prefixes(n, d)
+    want, _ = orc.count_prefixes(n, orc.prefixes(n, d)[0])
+    slots = max(n - d, 1)
+    for i, rec in enumerate(pre):
+        last = (1 << n) - 1
+        c = int(rec["cols"]) | (~last & M)
+        l, r = int(rec["ld"]), int(rec["rd"])
+        a0 = ~(c | l | r) & M
+        if d == n or d + 1 == n or a0 == 0:
+            sol = 1 if d == n else popc(a0)
+        else:
+            stack, state, top, sol = {0: LOOK_SENTINEL}, (c, (l << 1) & M, r >> 1, a0), 1, 0
+            while top > 0:
+                for _ in range(31):
+                    state, top, s = step_look(state, stack, top)
+                    sol += s
+                    assert top <= slots
+        assert sol == int(want[i]), (n, d, i)
+
+
+def test_look_ahead_sentinel_holds_32_idle_steps():
+    """Every bit is a candidate of the sentinel and none has a live child, so one
+    frame lasts a 31-step round from any step of the round before."""
+    stack, state, top = {0: LOOK_SENTINEL}, LOOK_SENTINEL, 0
+    for _ in range(31):
+        state, top, s = step_look(state, stack, top)
+        assert s == 0 and top == 0 and state[3] != 0
+    with pytest.raises(AssertionError, match="below"):
+        step_look(state, stack, top)
