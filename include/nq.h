@@ -252,7 +252,9 @@ int nq_total_ex(int N, const nq_config *cfg, uint64_t *total_out, uint64_t *node
  * added into its parent's entry. A prefix's subtree is the disjoint union of
  * its children's subtrees (Section 1), so the results equal nq_count_ex on
  * the prefixes themselves; the split restores load balance when there are
- * few heavy subproblems (fewer than the grid has lanes). Synchronous.
+ * few heavy subproblems (fewer than the grid has lanes). Synchronous. Layout
+ * REGP's production build splits the subtrees on the device as it needs to (in
+ * nq_count and nq_count_ex too): there the host only counts the children.
  *   h_prefixes [n] host records, any board sizes, n <= 2^20 (the tag width)
  *   rows       rows to add (capped at N - d per record); -1 = the fewest rows
  *              giving at least 32 children per resident lane of the launch
@@ -262,7 +264,8 @@ int nq_total_ex(int N, const nq_config *cfg, uint64_t *total_out, uint64_t *node
  *              rows d..N-1, as nq_count_ex; runs the diagnostic build)
  *   h_totals   optional [32] out (overwritten): weight x solutions per N
  *   rows_used  optional out: the rows added
- *   timing     optional: enumerate_ms = host split, prefixes = children
+ *   timing     optional: enumerate_ms = host split (REGP: counting the children,
+ *              beside the search), prefixes = children
  * More than 2^27 children is NQ_EOVERFLOW; malformed records NQ_EINVAL.
  */
 int nq_count_split(const nq_prefix *h_prefixes, uint64_t n, int rows, const nq_config *cfg,

@@ -146,13 +146,17 @@ int enqueue_search(const nq_prefix *d_prefixes, uint64_t n, int expect_n, int mi
     // (nq_count_split).
     const bool donate = reg && !constrained && !n_tags && !published && cfg && cfg->donate == 2;
     if (donate && (rc = make_plan(max_n, min_d, diag, constrained, cfg, &p, true))) return rc;
+    if ((rc = plan_records(max_n, min_d, diag, cfg, n, !n_tags, &p))) return rc;
+    if (p.levels && d_counts &&
+        cudaMemsetAsync(d_counts, 0, n * sizeof(uint64_t), s) != cudaSuccess)
+        return NQ_ECUDA;
     const size_t head_bytes = 128 + sizeof(DonateCtl);  // cursor line, counters
     const size_t bytes = donate ? head_bytes + kDonateCap * sizeof(DonateItem) : 64;
-    const bool own = donate || !cursor_ext;
+    const bool own = donate || (!cursor_ext && (!p.look || p.cursor));
     unsigned char *scratch = nullptr;
     if (own && cudaMallocAsync(reinterpret_cast<void **>(&scratch), bytes, s) != cudaSuccess)
         return NQ_ENOMEM;
-    unsigned long long *cursor =
+    unsigned long long *cursor =  // (NULL: the launch needs none)
         own ? reinterpret_cast<unsigned long long *>(scratch) : cursor_ext;
     if (own) rc = cuda_rc(cudaMemsetAsync(scratch, 0, donate ? bytes : 64, s));
     if (!rc && donate && d_counts)
@@ -428,12 +432,30 @@ extern "C" int nq_total(int N, uint64_t *total_out) {
     return nq_total_ex(N, nullptr, total_out, nullptr, nullptr);
 }
 
+// The three timing events of a split call.
+struct SplitEvents {
+    cudaEvent_t e[3] = {};
+    int init() {
+        for (auto &x : e)
+            if (cudaEventCreate(&x) != cudaSuccess) {
+                x = nullptr;
+                return NQ_ECUDA;
+            }
+        return NQ_OK;
+    }
+    ~SplitEvents() {
+        for (auto &x : e)
+            if (x) cudaEventDestroy(x);
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Host-side split: few heavy subproblems (fewer than the grid has lanes) are
 // extended a few rows deeper on the host, every child carrying its parent's
 // index in the tag field, and the kernel adds each child's count into its
 // parent's entry. The subtree of a prefix is the disjoint union of its
-// children's subtrees (Section 1), so the per-parent sums are exact.
+// children's subtrees (Section 1), so the per-parent sums are exact. (The
+// default form's production build splits on the device instead.)
 // ---------------------------------------------------------------------------
 extern "C" int nq_count_split(const nq_prefix *h_prefixes, uint64_t n, int rows,
                               const nq_config *cfg, uint64_t *h_counts, uint64_t *h_nodes,
@@ -456,25 +478,99 @@ extern "C" int nq_count_split(const nq_prefix *h_prefixes, uint64_t n, int rows,
     if (max_n < 1 || max_n > NQ_MAX_N) return NQ_EINVAL;
     const bool diag = h_nodes != nullptr;
     int r = rows, rc;
+    if ((rc = check_parents(h_prefixes, n))) return rc;
     uint64_t m = 0;
-    if (r < 0) {
-        // the fewest rows giving at least 32 children per resident lane
-        Plan p{};
-        if ((rc = make_plan(max_n, min_d, diag, false, cfg, &p))) return rc;
-        const uint64_t want = 32ull * (uint64_t)p.grid * (uint64_t)p.block;
-        for (r = 0; r < max_n - min_d; ++r) {
-            if ((rc = split_prefixes(h_prefixes, n, r, nullptr, nullptr, &m))) return rc;
-            if (m >= want) break;
+    Plan shape{};
+    const int lay = cfg->layout ? cfg->layout : NQ_LAYOUT_DEFAULT_SEARCH;
+    if ((rows < 0 || (lay == NQ_LAYOUT_REGP && !diag)) &&
+        (rc = make_plan(max_n, min_d, diag, false, cfg, &shape)))
+        return rc;
+    // -1: the fewest rows giving at least 32 children per resident lane
+    const uint64_t want = 32ull * (uint64_t)shape.grid * (uint64_t)shape.block;
+    auto count_rows = [&]() -> int {
+        if (r < 0) {
+            for (r = 0; r < max_n - min_d; ++r) {
+                if (const int e = split_prefixes(h_prefixes, n, r, nullptr, nullptr, &m)) return e;
+                if (m >= want) return m > kMaxSplitChildren ? NQ_EOVERFLOW : NQ_OK;
+            }
         }
+        if (const int e = split_prefixes(h_prefixes, n, r, nullptr, nullptr, &m)) return e;
+        return m > kMaxSplitChildren ? NQ_EOVERFLOW : NQ_OK;
+    };
+    auto kid_depth = [&]() {
+        int k = NQ_MAX_N;
+        for (uint64_t i = 0; i < n; ++i)
+            k = std::min(k, std::min((int)NQ_META_N(h_prefixes[i].meta),
+                                     (int)NQ_META_D(h_prefixes[i].meta) + r));
+        return k;
+    };
+    if (shape.look) {
+        // The default form splits subtrees by itself (plan_records): the parents
+        // are searched as they are, and the host only counts the children, while
+        // the search runs unless there might be too many of them to accept.
+        int left = 0;  // rows below the shallowest record
+        for (uint64_t i = 0; i < n; ++i)
+            left = std::max(left, (int)NQ_META_N(h_prefixes[i].meta) -
+                                      (int)NQ_META_D(h_prefixes[i].meta));
+        double most = r < 0 ? (double)want * std::max(left, 1) : (double)n;
+        for (int j = 0; j < r && j < left; ++j) most *= left - j;
+        const bool count_first = std::max(most, (double)n) > (double)kMaxSplitChildren;
+        if (count_first && (rc = count_rows())) return rc;
+        CallCtx ctx;
+        if ((rc = ctx.init())) return rc;
+        nq_prefix *d_pre = nullptr;
+        uint64_t *d_out = nullptr;  // [0..31] totals, [32] status, then the counts
+        if ((rc = ctx.alloc(&d_pre, n * sizeof(nq_prefix)))) return rc;
+        if ((rc = ctx.alloc(&d_out, (34 + n) * sizeof(uint64_t)))) return rc;
+        SplitEvents ev;
+        if ((rc = ev.init())) return rc;
+        cudaEventRecord(ev.e[0], ctx.s);
+        rc = cuda_rc(cudaMemcpyAsync(d_pre, h_prefixes, n * sizeof(nq_prefix),
+                                     cudaMemcpyHostToDevice, ctx.s));
+        if (!rc) rc = cuda_rc(cudaMemsetAsync(d_out, 0, 34 * sizeof(uint64_t), ctx.s));
+        cudaEventRecord(ev.e[1], ctx.s);
+        Plan p{};
+        int *d_status = reinterpret_cast<int *>(d_out + 32);
+        if (!rc)
+            rc = enqueue_search(d_pre, n, 0, max_n - left, max_n, d_out + 34, nullptr, d_out, cfg,
+                                nullptr, ctx.s, &p, d_status);
+        cudaEventRecord(ev.e[2], ctx.s);
+        const auto t_count = Clock::now();
+        const int crc = count_first ? NQ_OK : count_rows();
+        const double count_ms = ms_since(t_count);
+        if (!rc)
+            rc = cuda_rc(cudaMemcpyAsync(h_counts, d_out + 34, n * sizeof(uint64_t),
+                                         cudaMemcpyDeviceToHost, ctx.s));
+        if (!rc && h_totals)
+            rc = cuda_rc(cudaMemcpyAsync(h_totals, d_out, 32 * sizeof(uint64_t),
+                                         cudaMemcpyDeviceToHost, ctx.s));
+        if (cudaStreamSynchronize(ctx.s) != cudaSuccess) return NQ_ECUDA;
+        if (rc || crc) return rc ? rc : crc;
+        const int st = take_status(d_status, ctx.s);
+        if (st) return st;
+        if (rows_used) *rows_used = r;
+        if (timing) {
+            float up = 0, kern = 0;
+            cudaEventElapsedTime(&up, ev.e[0], ev.e[1]);
+            cudaEventElapsedTime(&kern, ev.e[1], ev.e[2]);
+            timing->enumerate_ms = count_ms;
+            timing->upload_ms = up;
+            timing->kernel_ms = kern;
+            timing->prefixes = m;
+            timing->d = kid_depth();
+            timing->layout = p.layout;
+            timing->block = p.block;
+            timing->grid = p.grid;
+            timing->total_ms = ms_since(t_start);
+        }
+        return NQ_OK;
     }
+    if (r < 0 && (rc = count_rows())) return rc;
     std::vector<nq_prefix> kids;
     std::vector<uint64_t> extra;
     if ((rc = split_prefixes(h_prefixes, n, r, &kids, &extra, &m))) return rc;
     const double split_ms = ms_since(t_start);
-    int kid_min_d = NQ_MAX_N;
-    for (uint64_t i = 0; i < n; ++i)
-        kid_min_d = std::min(kid_min_d, std::min((int)NQ_META_N(h_prefixes[i].meta),
-                                                 (int)NQ_META_D(h_prefixes[i].meta) + r));
+    const int kid_min_d = kid_depth();
 
     CallCtx ctx;
     if ((rc = ctx.init())) return rc;
@@ -485,15 +581,9 @@ extern "C" int nq_count_split(const nq_prefix *h_prefixes, uint64_t n, int rows,
     if (diag && (rc = ctx.alloc(&d_nodes, n * sizeof(uint64_t)))) return rc;
     if ((rc = ctx.alloc(&d_tot, 32 * sizeof(uint64_t) + 16))) return rc;
     int *d_status = reinterpret_cast<int *>(d_tot + 32);
-    cudaEvent_t ev[3];
-    for (auto &e : ev)
-        if (cudaEventCreate(&e) != cudaSuccess) return NQ_ECUDA;
-    struct EvGuard {
-        cudaEvent_t *e;
-        ~EvGuard() {
-            for (int i = 0; i < 3; ++i) cudaEventDestroy(e[i]);
-        }
-    } evg{ev};
+    SplitEvents evs;
+    if ((rc = evs.init())) return rc;
+    cudaEvent_t *ev = evs.e;
     cudaEventRecord(ev[0], ctx.s);
     rc = m ? cuda_rc(cudaMemcpyAsync(d_kids, kids.data(), m * sizeof(nq_prefix),
                                      cudaMemcpyHostToDevice, ctx.s))

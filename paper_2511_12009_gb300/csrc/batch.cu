@@ -159,6 +159,7 @@ extern "C" int nq_batch_create(const int *ns, const int *ds, int k, const nq_con
         return NQ_ECUDA;
     }
     int rc = nqi::make_plan(b->max_n, b->min_d, false, false, cfg, &b->plan);
+    if (!rc) rc = nqi::plan_records(b->max_n, b->min_d, false, cfg, total, true, &b->plan);
     if (rc) {
         release(b);
         return rc;
@@ -173,6 +174,8 @@ extern "C" int nq_batch_create(const int *ns, const int *ds, int k, const nq_con
     bool ok = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     ok = ok && cudaMemsetAsync(b->d_cursor, 0, 16, s) == cudaSuccess;  // cursor and status
     ok = ok && cudaMemsetAsync(b->d_totals, 0, 32 * sizeof(uint64_t), s) == cudaSuccess;
+    if (b->plan.levels)  // split work adds into the counts
+        ok = ok && cudaMemsetAsync(b->d_counts, 0, total * sizeof(uint64_t), s) == cudaSuccess;
     ok = ok && nqi::launch_search(a, b->plan, false, false, s) == NQ_OK;
     ok = ok && cudaMemcpyAsync(b->h_totals, b->d_totals, 32 * sizeof(uint64_t),
                                cudaMemcpyDeviceToHost, s) == cudaSuccess;
@@ -235,8 +238,11 @@ extern "C" int nq_batch_run_separate(nq_batch *b, void *stream, uint64_t *totals
     // One plan per board (each with its own stack size and occupancy).
     std::vector<nqi::Plan> plans(b->k);
     for (int j = 0; j < b->k; ++j) {
-        const int rc = nqi::make_plan(b->sorted_n[j], b->sorted_d[j], false, false,
-                                      b->has_cfg ? &b->cfg : nullptr, &plans[j]);
+        const nq_config *cfg = b->has_cfg ? &b->cfg : nullptr;
+        int rc = nqi::make_plan(b->sorted_n[j], b->sorted_d[j], false, false, cfg, &plans[j]);
+        if (!rc)
+            rc = nqi::plan_records(b->sorted_n[j], b->sorted_d[j], false, cfg,
+                                   b->first[j + 1] - b->first[j], true, &plans[j]);
         if (rc) return rc;
     }
     cudaEvent_t e0, e1;
@@ -258,6 +264,11 @@ extern "C" int nq_batch_run_separate(nq_batch *b, void *stream, uint64_t *totals
         }
         const nqi::SearchArgs a = args_for(b, b->d_pre + b->first[j], n, b->sorted_n[j],
                                            b->sorted_d[j], plans[j].slots);
+        if (plans[j].levels &&
+            cudaMemsetAsync(a.counts, 0, n * sizeof(uint64_t), s) != cudaSuccess) {
+            rc = NQ_ECUDA;
+            break;
+        }
         rc = nqi::launch_search(a, plans[j], false, false, s);
     }
     if (!rc && (cudaMemcpyAsync(b->h_totals, b->d_totals, 32 * sizeof(uint64_t),

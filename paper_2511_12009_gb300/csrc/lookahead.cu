@@ -17,12 +17,22 @@
 // compare for the last column in place of the population count (22.4 ms),
 // dropping the candidates that a forced next row rules out (25.7 ms: five more
 // instructions for 16 % fewer steps).
+//
+// Records that are few or heavy are split into units (look_kernel_split) by the
+// digits of the unit's index, so that splitting needs no memory and no launch of
+// its own; the lanes of a warp that has nothing left to take share its last
+// subtrees. Before, one lane searched each record: 2048 records of N = 22, d = 7
+// took 509 ms of which 3.5 ms were work, now 4.3 ms; N = 14 from d = 3 1.97 ms,
+// now 0.07 ms; N = 18 from d = 5 53.6 ms, now 18.5 ms.
 #include "nq_internal.h"
 
 namespace nqi {
 namespace {
 
 constexpr int kLookSteps = 31;  // steps between bookkeeping points
+// Idle lanes for which a warp of a split launch takes a new range (before that
+// they take frames of the warp's own busy lanes).
+constexpr int kRefill = 8;
 
 // The sentinel frame, in slot 0 of every stack: whatever candidate bit p is
 // taken, cols + p, L + 2p and R + p/2 together cover all 32 bits (each of the
@@ -94,13 +104,67 @@ __device__ __forceinline__ void look_step(uint32_t &c, uint32_t &L, uint32_t &R,
         : "memory");
 }
 
-// The persistent search: every warp takes ranges of `kRange x claim` record
-// indices (the first one by its number, the others from the work cursor) and
-// hands them to its lanes as they become idle. One atomic serves a whole
-// range, and a launch whose records fit the first ranges needs no cursor.
-// Consecutive ranges go to different blocks first, so that few records spread
-// over the SMs.
-template <bool STREAM>
+// One unit of split work: the part of a record's subtree that the digits of s
+// name. Level j (row d + j) has a digit of several bits, the most significant
+// level first. Every level but the last: the t-th free column, or nothing
+// when there are fewer (the digit covers every column the row could have
+// free). The last level: the free columns t, t + R, t + 2R, ... of R = 2^bits,
+// so nothing is left out there with a small digit. The units of a record
+// partition its solutions.
+//   returns  0: nothing here, 1: search from (c, l, r) with candidates av
+//            (l, r as they reach this row), 2: *found solutions and no search
+//   skip     units to the next one that may hold something
+__device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint32_t digits,
+                                          int shift, uint32_t &c, uint32_t &l, uint32_t &r,
+                                          uint32_t &av, uint32_t &found, uint32_t &skip) {
+    skip = 1u;
+    for (int j = 0; j < levels; ++j, digits >>= 4) {
+        const uint32_t bits = digits & 15u;
+        const uint32_t here = s & ((1u << shift) - 1u);  // this level's digit and those below
+        shift -= (int)bits;
+        if (c == ~0u) {  // every row is placed: the solution belongs to the unit of zeros
+            skip = (1u << (shift + (int)bits)) - here;
+            found = here == 0u ? 1u : 0u;
+            return 2;
+        }
+        uint32_t x = ~(c | l | r);
+        for (uint32_t t = here >> shift; t && x; --t) x &= x - 1u;
+        if (x == 0u) {  // and nothing at any higher value of this digit
+            skip = (1u << (shift + (int)bits)) - here;
+            return 0;
+        }
+        const uint32_t p = x & (0u - x);
+        if (j + 1 < levels) {
+            c |= p;
+            l = (l | p) << 1;
+            r = (r | p) >> 1;
+        } else {
+            av = p;
+            for (x ^= p; x;) {
+                for (uint32_t t = (1u << bits) - 1u; t && x; --t) x &= x - 1u;
+                const uint32_t q = x & (0u - x);
+                av |= q;
+                x ^= q;
+            }
+        }
+    }
+    if (__popc(c) == 31) {  // the last row: each candidate is a solution
+        found = (uint32_t)__popc(av);
+        return 2;
+    }
+    return 1;
+}
+
+// The persistent search: every warp takes ranges of record indices (the first
+// one by its number, the others from the work cursor) and hands them to its
+// lanes as they become idle. One atomic serves a whole range, and a launch
+// whose records fit the first ranges needs no cursor. Consecutive ranges go to
+// different blocks first, so that few records spread over the SMs.
+// SPLIT: the indices are units (split_unit), 2^split_shift to a record, and a
+// unit's count is added into its record's entry (zeroed before the launch).
+// Units that cannot hold anything are passed over in one go: the warp's
+// position moves on by the last asking lane's skip.
+template <bool STREAM, bool SPLIT>
 __device__ __forceinline__ void look_body(const SearchArgs &a) {
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(look_smem);
     const uint32_t stride = stack_slot_offset(blockDim.x, 0u, 1u, 16u);
@@ -108,10 +172,12 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt_mask = (1u << lane) - 1u;
     const uint32_t m1 = a.mul[0], m2 = a.mul[1], mneg = a.mul[2];
-    const uint32_t range = kLookRange * (a.claim > 0 ? (uint32_t)a.claim : 1u);
+    const uint32_t range = a.range;
+    const uint64_t total = SPLIT ? a.n << a.split_shift : a.n;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
 
     uint32_t c = kSentC, L = kSentL, R = kSentR, av = kSentAv, top = base;
+    uint32_t bot = base;        // SPLIT: the lane's sentinel slot (frames below were given away)
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
                  :
                  : "r"(base), "r"(c), "r"(L), "r"(R), "r"(av)
@@ -125,17 +191,14 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     uint32_t wsum_n = 0;
     // the warp's range (the same in every lane)
     uint64_t next = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * range;
-    uint32_t rem = next < a.n ? (uint32_t)(a.n - next < range ? a.n - next : range) : 0u;
+    uint32_t rem = next < total ? (uint32_t)(total - next < range ? total - next : range) : 0u;
     bool exhausted = a.cursor == nullptr;
     uint32_t waits = 0;
 
     auto finish = [&](uint64_t i, uint64_t s, uint32_t w_n) {
-        if (a.by_tag) {  // split subproblems: the count goes to the parent named by the tag
-            const uint64_t parent = __ldg(reinterpret_cast<const uint32_t *>(a.pre + i) + 3) >> 12;
-            if (parent >= a.n_tags)
-                look_error(a.status, NQ_EINVAL);
-            else if (a.counts && s)
-                atomicAdd(reinterpret_cast<unsigned long long *>(&a.counts[parent]),
+        if (SPLIT) {
+            if (a.counts && s)
+                atomicAdd(reinterpret_cast<unsigned long long *>(&a.counts[i]),
                           (unsigned long long)s);
         } else if (a.counts) {
             a.counts[i] = s;
@@ -153,10 +216,11 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     };
 
     for (;;) {
-        const bool idle = top == base;  // on the sentinel
+        const bool idle = top == (SPLIT ? bot : base);  // on the sentinel
         if (idle) {
             if (busy) finish(idx, sol, wn);
             busy = false;
+            if (SPLIT) bot = top = base;
             c = kSentC;
             L = kSentL;
             R = kSentR;
@@ -166,15 +230,15 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
         unsigned need_mask = __ballot_sync(~0u, need);
         while (need_mask) {
             if (rem == 0u) {
-                if (exhausted) break;
+                if (exhausted || (SPLIT && __popc(need_mask) < kRefill)) break;
                 unsigned long long f = 0;
                 if (lane == 0) f = atomicAdd(a.cursor, (unsigned long long)range);
                 next = __shfl_sync(~0u, f, 0) + warps * range;
-                if (next >= a.n) {
+                if (next >= total) {
                     exhausted = true;
                     break;
                 }
-                rem = a.n - next < range ? (uint32_t)(a.n - next) : range;
+                rem = total - next < range ? (uint32_t)(total - next) : range;
             }
             uint32_t ready = rem;
             if (STREAM) {  // streamed input: only what has been published may be read
@@ -187,8 +251,15 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                 if (ready == 0u) break;
             }
             const uint32_t rank = __popc(need_mask & lt_mask);
+            uint32_t skip = 1u;
             if (need && rank < ready) {
-                const uint64_t pi = a.order ? a.n - 1 - (next + rank) : next + rank;
+                uint64_t at = next + rank;
+                uint32_t s = 0u;  // the unit's digits
+                if (SPLIT) {
+                    s = (uint32_t)at & ((1u << a.split_shift) - 1u);
+                    at >>= a.split_shift;
+                }
+                const uint64_t pi = a.order ? a.n - 1 - at : at;
                 uint4 P;
                 if (STREAM)  // (a line may have been cached before its copy arrived)
                     asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
@@ -202,13 +273,29 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                 const bool ok = n >= 1u && (a.expect_n == 0 || (int)n == a.expect_n) &&
                                 (w == 1u || w == 2u) && d <= n && (P.x & ~last) == 0u &&
                                 (uint32_t)__popc(P.x) == d;
-                // the stack: the sentinel and the ancestors of rows d..N-2
-                if (!ok) {
-                    look_error(a.status, NQ_EINVAL);
+                // (the stack holds the sentinel and the ancestors down to row N-2
+                // of a record with a.rows rows left)
+                if (!ok || (d + 1u < n && (int)(n - d) > a.rows)) {
+                    look_error(a.status, ok ? NQ_ESTACK : NQ_EINVAL);
                     finish(pi, 0, 0);
-                } else if (d + 1u < n && (int)(n - d) > a.slots) {
-                    look_error(a.status, NQ_ESTACK);
-                    finish(pi, 0, 0);
+                    if (SPLIT) skip = (1u << a.split_shift) - s;
+                } else if (SPLIT) {
+                    uint32_t cc = P.x | ~last, ll = P.y, rr = P.z & last, a0 = 0, found = 0;
+                    const int got = split_unit(s, a.levels, a.digits, a.split_shift, cc, ll, rr,
+                                               a0, found, skip);
+                    if (got == 2) finish(pi, found, w | (n << 2));
+                    if (got == 1) {
+                        idx = pi;
+                        wn = w | (n << 2);
+                        sol = 0;
+                        busy = true;
+                        c = cc;
+                        L = ll << 1;
+                        R = rr >> 1;
+                        av = a0;
+                        top = base + stride;
+                        need = false;
+                    }
                 } else {
                     const uint32_t c0 = P.x | ~last;
                     const uint32_t l0 = P.y, r0 = P.z & last;
@@ -232,7 +319,11 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                 }
             }
             const uint32_t asked = __popc(need_mask);
-            const uint32_t taken = asked < ready ? asked : ready;
+            uint32_t taken = asked < ready ? asked : ready;
+            if (SPLIT && asked <= ready) {  // every asker had a unit: pass over empty ones
+                taken += __shfl_sync(~0u, skip, 31 - __clz((int)need_mask)) - 1u;
+                taken = taken < rem ? taken : rem;
+            }
             next += taken;
             rem -= taken;
             need_mask = __ballot_sync(~0u, need);
@@ -246,6 +337,42 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
             }
             __nanosleep(256);
             continue;
+        }
+
+        if (SPLIT && need_mask && rem == 0u) {
+            // Each idle lane takes the shallowest saved frame of a busy lane of
+            // its warp, and leaves a sentinel in its place.
+            const bool giver = !need && top > bot + stride;
+            const unsigned givers = __ballot_sync(~0u, giver);
+            if (givers) {
+                const uint32_t pairs = min(__popc(need_mask), __popc(givers));
+                const uint32_t rank = __popc((need ? need_mask : givers) & lt_mask);
+                const bool taker = need && rank < pairs;
+                const int from = taker ? (int)__fns(givers, 0, (int)rank + 1) : (int)lane;
+                const uint32_t slot = __shfl_sync(~0u, bot + stride, from);
+                const uint64_t i = __shfl_sync(~0u, idx, from);
+                const uint32_t w_n = __shfl_sync(~0u, wn, from);
+                if (taker) {
+                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(c), "=r"(L), "=r"(R), "=r"(av)
+                                 : "r"(slot)
+                                 : "memory");
+                    idx = i;
+                    wn = w_n;
+                    sol = 0;
+                    busy = true;
+                    top = base + stride;
+                }
+                __syncwarp();
+                if (giver && rank < pairs) {
+                    bot += stride;
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
+                                 :
+                                 : "r"(bot), "r"(kSentC), "r"(kSentL), "r"(kSentR), "r"(kSentAv)
+                                 : "memory");
+                }
+                __syncwarp();
+            }
         }
 
         uint32_t s32 = 0;
@@ -272,14 +399,20 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     }
 }
 
-__global__ void __maxnreg__(48) look_kernel(const SearchArgs a) { look_body<false>(a); }
-__global__ void __maxnreg__(48) look_kernel_stream(const SearchArgs a) { look_body<true>(a); }
+__global__ void __maxnreg__(48) look_kernel(const SearchArgs a) { look_body<false, false>(a); }
+__global__ void __maxnreg__(48) look_kernel_stream(const SearchArgs a) {
+    look_body<true, false>(a);
+}
+__global__ void __maxnreg__(48) look_kernel_split(const SearchArgs a) {
+    look_body<false, true>(a);
+}
 
 }  // namespace
 
-void *look_kernel_ptr(bool stream) {
+void *look_kernel_ptr(bool stream, bool split) {
     return stream ? reinterpret_cast<void *>(&look_kernel_stream)
-                  : reinterpret_cast<void *>(&look_kernel);
+           : split ? reinterpret_cast<void *>(&look_kernel_split)
+                   : reinterpret_cast<void *>(&look_kernel);
 }
 
 }  // namespace nqi

@@ -94,7 +94,10 @@ extern "C" int nq_count_host_noalloc(int N, int d, const nq_prefix *h_prefixes, 
         return fail(NQ_ECUDA);
     nqi::Plan plan;
     rc = nqi::make_plan(N, d, false, false, nullptr, &plan);
+    if (!rc) rc = nqi::plan_records(N, d, false, nullptr, n, true, &plan);
     if (rc) return fail(rc);
+    if (plan.levels && cudaMemsetAsync(counts, 0, n * sizeof(uint64_t), s) != cudaSuccess)
+        return fail(NQ_ECUDA);
     nqi::SearchArgs a{};
     a.pre = pre;
     a.n = n;

@@ -68,6 +68,14 @@ struct SearchArgs {
     // Where the launch records the first error it finds (a device int the
     // caller zeroed; NULL: errors are not recorded).
     int *status;
+    // Layout REGP's production kernel only (lookahead.cu):
+    int rows;           // rows that a record may have left (max_n - min_d)
+    uint32_t range;     // indices a warp takes at once
+    // work split below the records (levels 0: not split): 2^split_shift units
+    // to a record, level j's digit in the j-th nibble of `digits`, in bits
+    int levels;
+    int split_shift;
+    uint32_t digits;
 };
 // Bookkeeping rounds a lane may wait for an unpublished index (each round is
 // one chunk of idle steps, plus a short sleep once the whole warp waits):
@@ -183,10 +191,9 @@ struct ServeArgs {
     int *status;                     // the server's error word (device)
 };
 
-// The production kernel of layout REGP (lookahead.cu), plain or for streamed input.
-void *look_kernel_ptr(bool stream);
-// Records a warp of it takes at once (times SearchArgs::claim).
-constexpr uint32_t kLookRange = 32;
+// The production kernel of layout REGP (lookahead.cu), plain, for streamed
+// input, or with the records' subtrees split.
+void *look_kernel_ptr(bool stream, bool split);
 
 int launch_serve(const ServeArgs &a, int grid, int block, size_t smem, cudaStream_t s);
 int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *smem,
@@ -202,6 +209,11 @@ struct Plan {
     int sms;        // multiprocessors of the device
     bool donate;    // the kernel variant with subtree donation
     bool stream;    // the kernel variant for streamed input (SearchArgs::published)
+    // layout REGP's production kernel (SearchArgs has the same names)
+    bool look;
+    int rows, levels, split_shift;
+    uint32_t digits, range;
+    bool cursor;    // the launch takes more than every warp's first range
 };
 
 // Stack slots a layout needs for prefixes of depth >= min_d on boards <= max_n
@@ -210,7 +222,14 @@ int slots_needed(int layout, int max_n, int min_d);
 
 // Resolve cfg (may be NULL) into a launch shape for the current device.
 int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config *cfg, Plan *plan,
-              bool donate = false, bool stream = false);
+              bool donate = false, bool stream = false, int levels = 0);
+
+// Complete a plan for n records (how a warp takes them), splitting their
+// subtrees where they are too few or too uneven for the grid (layout REGP's
+// production build, not streamed). A split launch adds into its counts, which
+// have to be zero before it.
+int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t n, bool may_split,
+                 Plan *plan);
 
 // Enqueue the search kernel. Returns NQ_OK or NQ_ECUDA.
 int launch_search(const SearchArgs &a, const Plan &p, bool diag, bool constrained, cudaStream_t s);
@@ -235,6 +254,7 @@ uint32_t meta_of(int weight, int n, int d);
 // out == nullptr: count only.
 constexpr uint64_t kMaxSplitParents = 1ull << 20;    // the 20-bit tag field
 constexpr uint64_t kMaxSplitChildren = 1ull << 27;   // 2 GiB of records
+int check_parents(const nq_prefix *in, uint64_t n);  // the records may be split
 int split_prefixes(const nq_prefix *in, uint64_t n, int rows, std::vector<nq_prefix> *out,
                    std::vector<uint64_t> *extra_nodes, uint64_t *n_children);
 

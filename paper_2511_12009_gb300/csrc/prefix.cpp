@@ -305,6 +305,11 @@ void expand_rec(int n, int target, int row, uint32_t cols, uint32_t ld, uint32_t
         return;
     }
     uint32_t av = last & ~(cols | ld | rd);
+    if (!out && row + 1 == target) {  // counting only: the last row's placements need no visit
+        cnt += (uint64_t)__builtin_popcount(av);
+        nodes += (uint64_t)__builtin_popcount(av);
+        return;
+    }
     while (av) {
         const uint32_t p = low_bit(av);
         av ^= p;
@@ -315,9 +320,8 @@ void expand_rec(int n, int target, int row, uint32_t cols, uint32_t ld, uint32_t
 }
 }  // namespace
 
-int split_prefixes(const nq_prefix *in, uint64_t n, int rows, std::vector<nq_prefix> *out,
-                   std::vector<uint64_t> *extra_nodes, uint64_t *n_children) {
-    if (n > kMaxSplitParents || rows < 0 || (n && !in)) return NQ_EINVAL;
+int check_parents(const nq_prefix *in, uint64_t n) {
+    if (n > kMaxSplitParents || (n && !in)) return NQ_EINVAL;
     for (uint64_t i = 0; i < n; ++i) {
         const int N = (int)NQ_META_N(in[i].meta), d = (int)NQ_META_D(in[i].meta);
         const int w = (int)NQ_META_WEIGHT(in[i].meta);
@@ -325,6 +329,13 @@ int split_prefixes(const nq_prefix *in, uint64_t n, int rows, std::vector<nq_pre
             __builtin_popcount(in[i].cols) != d)
             return NQ_EINVAL;
     }
+    return NQ_OK;
+}
+
+int split_prefixes(const nq_prefix *in, uint64_t n, int rows, std::vector<nq_prefix> *out,
+                   std::vector<uint64_t> *extra_nodes, uint64_t *n_children) {
+    if (rows < 0) return NQ_EINVAL;
+    if (const int rc = check_parents(in, n)) return rc;
     auto run = [&](uint64_t i, nq_prefix *dst, uint64_t &cnt, uint64_t &nodes) {
         const int N = (int)NQ_META_N(in[i].meta), d = (int)NQ_META_D(in[i].meta);
         const uint32_t hi = NQ_META_WEIGHT(in[i].meta) | ((uint32_t)N << 2) | ((uint32_t)i << 12);

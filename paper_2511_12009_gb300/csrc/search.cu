@@ -35,6 +35,8 @@
 // the next-row mask is additionally ANDed with allowed[row].
 #include <cuda.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <map>
 #include <mutex>
@@ -54,6 +56,7 @@ __device__ int g_stream_status[kStatusWords];
 
 namespace {
 
+constexpr int kSplitMaxLevels = 7;  // of split work (plan_records); a nibble each
 constexpr uint64_t kNone = ~0ull;
 constexpr int kChunk = 15;
 static_assert(kChunk < 16, "the sentinel frame holds 16 idle steps (32 for ~0 masks)");
@@ -1378,12 +1381,12 @@ void *plain_ptr(bool diag) {
 }
 
 void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
-                  bool stream = false) {
+                  bool stream = false, bool split = false) {
     if (stream) {
         switch (layout) {
             case NQ_LAYOUT_REGM: return stream_ptr<NQ_LAYOUT_REGM>(diag);
             case NQ_LAYOUT_REGP:
-                return diag ? stream_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(true);
+                return diag ? stream_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(true, false);
             case NQ_LAYOUT_REGZ: return stream_ptr<NQ_LAYOUT_REGZ>(diag);
             case NQ_LAYOUT_REGPZ: return stream_ptr<NQ_LAYOUT_REGPZ>(diag);
             default: return stream_ptr<NQ_LAYOUT_REG>(diag);
@@ -1406,7 +1409,7 @@ void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
         case NQ_LAYOUT_WTM: return plain_ptr<NQ_LAYOUT_WTM>(diag);
         case NQ_LAYOUT_REGM: return plain_ptr<NQ_LAYOUT_REGM>(diag);
         case NQ_LAYOUT_REGP:
-            return diag ? kernel_ptr<NQ_LAYOUT_REGP, true, false>() : look_kernel_ptr(false);
+            return diag ? kernel_ptr<NQ_LAYOUT_REGP, true, false>() : look_kernel_ptr(false, split);
         case NQ_LAYOUT_REGZ: return plain_ptr<NQ_LAYOUT_REGZ>(diag);
         case NQ_LAYOUT_REGPZ: return plain_ptr<NQ_LAYOUT_REGPZ>(diag);
         case NQ_LAYOUT_AVAIL: return plain_ptr<NQ_LAYOUT_AVAIL>(diag);
@@ -1429,7 +1432,7 @@ int slots_needed(int layout, int max_n, int min_d) {
 }
 
 int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config *cfg,
-              Plan *plan, bool donate, bool stream) {
+              Plan *plan, bool donate, bool stream, int levels) {
     if (max_n < 1 || max_n > NQ_MAX_N || min_d < 0 || min_d > max_n) return NQ_EINVAL;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return NQ_ECUDA;
@@ -1447,7 +1450,11 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
     // split-word kernels are compiled for one block size
     if (layout_split_words(p.layout) && p.block != (int)kZBlock) return NQ_EINVAL;
     if (p.layout == NQ_LAYOUT_AVAIL && max_n > 30) return NQ_EINVAL;  // guard columns
-    p.slots = slots_needed(p.layout, max_n, min_d);
+    p.look = p.layout == NQ_LAYOUT_REGP && !diag && !constrained;
+    p.levels = p.look ? levels : 0;
+    p.rows = max_n - min_d;
+    // (a split record's search starts `levels - 1` rows further down)
+    p.slots = slots_needed(p.layout, max_n, p.levels ? std::min(max_n, min_d + p.levels - 1) : min_d);
     const size_t per_thread = (size_t)p.slots * (p.layout == NQ_LAYOUT_AVAIL ? 4u : 16u);
     const size_t extra = constrained ? 32u * 4u : 0u;
     if ((size_t)p.block * per_thread + extra > (size_t)max_smem) {
@@ -1458,7 +1465,7 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
     p.donate = donate && (p.layout == NQ_LAYOUT_REG || p.layout == NQ_LAYOUT_REGM) && !constrained;
     p.stream = stream && !p.donate && !constrained && layout_register_top(p.layout);
     if (stream && !p.stream) return NQ_EINVAL;
-    void *k = pick_kernel(p.layout, diag, constrained, p.donate, p.stream);
+    void *k = pick_kernel(p.layout, diag, constrained, p.donate, p.stream, p.levels > 0);
     if (!(cfg && cfg->block) && !layout_split_words(p.layout)) {
         // No block size asked for: the one that keeps the most threads resident
         // per SM under this stack footprint (ties: the larger block). A frame
@@ -1502,12 +1509,107 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
     return NQ_OK;
 }
 
+namespace {
+
+// Search steps below one record of an N x N board with `rows` rows left, to a
+// factor of two: a quadratic fit of the logarithm to random-descent estimates
+// for N = 10..28 and 6 <= rows <= 20.
+double subtree_steps(int n, int rows) {
+    const double k = rows;
+    return std::exp(-1.0958 + 0.97935 * k - 0.25224 * n + 0.0752 * k * k - 0.04991 * n * k +
+                    0.013134 * n * n);
+}
+
+// Digit of a split level: enough bits for every column that the row could have
+// free, and 2 on the last level, whose digit strides over the free columns.
+int digit_bits(int free_columns, bool last) {
+    int b = 1;
+    while ((1 << b) < free_columns) ++b;
+    return last ? 2 : b;
+}
+
+}  // namespace
+
+int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t n, bool may_split,
+                 Plan *plan) {
+    if (!plan->look) return NQ_OK;
+    Plan p = *plan;
+    const uint32_t claim = cfg && cfg->claim > 0 ? (uint32_t)cfg->claim : 1u;
+    const double lanes = (double)p.grid * p.block;
+    int levels = 0, shift = 0;
+    uint32_t digits = 0;
+    if (may_split && !p.stream && n) {
+        // Split while there is less than a unit for every fourth lane and a unit
+        // is not small in itself (setting one up costs some ten steps), or while
+        // a unit is more than an eighth of a lane's share of the work (the
+        // largest are a few times the mean). A level more or less where the line
+        // lies costs little (N = 16, d = 5: 1 level 0.60 ms, 2 levels 0.56 ms,
+        // none 1.25 ms; N = 18, d = 5: 20.3, 18.4, 38.9 ms), a missing one much
+        // (2048 records of N = 22, d = 7: 1 level 44 ms, 3 levels 5.5 ms, 4
+        // levels 4.5 ms, 5 levels 6.5 ms, none 326 ms).
+        const double share = (double)n * subtree_steps(max_n, p.rows) / lanes;
+        double live = (double)n;                            // units that hold something
+        double unit = subtree_steps(max_n, p.rows);         // steps below one
+        while (levels < kSplitMaxLevels && levels < p.rows) {
+            const bool few = live < lanes / 4.0 && unit > 150.0;
+            const bool uneven = unit > std::max(750.0, share / 8.0);
+            if (!few && !uneven) break;
+            int sh = 0;
+            uint32_t dg = 0;
+            double lv = (double)n, un = 0.0;
+            for (int j = 0; j <= levels; ++j) {
+                const bool last = j == levels;
+                const int b = digit_bits(p.rows - j, last);
+                const double open = 0.6 * (p.rows - j);  // free columns of a row, about
+                dg |= (uint32_t)b << (4 * j);
+                sh += b;
+                lv *= last ? std::min(open, (double)(1 << b)) : open;
+                if (last)
+                    un = subtree_steps(max_n, p.rows - j) / std::max(1.0, std::min(open, (double)(1 << b)));
+            }
+            if (sh > 31 || n > (1ull << (62 - sh))) break;
+            ++levels;
+            shift = sh;
+            digits = dg;
+            live = lv;
+            unit = un;
+        }
+    }
+    if (levels) {
+        const int rc = make_plan(max_n, min_d, diag, false, cfg, &p, false, false, levels);
+        if (rc) return rc;
+    }
+    p.split_shift = shift;
+    p.digits = digits;
+    // A warp takes 32 indices x claim at once. Of split work: half of that
+    // where the first ranges cover everything (other warps get the rest and
+    // each one's lanes share), and more where the empty units among them are
+    // many, as long as every warp still takes about 64 ranges.
+    const uint64_t total = n << shift;
+    const uint64_t warps = (uint64_t)p.grid * (uint64_t)(p.block / 32);
+    p.range = 32u * std::min(claim, 1024u);
+    if (levels && total <= warps * 16u) p.range = 16u;
+    while (levels && p.range < 32768u && total / p.range > 128 * warps) p.range *= 2u;
+    p.cursor = total > warps * p.range;
+    if (!p.cursor)  // no more blocks than ranges: few records take one warp of each block
+        p.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(p.grid, (total + p.range - 1) / p.range));
+    *plan = p;
+    return NQ_OK;
+}
+
 int launch_search(const SearchArgs &a, const Plan &p, bool diag, bool constrained,
                   cudaStream_t s) {
     if (a.n == 0) return NQ_OK;
     if ((a.published != nullptr) != p.stream) return NQ_EINVAL;
-    void *k = pick_kernel(p.layout, diag, constrained, p.donate && a.dq != nullptr, p.stream);
+    void *k = pick_kernel(p.layout, diag, constrained, p.donate && a.dq != nullptr, p.stream,
+                          p.levels > 0);
     SearchArgs args = a;
+    args.rows = p.rows;
+    args.range = p.range;
+    args.levels = p.levels;
+    args.split_shift = p.split_shift;
+    args.digits = p.digits;
+    if (p.look && !p.cursor) args.cursor = nullptr;
     void *params[] = {&args};
     const cudaError_t e = cudaLaunchKernel(k, dim3(p.grid), dim3(p.block), params, p.smem, s);
     return e == cudaSuccess ? NQ_OK : NQ_ECUDA;

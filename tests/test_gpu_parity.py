@@ -449,3 +449,37 @@ def test_default_form_record_ranges(orc, n, d, m, claim, order, shape):
     m = m or len(pre)
     got, _, tot = run(pre[:m], d, n, "regp", claim=claim, order=order, **shape)
     assert np.array_equal(got, want[:m]) and int(tot[n]) == weighted(pre[:m], want[:m])
+
+
+@pytest.mark.parametrize("n,d", [(16, 0), (15, 2), (14, 3), (17, 3), (16, 4), (18, 4)])
+def test_split_records_equal_unsplit(n, d):
+    """Few heavy records: the default form splits their subtrees over the grid.
+    Counts and totals equal those of REG, which does not split."""
+    pre = nq.enumerate_prefixes(n, d)
+    want, _, wt = run(pre, d, n, "reg", donate=1)
+    for m in sorted({1, 3, len(pre) // 2, len(pre)}):
+        got, _, tot = run(pre[:m], d, n, "regp")
+        assert np.array_equal(got, want[:m]) and int(tot[n]) == weighted(pre[:m], want[:m])
+    assert int(wt[n]) == Q[n]
+
+
+def test_split_launch_with_boards_that_end_early():
+    """A split launch (N = 16 from d = 2) that also holds solved boards, last rows,
+    dead ends, shallow small boards and malformed records, at the record positions
+    that a warp's range starts and ends on."""
+    parts = [nq.enumerate_prefixes(n, d) for n, d in [(16, 2), (1, 0), (1, 1), (4, 4), (6, 5), (6, 6),
+                                                      (5, 0), (8, 1), (10, 7), (9, 8), (14, 0)]]
+    pre = np.concatenate(parts)
+    pre = pre[np.random.default_rng(3).permutation(len(pre))]
+    want, _, wt = run(pre, 2, 16, "reg")
+    got, _, tot = run(pre, 2, 16, "regp")
+    assert np.array_equal(got, want) and np.array_equal(tot, wt)
+    bad = pre.copy()
+    bad["meta"][7] &= ~np.uint32(3)
+    cnt = torch.full((len(bad),), -1, dtype=torch.int64, device="cuda")
+    nq.count_ex(nq.to_device(bad), 2, 16, cnt)
+    with pytest.raises(nq.NQError) as e:
+        nq.sync()
+    assert e.value.code == nq.NQ_EINVAL
+    want[7] = 0
+    assert np.array_equal(u64(cnt), want)

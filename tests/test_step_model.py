@@ -383,3 +383,74 @@ def test_look_ahead_sentinel_holds_32_idle_steps():
         assert s == 0 and top == 0 and state[3] != 0
     with pytest.raises(AssertionError, match="below"):
         step_look(state, stack, top)
+
+
+# --- work split below a record (layout REGP) ----------------------------------------
+
+def digit_bits(free_columns, last):
+    b = 1
+    while (1 << b) < free_columns:
+        b += 1
+    return 2 if last else b
+
+
+def split_unit(s, bits, c, l, r):
+    """(kind, state, candidates, found, skip) of unit s of a record, as the split
+    kernel decodes it: kind 0 nothing, 1 search, 2 solutions found."""
+    shift = sum(bits)
+    av = 0
+    for j, b in enumerate(bits):
+        here = s & ((1 << shift) - 1)
+        shift -= b
+        if c == M:
+            return 2, None, 0, int(here == 0), (1 << (shift + b)) - here
+        x = ~(c | l | r) & M
+        for _ in range(here >> shift):
+            x &= x - 1 if x else 0
+        if x == 0:
+            return 0, None, 0, 0, (1 << (shift + b)) - here
+        p = x & -x
+        if j + 1 < len(bits):
+            c, l, r = c | p, ((l | p) << 1) & M, (r | p) >> 1
+        else:
+            av, x = p, x ^ p
+            while x:
+                for _ in range((1 << b) - 1):
+                    x &= x - 1 if x else 0
+                av |= x & -x
+                x &= x - 1 if x else 0
+    if popc(c) == 31:
+        return 2, None, 0, popc(av), 1
+    return 1, (c, l, r), av, 0, 1
+
+
+def below(c, l, r, av):
+    """Solutions below a frame with candidates av."""
+    sol = 0
+    while av:
+        p = av & -av
+        av ^= p
+        c2, l2, r2 = c | p, ((l | p) << 1) & M, (r | p) >> 1
+        sol += 1 if c2 == M else below(c2, l2, r2, ~(c2 | l2 | r2) & M)
+    return sol
+
+
+@pytest.mark.parametrize("n,d,levels,rows", [(8, 0, 3, 8), (9, 2, 4, 9), (7, 3, 7, 9), (6, 6, 2, 6),
+                                             (6, 5, 3, 4), (10, 4, 1, 6), (9, 1, 2, 8), (5, 1, 6, 20)])
+def test_split_units_partition_the_subtree(orc, n, d, levels, rows):
+    """The units of a record, walked with the skips that the kernel takes, hold
+    every solution below it once -- also where the board ends above the last
+    level (rows may be larger than the board's own in a mixed launch)."""
+    bits = [digit_bits(max(rows - j, 1), j == levels - 1) for j in range(levels)]
+    pre = nq.enumerate_prefixes(n, d)
+    want, _ = orc.count_prefixes(n, orc.prefixes(n, d)[0])
+    for i in sorted(set([0, len(pre) // 2, len(pre) - 1])):
+        rec, last = pre[i], (1 << n) - 1
+        state = int(rec["cols"]) | (~last & M), int(rec["ld"]), int(rec["rd"])
+        s = total = 0
+        while s < 1 << sum(bits):
+            kind, st, av, found, skip = split_unit(s, bits, *state)
+            total += found if kind == 2 else below(*st, av) if kind == 1 else 0
+            assert skip >= 1
+            s += skip
+        assert total == int(want[i])
