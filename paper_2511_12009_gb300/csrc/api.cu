@@ -146,7 +146,7 @@ int enqueue_search(const nq_prefix *d_prefixes, uint64_t n, int expect_n, int mi
     // (nq_count_split).
     const bool donate = reg && !constrained && !n_tags && !published && cfg && cfg->donate == 2;
     if (donate && (rc = make_plan(max_n, min_d, diag, constrained, cfg, &p, true))) return rc;
-    if ((rc = plan_records(max_n, min_d, diag, cfg, n, !n_tags, &p))) return rc;
+    if ((rc = plan_records(max_n, min_d, diag, cfg, n, !n_tags, &p, allowed))) return rc;
     if (p.levels && d_counts &&
         cudaMemsetAsync(d_counts, 0, n * sizeof(uint64_t), s) != cudaSuccess)
         return NQ_ECUDA;
@@ -630,9 +630,7 @@ extern "C" int nq_count_split(const nq_prefix *h_prefixes, uint64_t n, int rows,
 
 // ---------------------------------------------------------------------------
 // Partial-board constraints: every listed queen's row may take only its
-// column, every other row loses the cells the listed queens attack. The
-// prefix rows are enumerated under the same masks (no symmetry: weight 1) and
-// the constrained kernel applies the masks below the prefix.
+// column, every other row loses the cells the listed queens attack.
 // ---------------------------------------------------------------------------
 extern "C" int nq_count_constrained(int N, const nq_queen *q, int k, uint64_t *count_out) {
     if (!count_out) return NQ_EINVAL;
@@ -644,43 +642,28 @@ extern "C" int nq_count_constrained(int N, const nq_queen *q, int k, uint64_t *c
         *count_out = 0;
         return NQ_OK;
     }
-    // Depth: the default, then deeper while the subproblems are fewer than four
-    // per resident lane (queens given in the first rows leave few, heavy
-    // subtrees), up to 2^26 records.
-    int d = std::min(nq_default_depth(N), N);
-    {
-        Plan p{};
-        int prc = make_plan(N, d, false, true, nullptr, &p);
-        if (prc) return prc;
-        const uint64_t lanes = (uint64_t)p.grid * (uint64_t)p.block;
-        uint64_t cnt = count_constrained_prefixes(N, d, allowed);
-        while (d + 1 <= N - 2 && cnt < 4 * lanes) {
-            const uint64_t next = count_constrained_prefixes(N, d + 1, allowed);
-            if (next > (1ull << 26)) break;
-            ++d;
-            cnt = next;
+    if (k == 0) return nq_total(N, count_out);  // nothing given: the board's symmetries hold
+    for (int r = 0; r < N; ++r)
+        if (!allowed[r]) {  // a row that the given queens leave no column
+            *count_out = 0;
+            return NQ_OK;
         }
-    }
-    std::vector<nq_prefix> pre;
-    constrained_prefixes(N, d, allowed, 0, pre);
-    if (pre.empty()) {
-        *count_out = 0;
-        return NQ_OK;
-    }
+    // The whole board as one record; the launch splits it (plan_records).
+    const nq_prefix root{0, 0, 0, NQ_META(1, N, 0, 0)};
     CallCtx ctx;
     int rc = ctx.init();
     if (rc) return rc;
     nq_prefix *d_pre = nullptr;
     uint64_t *d_tot = nullptr;
-    if ((rc = ctx.alloc(&d_pre, pre.size() * sizeof(nq_prefix)))) return rc;
+    if ((rc = ctx.alloc(&d_pre, sizeof(nq_prefix)))) return rc;
     if ((rc = ctx.alloc(&d_tot, 32 * sizeof(uint64_t) + 16))) return rc;
     int *d_status = reinterpret_cast<int *>(d_tot + 32);
-    rc = cuda_rc(cudaMemcpyAsync(d_pre, pre.data(), pre.size() * sizeof(nq_prefix),
-                                 cudaMemcpyHostToDevice, ctx.s));
+    rc = cuda_rc(
+        cudaMemcpyAsync(d_pre, &root, sizeof(root), cudaMemcpyHostToDevice, ctx.s));
     if (!rc) rc = cuda_rc(cudaMemsetAsync(d_tot, 0, 32 * sizeof(uint64_t) + 16, ctx.s));
     if (!rc)
-        rc = enqueue_search(d_pre, pre.size(), N, d, N, nullptr, nullptr, d_tot, nullptr,
-                            allowed, ctx.s, nullptr, d_status);
+        rc = enqueue_search(d_pre, 1, N, 0, N, nullptr, nullptr, d_tot, nullptr, allowed, ctx.s,
+                            nullptr, d_status);
     uint64_t tot = 0;
     if (!rc)
         rc = cuda_rc(cudaMemcpyAsync(&tot, d_tot + N, sizeof(uint64_t), cudaMemcpyDeviceToHost,

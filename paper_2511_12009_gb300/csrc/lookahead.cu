@@ -41,6 +41,8 @@ constexpr int kRefill = 8;
 // 32 idle steps: one frame lasts a whole round.
 constexpr uint32_t kSentC = 0x55555555u, kSentL = 0xAAAAAAAAu, kSentR = 0x55555555u;
 constexpr uint32_t kSentAv = 0xFFFFFFFFu;
+// Under masks: the frame above row 31, whose masks are 0, with no diagonals.
+constexpr uint32_t kSentMaskedC = 31u << kRowShift;
 static_assert(kLookSteps < 32, "an idle lane must not use up the sentinel's candidates");
 
 extern __shared__ __align__(16) unsigned char look_smem[];
@@ -104,6 +106,63 @@ __device__ __forceinline__ void look_step(uint32_t &c, uint32_t &L, uint32_t &R,
         : "memory");
 }
 
+// The same step under per-row masks (partial-board queries): the row rides in
+// bits 27..31 of c, already counted up for the child (c = columns | (row + 1)
+// << 27), so entering a child adds the next row where look_step moves a
+// register. The masks of the child's row and of the row after it come as one
+// 8-byte load whose address depends on the frame alone; rows at or below the
+// last have mask 0 after them, so a last-row child is counted and not entered.
+// The last row is a compare of the row field, no population count.
+// Six queries of two queens at N = 16: 98 ms with the host enumerating the
+// subproblems on one core, 1.8 ms as one split record (of which 1.2 ms are the
+// six calls' own cost).
+__device__ __forceinline__ void look_step_masked(uint32_t &c, uint32_t &L, uint32_t &R,
+                                                 uint32_t &av, uint32_t &top,
+                                                 const uint32_t stride, const uint32_t table,
+                                                 const uint32_t thr, uint32_t &s32,
+                                                 const uint32_t m1, const uint32_t m2,
+                                                 const uint32_t mneg) {
+    uint32_t A1, A2;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
+                 : "=r"(A1), "=r"(A2)
+                 : "r"(((c >> kRowShift) << 3) + table)
+                 : "memory");
+    const uint32_t p = av & (av * mneg);
+    const uint32_t ar = p * mneg + av;
+    const uint32_t c2 = p * m1 + c;
+    const uint32_t l2 = L + 2u * p;
+    const uint32_t r2 = (p >> 1) + R;
+    const uint32_t L2 = l2 * m2;
+    const uint32_t R2 = r2 >> 1;
+    const uint32_t t1 = c2 | l2 | r2, t2 = c2 | L2 | R2;
+    // operands as in look_step, but %6 t1, %7 thr, %10 t2, %14 A1, %15 A2;
+    // lop3 table 0x30: the first input without the second
+    asm volatile(
+        "{\n\t"
+        ".reg .pred ptrue, plive, ppush, pcnt, psave, ppop;\n\t"
+        ".reg .b32 a2, b2;\n\t"
+        "setp.eq.u32 ptrue, 0, 0;\n\t"
+        "lop3.and.b32 a2|plive, %14, %6, 0, 0x30, ptrue;\n\t"    // the child's row has a column
+        "lop3.and.b32 b2|ppush, %15, %10, 0, 0x30, plive;\n\t"   // ... and so has the row after
+        "setp.ge.and.u32 pcnt, %9, %7, plive;\n\t"               // the last row has one: a solution
+        "@pcnt add.u32 %5, %5, 1;\n\t"
+        "setp.ne.and.u32 psave, %8, 0, ppush;\n\t"
+        "setp.eq.and.u32 ppop, %8, 0, !ppush;\n\t"
+        "@psave st.shared.v4.u32 [%4], {%0, %1, %2, %8};\n\t"
+        "@psave add.u32 %4, %4, %11;\n\t"
+        "@ppop sub.u32 %4, %4, %11;\n\t"
+        "selp.b32 %3, a2, %8, ppush;\n\t"
+        "@ppush add.u32 %0, %9, %16;\n\t"
+        "@ppush mov.b32 %1, %12;\n\t"
+        "@ppush mov.b32 %2, %13;\n\t"
+        "@ppop ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n\t"
+        "}"
+        : "+r"(c), "+r"(L), "+r"(R), "+r"(av), "+r"(top), "+r"(s32)
+        : "r"(t1), "r"(thr), "r"(ar), "r"(c2), "r"(t2), "r"(stride), "r"(L2), "r"(R2), "r"(A1),
+          "r"(A2), "n"(1u << kRowShift)
+        : "memory");
+}
+
 // One unit of split work: the part of a record's subtree that the digits of s
 // name. Level j (row d + j) has a digit of several bits, the most significant
 // level first. Every level but the last: the t-th free column, or nothing
@@ -114,20 +173,29 @@ __device__ __forceinline__ void look_step(uint32_t &c, uint32_t &L, uint32_t &R,
 //   returns  0: nothing here, 1: search from (c, l, r) with candidates av
 //            (l, r as they reach this row), 2: *found solutions and no search
 //   skip     units to the next one that may hold something
+// MASKED: row `row` takes only the columns of its mask (table: 8 bytes a row),
+// and the board ends after `rows` rows; c holds no pre-set columns.
+template <bool MASKED>
 __device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint32_t digits,
                                           int shift, uint32_t &c, uint32_t &l, uint32_t &r,
-                                          uint32_t &av, uint32_t &found, uint32_t &skip) {
+                                          uint32_t &av, uint32_t &found, uint32_t &skip,
+                                          const uint32_t table, uint32_t row, uint32_t rows) {
     skip = 1u;
-    for (int j = 0; j < levels; ++j, digits >>= 4) {
+    for (int j = 0; j < levels; ++j, digits >>= 4, ++row) {
         const uint32_t bits = digits & 15u;
         const uint32_t here = s & ((1u << shift) - 1u);  // this level's digit and those below
         shift -= (int)bits;
-        if (c == ~0u) {  // every row is placed: the solution belongs to the unit of zeros
+        if (MASKED ? row == rows : c == ~0u) {  // every row is placed: the solution belongs to the unit of zeros
             skip = (1u << (shift + (int)bits)) - here;
             found = here == 0u ? 1u : 0u;
             return 2;
         }
         uint32_t x = ~(c | l | r);
+        if (MASKED) {
+            uint32_t mask;
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mask) : "r"(table + 8u * row) : "memory");
+            x &= mask;
+        }
         for (uint32_t t = here >> shift; t && x; --t) x &= x - 1u;
         if (x == 0u) {  // and nothing at any higher value of this digit
             skip = (1u << (shift + (int)bits)) - here;
@@ -148,7 +216,8 @@ __device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint32_t
             }
         }
     }
-    if (__popc(c) == 31) {  // the last row: each candidate is a solution
+    // the last row (the last level's row is row - 1 now): each candidate is a solution
+    if (MASKED ? row == rows : __popc(c) == 31) {
         found = (uint32_t)__popc(av);
         return 2;
     }
@@ -164,8 +233,12 @@ __device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint32_t
 // unit's count is added into its record's entry (zeroed before the launch).
 // Units that cannot hold anything are passed over in one go: the warp's
 // position moves on by the last asking lane's skip.
-template <bool STREAM, bool SPLIT>
+// MASKED (split only): one table of row masks for the launch, above the stacks.
+template <bool STREAM, bool SPLIT, bool MASKED>
 __device__ __forceinline__ void look_body(const SearchArgs &a) {
+    static_assert(SPLIT || !MASKED, "masked searches are split");
+    constexpr uint32_t kSC = MASKED ? kSentMaskedC : kSentC, kSL = MASKED ? 0u : kSentL,
+                       kSR = MASKED ? 0u : kSentR;
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(look_smem);
     const uint32_t stride = stack_slot_offset(blockDim.x, 0u, 1u, 16u);
     const uint32_t base = sbase + stack_slot_offset(blockDim.x, threadIdx.x, 0u, 16u);
@@ -176,7 +249,19 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     const uint64_t total = SPLIT ? a.n << a.split_shift : a.n;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
 
-    uint32_t c = kSentC, L = kSentL, R = kSentR, av = kSentAv, top = base;
+    const uint32_t table = sbase + (uint32_t)a.slots * stride;
+    const uint32_t thr = MASKED ? (uint32_t)(a.expect_n - 1) << kRowShift : 0u;
+    if (MASKED) {
+        if (threadIdx.x < 32u)
+            asm volatile("st.shared.v2.u32 [%0], {%1, %2};"
+                         :
+                         : "r"(table + 8u * threadIdx.x), "r"(a.allowed[threadIdx.x]),
+                           "r"(threadIdx.x < 31u ? a.allowed[threadIdx.x + 1u] : 0u)
+                         : "memory");
+        __syncthreads();
+    }
+
+    uint32_t c = kSC, L = kSL, R = kSR, av = kSentAv, top = base;
     uint32_t bot = base;        // SPLIT: the lane's sentinel slot (frames below were given away)
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
                  :
@@ -221,9 +306,9 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
             if (busy) finish(idx, sol, wn);
             busy = false;
             if (SPLIT) bot = top = base;
-            c = kSentC;
-            L = kSentL;
-            R = kSentR;
+            c = kSC;
+            L = kSL;
+            R = kSR;
             av = kSentAv;
         }
         bool need = idle;
@@ -280,16 +365,17 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                     finish(pi, 0, 0);
                     if (SPLIT) skip = (1u << a.split_shift) - s;
                 } else if (SPLIT) {
-                    uint32_t cc = P.x | ~last, ll = P.y, rr = P.z & last, a0 = 0, found = 0;
-                    const int got = split_unit(s, a.levels, a.digits, a.split_shift, cc, ll, rr,
-                                               a0, found, skip);
+                    uint32_t cc = MASKED ? P.x : P.x | ~last;
+                    uint32_t ll = P.y, rr = P.z & last, a0 = 0, found = 0;
+                    const int got = split_unit<MASKED>(s, a.levels, a.digits, a.split_shift, cc,
+                                                       ll, rr, a0, found, skip, table, d, n);
                     if (got == 2) finish(pi, found, w | (n << 2));
                     if (got == 1) {
                         idx = pi;
                         wn = w | (n << 2);
                         sol = 0;
                         busy = true;
-                        c = cc;
+                        c = MASKED ? cc | ((d + (uint32_t)a.levels) << kRowShift) : cc;
                         L = ll << 1;
                         R = rr >> 1;
                         av = a0;
@@ -368,7 +454,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                     bot += stride;
                     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
                                  :
-                                 : "r"(bot), "r"(kSentC), "r"(kSentL), "r"(kSentR), "r"(kSentAv)
+                                 : "r"(bot), "r"(kSC), "r"(kSL), "r"(kSR), "r"(kSentAv)
                                  : "memory");
                 }
                 __syncwarp();
@@ -377,7 +463,12 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
 
         uint32_t s32 = 0;
 #pragma unroll
-        for (int j = 0; j < kLookSteps; ++j) look_step(c, L, R, av, top, stride, s32, m1, m2, mneg);
+        for (int j = 0; j < kLookSteps; ++j) {
+            if constexpr (MASKED)
+                look_step_masked(c, L, R, av, top, stride, table, thr, s32, m1, m2, mneg);
+            else
+                look_step(c, L, R, av, top, stride, s32, m1, m2, mneg);
+        }
         sol += s32;
     }
 
@@ -399,20 +490,26 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     }
 }
 
-__global__ void __maxnreg__(48) look_kernel(const SearchArgs a) { look_body<false, false>(a); }
+__global__ void __maxnreg__(48) look_kernel(const SearchArgs a) {
+    look_body<false, false, false>(a);
+}
 __global__ void __maxnreg__(48) look_kernel_stream(const SearchArgs a) {
-    look_body<true, false>(a);
+    look_body<true, false, false>(a);
 }
 __global__ void __maxnreg__(48) look_kernel_split(const SearchArgs a) {
-    look_body<false, true>(a);
+    look_body<false, true, false>(a);
+}
+__global__ void __maxnreg__(48) look_kernel_masked(const SearchArgs a) {
+    look_body<false, true, true>(a);
 }
 
 }  // namespace
 
-void *look_kernel_ptr(bool stream, bool split) {
-    return stream ? reinterpret_cast<void *>(&look_kernel_stream)
-           : split ? reinterpret_cast<void *>(&look_kernel_split)
-                   : reinterpret_cast<void *>(&look_kernel);
+void *look_kernel_ptr(bool stream, bool split, bool masked) {
+    return stream   ? reinterpret_cast<void *>(&look_kernel_stream)
+           : masked ? reinterpret_cast<void *>(&look_kernel_masked)
+           : split  ? reinterpret_cast<void *>(&look_kernel_split)
+                    : reinterpret_cast<void *>(&look_kernel);
 }
 
 }  // namespace nqi

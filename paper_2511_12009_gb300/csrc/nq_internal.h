@@ -191,9 +191,9 @@ struct ServeArgs {
     int *status;                     // the server's error word (device)
 };
 
-// The production kernel of layout REGP (lookahead.cu), plain, for streamed
-// input, or with the records' subtrees split.
-void *look_kernel_ptr(bool stream, bool split);
+// The production kernel of layout REGP (lookahead.cu): plain, for streamed
+// input, with the records' subtrees split, or split and under row masks.
+void *look_kernel_ptr(bool stream, bool split, bool masked);
 
 int launch_serve(const ServeArgs &a, int grid, int block, size_t smem, cudaStream_t s);
 int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *smem,
@@ -227,9 +227,10 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
 // Complete a plan for n records (how a warp takes them), splitting their
 // subtrees where they are too few or too uneven for the grid (layout REGP's
 // production build, not streamed). A split launch adds into its counts, which
-// have to be zero before it.
+// have to be zero before it. allowed: the row masks of a constrained plan,
+// which is always split.
 int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t n, bool may_split,
-                 Plan *plan);
+                 Plan *plan, const uint32_t *allowed = nullptr);
 
 // Enqueue the search kernel. Returns NQ_OK or NQ_ECUDA.
 int launch_search(const SearchArgs &a, const Plan &p, bool diag, bool constrained, cudaStream_t s);

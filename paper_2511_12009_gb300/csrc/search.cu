@@ -23,13 +23,16 @@
 //   - the loop body is branch-free: a sentinel frame at the bottom of every
 //     stack keeps a finished lane harmlessly "searching" a board with no free
 //     column until the next bookkeeping point, which comes every kChunk = 15
-//     steps (31 for the default layout REGM, whose stacks hold two sentinel
+//     steps (31 for REGM, REGZ and REGPZ, whose stacks hold two sentinel
 //     frames: the sentinels' candidate bits must not run out within a round);
 //   - uint64 solution counts per subproblem; weighted totals reduced per warp
 //     with shuffles, one atomicAdd per warp and board size.
 //
-// Constrained mode (partial-board queries, the serving extension; not in the
-// paper): every row r has a mask allowed[r] of the columns it may take (one
+// The default layout REGP's production kernel, and the search under row masks
+// that nq_count_constrained makes, are in lookahead.cu; this file's REGP is its
+// diagnostic build.
+//
+// Served mode (partial-board queries; not in the paper): every row r has a mask allowed[r] of the columns it may take (one
 // column for a row with a given queen; the cells the given queens attack
 // removed elsewhere), the frame's row index rides in bits 27..31 of cols, and
 // the next-row mask is additionally ANDed with allowed[row].
@@ -56,7 +59,7 @@ __device__ int g_stream_status[kStatusWords];
 
 namespace {
 
-constexpr int kSplitMaxLevels = 7;  // of split work (plan_records); a nibble each
+constexpr int kSplitMaxLevels = 8;  // of split work (plan_records); a nibble each
 constexpr uint64_t kNone = ~0ull;
 constexpr int kChunk = 15;
 static_assert(kChunk < 16, "the sentinel frame holds 16 idle steps (32 for ~0 masks)");
@@ -182,7 +185,7 @@ struct Lane {
 // pushed like any other and a solution is the step that fills every column
 // (cols == ~0 with the columns >= N pre-set). SPLIT: split-word frames.
 // (The diagnostic builds of REGM, REGP, REGZ and REGPZ run this form.)
-template <bool DIAG, bool CONSTR, bool MADD = false, bool PUSHLAST = false, bool SPLIT = false>
+template <bool DIAG, bool MADD = false, bool PUSHLAST = false, bool SPLIT = false>
 __device__ __forceinline__ void step_reg(uint32_t &c, uint32_t &l, uint32_t &r, uint32_t &av,
                                          uint32_t &top, const Lane &k, uint32_t &s32,
                                          uint32_t &n32, const uint32_t m1 = 1u,
@@ -200,17 +203,9 @@ __device__ __forceinline__ void step_reg(uint32_t &c, uint32_t &l, uint32_t &r, 
         l2 = (l | p) << 1;
         r2 = (r | p) >> 1;
     }
-    uint32_t c2, a2;
-    bool lastrow;
-    if (CONSTR) {
-        c2 = (MADD ? p * m1 + c : (c | p)) + kRowInc;
-        a2 = ~(c2 | l2 | r2) & lds1(k.table + ((c2 >> kRowShift) << 2));
-        lastrow = c2 >= k.thr;
-    } else {
-        c2 = MADD ? p * m1 + c : c | p;
-        a2 = ~(c2 | l2 | r2);  // free columns of the next row
-        lastrow = PUSHLAST ? false : one_free(c2);
-    }
+    const uint32_t c2 = MADD ? p * m1 + c : c | p;
+    const uint32_t a2 = ~(c2 | l2 | r2);  // free columns of the next row
+    const bool lastrow = PUSHLAST ? false : one_free(c2);
     const bool live = a2 != 0u;
     if (PUSHLAST)
         s32 += (c2 == ~0u) ? 1u : 0u;  // every column holds a queen: a solution
@@ -233,9 +228,8 @@ __device__ __forceinline__ void step_reg(uint32_t &c, uint32_t &l, uint32_t &r, 
             c = f.x; l = f.y; r = f.z; av = f.w;
         } else {
             record_error(k.status, NQ_ESTACK);
-            c = CONSTR ? kSentinelC : MADD ? 0xAAAAAAAAu : ~0u;
-            l = r = CONSTR ? kSentinelLrC : MADD ? 0xAAAAAAAAu : ~0u;
-            av = CONSTR ? kSentinelAvC : MADD ? 0x55555555u : ~0u;
+            c = l = r = MADD ? 0xAAAAAAAAu : ~0u;
+            av = MADD ? 0x55555555u : ~0u;
         }
     } else if (push) {
         c = c2; l = l2; r = r2; av = a2;
@@ -601,7 +595,7 @@ __device__ __forceinline__ void step_paper(uint32_t &top, const Lane &k, uint32_
     }
 }
 
-template <int LAYOUT, bool DIAG, bool CONSTR, bool DONATE, bool STREAM = false>
+template <int LAYOUT, bool DIAG, bool DONATE, bool STREAM = false>
 __device__ __forceinline__ void search_body(const SearchArgs &a) {
     // the multiply-add family: REGM, and its forms with the last row pushed
     // (REGP), split-word frames (REGZ) or both (REGPZ)
@@ -622,9 +616,8 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
     // (half the bookkeeping per node; measured 2.2 % faster at N=18).
     constexpr bool kTwo = kRegm && !DIAG && !DONATE;
     constexpr int kSteps = kTwo ? 31 : kChunk;
-    static_assert(kSteps < 32, "two 16-step sentinels hold 32 idle steps (54 constrained)");
-    static_assert(kReg || !CONSTR, "constrained mode uses the REG layout");
-    static_assert(!(kPushLast || kSplit || kAvail) || (!CONSTR && !DONATE),
+    static_assert(kSteps < 32, "two 16-step sentinels hold 32 idle steps");
+    static_assert(!(kPushLast || kSplit || kAvail) || !DONATE,
                   "REGP / REGZ / REGPZ / AVAIL: plain and streamed search only");
     constexpr uint32_t kElem = stack_elem_bytes(kWt32);  // bytes of one slot in one array
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(nq_smem);
@@ -645,21 +638,15 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
         k.base = sbase + stack_slot_offset(blockDim.x, threadIdx.x, 0u, kElem);
     }
     k.limit = k.base + (uint32_t)a.slots * k.stride;
-    // WT32: bytes per array; constrained mode: address of allowed[] after the stacks
-    const uint32_t arr = stack_array_bytes(blockDim.x, (uint32_t)a.slots, kElem);
-    k.table = kWt32 ? arr : sbase + arr;
-    k.thr = 0;
+    // WT32: bytes per array
+    k.table = stack_array_bytes(blockDim.x, (uint32_t)a.slots, kElem);
     k.status = a.status;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt_mask = (1u << lane) - 1u;
     const uint32_t m1 = a.mul[0], m2 = a.mul[1], mneg = a.mul[2], mhalf = a.mul[3];
-    if (CONSTR) {
-        if (threadIdx.x < 32) sts1(k.table + threadIdx.x * 4u, a.allowed[threadIdx.x]);
-        __syncthreads();
-    }
-    const uint32_t sent_c = CONSTR ? kSentinelC : kArith ? 0xAAAAAAAAu : ~0u;
-    const uint32_t sent_lr = CONSTR ? kSentinelLrC : kArith ? 0xAAAAAAAAu : ~0u;
-    const uint32_t sent_av = CONSTR ? kSentinelAvC : kArith ? 0x55555555u : ~0u;
+    const uint32_t sent_c = kArith ? 0xAAAAAAAAu : ~0u;
+    const uint32_t sent_lr = sent_c;
+    const uint32_t sent_av = kArith ? 0x55555555u : ~0u;
 
     uint32_t c = sent_c, l = sent_lr, r = sent_lr, av = sent_av;  // the top frame
     uint32_t top = k.base;                                       // byte offset
@@ -693,7 +680,7 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
 
     // With donation a subproblem's count can arrive in several parts (the
     // host zeroes counts and nodes first), so the parts are added.
-    constexpr bool donating = DONATE && kReg && !CONSTR;
+    constexpr bool donating = DONATE && kReg;
     uint32_t waits = 0;
     uint64_t ticket = kNone;    // donation ticket this lane waits on
     // lane 0: the donation counters as loaded at the last bookkeeping point
@@ -813,7 +800,6 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
                     const bool ok = n >= 1u && (a.expect_n == 0 || (int)n == a.expect_n) &&
                                     (w == 1u || w == 2u) && d <= n && (P.x & ~last) == 0u &&
                                     (uint32_t)__popc(P.x) == d &&
-                                    (!CONSTR || n <= (uint32_t)kMaxConstrainedN) &&
                                     (!kAvail || n <= 30u);  // AVAIL: two guard columns
                     const int need_slots =
                         kAvail ? (int)n - 2 - (int)d  // words of rows d..N-3
@@ -830,14 +816,8 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
                     } else {
                         const uint32_t l0 = P.y;
                         const uint32_t r0 = P.z & last;
-                        uint32_t c0, a0;
-                        if (CONSTR) {
-                            c0 = P.x | (d << kRowShift);
-                            a0 = ~(c0 | l0 | r0) & lds1(k.table + (d << 2)) & last;
-                        } else {
-                            c0 = P.x | ~last;
-                            a0 = ~(c0 | l0 | r0);
-                        }
+                        const uint32_t c0 = P.x | ~last;
+                        const uint32_t a0 = ~(c0 | l0 | r0);
                         if (d == n) {
                             finish(pi, 1, 0, w, n);  // the prefix is a solution
                         } else if (d + 1u == n || a0 == 0u) {
@@ -845,7 +825,6 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
                             finish(pi, s, s, w, n);
                         } else {
                             idx = pi; wt = w; pn = n; sol = 0; nod = 0;
-                            k.thr = (n - 1u) << kRowShift;
                             if (kAvail) {  // columns moved up one bit, guards pre-set
                                 c = (P.x << 1) | ~(last << 1);
                                 l = l0 << 1;
@@ -1062,19 +1041,14 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
         for (int j = 0; j < kSteps; ++j) {
             if constexpr (kAvail)
                 step_avail<DIAG>(c, l, r, av, top, k, s32, n32, m1, m2, mneg, mhalf);
-            else if constexpr (kRegm && CONSTR && DIAG)
-                step_reg<DIAG, true, true>(c, l, r, av, top, k, s32, n32, m1, m2, mneg, mhalf);
-            else if constexpr (kRegm && CONSTR)
-                step_regm_constr(c, l, r, av, top, k.stride, k.table, k.thr, s32, m1, m2, mneg,
-                                 mhalf);
             else if constexpr (kRegm && DIAG)
-                step_reg<DIAG, false, true, kPushLast, kSplit>(c, l, r, av, top, k, s32, n32, m1,
+                step_reg<DIAG, true, kPushLast, kSplit>(c, l, r, av, top, k, s32, n32, m1,
                                                                m2, mneg, mhalf);
             else if constexpr (kRegm)
                 step_regm<kPushLast, kSplit>(c, l, r, av, top, k.stride, s32, m1, m2, mneg,
                                              mhalf);
             else if constexpr (kReg)
-                step_reg<DIAG, CONSTR>(c, l, r, av, top, k, s32, n32);
+                step_reg<DIAG>(c, l, r, av, top, k, s32, n32);
             else if constexpr (kWt)
                 step_wt<DIAG>(c, l, r, av, top, k, s32, n32);
             else if constexpr (kWt32)
@@ -1343,28 +1317,28 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
 
 // The production kernel is held to 48 registers (5 resident blocks of 256 at
 // N=18, d=7); the donating variant carries the queue logic and gets 64.
-template <int LAYOUT, bool DIAG, bool CONSTR>
+template <int LAYOUT, bool DIAG>
 __global__ void __maxnreg__(48) search_kernel(const SearchArgs a) {
-    search_body<LAYOUT, DIAG, CONSTR, false>(a);
+    search_body<LAYOUT, DIAG, false>(a);
 }
 template <int LAYOUT, bool DIAG>
 __global__ void __maxnreg__(64) search_kernel_donate(const SearchArgs a) {
-    search_body<LAYOUT, DIAG, false, true>(a);
+    search_body<LAYOUT, DIAG, true>(a);
 }
 
 // Streamed input (nq_total_ex): a build of its own, so that the plain kernel
 // carries none of the publication checks.
 template <int LAYOUT, bool DIAG>
 __global__ void __maxnreg__(48) search_kernel_stream(const SearchArgs a) {
-    search_body<LAYOUT, DIAG, false, false, true>(a);
+    search_body<LAYOUT, DIAG, false, true>(a);
 }
 
-template <int LAYOUT, bool DIAG, bool CONSTR, bool DONATE = false>
+template <int LAYOUT, bool DIAG, bool DONATE = false>
 void *kernel_ptr() {
     if constexpr (DONATE)
         return reinterpret_cast<void *>(&search_kernel_donate<LAYOUT, DIAG>);
     else
-        return reinterpret_cast<void *>(&search_kernel<LAYOUT, DIAG, CONSTR>);
+        return reinterpret_cast<void *>(&search_kernel<LAYOUT, DIAG>);
 }
 
 template <int LAYOUT, bool DIAG>
@@ -1377,7 +1351,7 @@ void *stream_ptr(bool diag) {
 }
 template <int LAYOUT>
 void *plain_ptr(bool diag) {
-    return diag ? kernel_ptr<LAYOUT, true, false>() : kernel_ptr<LAYOUT, false, false>();
+    return diag ? kernel_ptr<LAYOUT, true>() : kernel_ptr<LAYOUT, false>();
 }
 
 void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
@@ -1386,21 +1360,19 @@ void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
         switch (layout) {
             case NQ_LAYOUT_REGM: return stream_ptr<NQ_LAYOUT_REGM>(diag);
             case NQ_LAYOUT_REGP:
-                return diag ? stream_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(true, false);
+                return diag ? stream_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(true, false, false);
             case NQ_LAYOUT_REGZ: return stream_ptr<NQ_LAYOUT_REGZ>(diag);
             case NQ_LAYOUT_REGPZ: return stream_ptr<NQ_LAYOUT_REGPZ>(diag);
             default: return stream_ptr<NQ_LAYOUT_REG>(diag);
         }
     }
-    if (constrained)
+    if (constrained) return look_kernel_ptr(false, true, true);
+    if (donate && layout == NQ_LAYOUT_REGM)
         return diag ? kernel_ptr<NQ_LAYOUT_REGM, true, true>()
                     : kernel_ptr<NQ_LAYOUT_REGM, false, true>();
-    if (donate && layout == NQ_LAYOUT_REGM)
-        return diag ? kernel_ptr<NQ_LAYOUT_REGM, true, false, true>()
-                    : kernel_ptr<NQ_LAYOUT_REGM, false, false, true>();
     if (donate && layout == NQ_LAYOUT_REG)
-        return diag ? kernel_ptr<NQ_LAYOUT_REG, true, false, true>()
-                    : kernel_ptr<NQ_LAYOUT_REG, false, false, true>();
+        return diag ? kernel_ptr<NQ_LAYOUT_REG, true, true>()
+                    : kernel_ptr<NQ_LAYOUT_REG, false, true>();
     switch (layout) {
         case NQ_LAYOUT_PAPER: return plain_ptr<NQ_LAYOUT_PAPER>(diag);
         case NQ_LAYOUT_WT: return plain_ptr<NQ_LAYOUT_WT>(diag);
@@ -1409,7 +1381,7 @@ void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
         case NQ_LAYOUT_WTM: return plain_ptr<NQ_LAYOUT_WTM>(diag);
         case NQ_LAYOUT_REGM: return plain_ptr<NQ_LAYOUT_REGM>(diag);
         case NQ_LAYOUT_REGP:
-            return diag ? kernel_ptr<NQ_LAYOUT_REGP, true, false>() : look_kernel_ptr(false, split);
+            return diag ? kernel_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(false, split, false);
         case NQ_LAYOUT_REGZ: return plain_ptr<NQ_LAYOUT_REGZ>(diag);
         case NQ_LAYOUT_REGPZ: return plain_ptr<NQ_LAYOUT_REGPZ>(diag);
         case NQ_LAYOUT_AVAIL: return plain_ptr<NQ_LAYOUT_AVAIL>(diag);
@@ -1444,19 +1416,19 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
     Plan p{};
     p.layout = (cfg && cfg->layout) ? cfg->layout : NQ_LAYOUT_DEFAULT_SEARCH;
     if (p.layout < NQ_LAYOUT_PAPER || p.layout > NQ_LAYOUT_LAST) return NQ_EINVAL;
-    if (constrained) p.layout = NQ_LAYOUT_REGM;  // the constrained multiply-add step
+    if (constrained) p.layout = NQ_LAYOUT_REGP;  // (under row masks)
     p.block = (cfg && cfg->block) ? cfg->block : 256;
     if (p.block < 32 || p.block > 1024 || p.block % 32) return NQ_EINVAL;
     // split-word kernels are compiled for one block size
     if (layout_split_words(p.layout) && p.block != (int)kZBlock) return NQ_EINVAL;
     if (p.layout == NQ_LAYOUT_AVAIL && max_n > 30) return NQ_EINVAL;  // guard columns
-    p.look = p.layout == NQ_LAYOUT_REGP && !diag && !constrained;
+    p.look = p.layout == NQ_LAYOUT_REGP && !diag;
     p.levels = p.look ? levels : 0;
     p.rows = max_n - min_d;
     // (a split record's search starts `levels - 1` rows further down)
     p.slots = slots_needed(p.layout, max_n, p.levels ? std::min(max_n, min_d + p.levels - 1) : min_d);
     const size_t per_thread = (size_t)p.slots * (p.layout == NQ_LAYOUT_AVAIL ? 4u : 16u);
-    const size_t extra = constrained ? 32u * 4u : 0u;
+    const size_t extra = constrained ? 32u * 8u : 0u;  // the masks, two rows to an entry
     if ((size_t)p.block * per_thread + extra > (size_t)max_smem) {
         int fit = (int)(((size_t)max_smem - extra) / per_thread) / 32 * 32;
         if (fit < 32 || layout_split_words(p.layout)) return NQ_ESTACK;
@@ -1520,63 +1492,87 @@ double subtree_steps(int n, int rows) {
                     0.013134 * n * n);
 }
 
-// Digit of a split level: enough bits for every column that the row could have
-// free, and 2 on the last level, whose digit strides over the free columns.
-int digit_bits(int free_columns, bool last) {
-    int b = 1;
-    while ((1 << b) < free_columns) ++b;
-    return last ? 2 : b;
+// How the records' subtrees are cut into units.
+struct Cut {
+    int levels = 0, shift = 0;  // rows that the units fix, bits of a unit's index
+    uint32_t digits = 0;        // bits of each level's digit, a nibble each
+};
+
+// cap[j]: the most columns that row j below a record could have free (rows
+// with one are passed through), for `rows` rows; the records lie on boards
+// that search like a free board of size `board`.
+//
+// Split while there is less than a unit for every fourth lane and a unit is not
+// small in itself (setting one up costs some ten steps), or while a unit is
+// more than an eighth of a lane's share of the work (the largest are a few
+// times the mean). A level more or less where the line lies costs little
+// (N = 16, d = 5: 1 level 0.60 ms, 2 levels 0.56 ms, none 1.25 ms; N = 18, d =
+// 5: 20.3, 18.4, 38.9 ms), a missing one much (2048 records of N = 22, d = 7:
+// 1 level 44 ms, 3 levels 5.5 ms, 4 levels 4.5 ms, 5 levels 6.5 ms, none
+// 326 ms).
+Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, bool at_least_one) {
+    int open_rows[NQ_MAX_N + 2] = {};  // rows j.. with a choice
+    for (int j = rows - 1; j >= 0; --j) open_rows[j] = open_rows[j + 1] + (cap[j] > 1 ? 1 : 0);
+    Cut cut;
+    const double share = (double)n * subtree_steps(board, open_rows[0]) / lanes;
+    double live = (double)n;                              // units that hold something
+    double unit = subtree_steps(board, open_rows[0]);     // steps below one
+    while (cut.levels < rows) {
+        const bool few = live < lanes / 4.0 && unit > 150.0;
+        const bool uneven = unit > std::max(750.0, share / 8.0);
+        if (!few && !uneven && (cut.levels || !at_least_one)) break;
+        Cut c;
+        c.levels = cut.levels + 1;
+        while (c.levels < rows && cap[c.levels - 1] <= 1) ++c.levels;
+        if (c.levels > kSplitMaxLevels) break;
+        double lv = (double)n, un = 0.0;
+        for (int j = 0; j < c.levels; ++j) {
+            // Enough bits for every column that could be free; at most 2 on the
+            // last level, whose digit strides over the free columns.
+            const bool last = j + 1 == c.levels;
+            int b = 0;
+            while ((1 << b) < cap[j]) ++b;
+            if (last) b = std::min(b, 2);
+            const double open = std::max(1.0, 0.6 * cap[j]);  // columns free, about
+            const double taken = last ? std::min(open, (double)(1 << b)) : open;
+            c.digits |= (uint32_t)b << (4 * j);
+            c.shift += b;
+            lv *= taken;
+            if (last) un = subtree_steps(board, open_rows[j]) / taken;
+        }
+        if (c.shift > 31 || n > (1ull << (62 - c.shift))) break;
+        cut = c;
+        live = lv;
+        unit = un;
+    }
+    return cut;
 }
 
 }  // namespace
 
 int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t n, bool may_split,
-                 Plan *plan) {
+                 Plan *plan, const uint32_t *allowed) {
     if (!plan->look) return NQ_OK;
     Plan p = *plan;
     const uint32_t claim = cfg && cfg->claim > 0 ? (uint32_t)cfg->claim : 1u;
     const double lanes = (double)p.grid * p.block;
-    int levels = 0, shift = 0;
-    uint32_t digits = 0;
+    Cut cut;
     if (may_split && !p.stream && n) {
-        // Split while there is less than a unit for every fourth lane and a unit
-        // is not small in itself (setting one up costs some ten steps), or while
-        // a unit is more than an eighth of a lane's share of the work (the
-        // largest are a few times the mean). A level more or less where the line
-        // lies costs little (N = 16, d = 5: 1 level 0.60 ms, 2 levels 0.56 ms,
-        // none 1.25 ms; N = 18, d = 5: 20.3, 18.4, 38.9 ms), a missing one much
-        // (2048 records of N = 22, d = 7: 1 level 44 ms, 3 levels 5.5 ms, 4
-        // levels 4.5 ms, 5 levels 6.5 ms, none 326 ms).
-        const double share = (double)n * subtree_steps(max_n, p.rows) / lanes;
-        double live = (double)n;                            // units that hold something
-        double unit = subtree_steps(max_n, p.rows);         // steps below one
-        while (levels < kSplitMaxLevels && levels < p.rows) {
-            const bool few = live < lanes / 4.0 && unit > 150.0;
-            const bool uneven = unit > std::max(750.0, share / 8.0);
-            if (!few && !uneven) break;
-            int sh = 0;
-            uint32_t dg = 0;
-            double lv = (double)n, un = 0.0;
-            for (int j = 0; j <= levels; ++j) {
-                const bool last = j == levels;
-                const int b = digit_bits(p.rows - j, last);
-                const double open = 0.6 * (p.rows - j);  // free columns of a row, about
-                dg |= (uint32_t)b << (4 * j);
-                sh += b;
-                lv *= last ? std::min(open, (double)(1 << b)) : open;
-                if (last)
-                    un = subtree_steps(max_n, p.rows - j) / std::max(1.0, std::min(open, (double)(1 << b)));
+        int cap[NQ_MAX_N + 1] = {}, board = max_n;
+        for (int j = 0; j < p.rows; ++j) {
+            cap[j] = p.rows - j;
+            if (allowed) {
+                cap[j] = std::min(cap[j], __builtin_popcount(allowed[min_d + j]));
+                if (cap[j] <= 1 && board > 1) --board;  // a given queen takes its row and column
             }
-            if (sh > 31 || n > (1ull << (62 - sh))) break;
-            ++levels;
-            shift = sh;
-            digits = dg;
-            live = lv;
-            unit = un;
         }
+        cut = choose_cut(cap, p.rows, board, n, lanes, allowed != nullptr);
     }
+    const int levels = cut.levels, shift = cut.shift;
+    const uint32_t digits = cut.digits;
     if (levels) {
-        const int rc = make_plan(max_n, min_d, diag, false, cfg, &p, false, false, levels);
+        const int rc =
+            make_plan(max_n, min_d, diag, allowed != nullptr, cfg, &p, false, false, levels);
         if (rc) return rc;
     }
     p.split_shift = shift;
@@ -1584,12 +1580,15 @@ int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t
     // A warp takes 32 indices x claim at once. Of split work: half of that
     // where the first ranges cover everything (other warps get the rest and
     // each one's lanes share), and more where the empty units among them are
-    // many, as long as every warp still takes about 64 ranges.
+    // many, as long as every warp still takes some 64 ranges -- 8 under row
+    // masks, where one record's units are nearly all empty (six queries at N =
+    // 16: 2.0 ms at 64 ranges, 1.7 ms at 8; 2048 records of N = 22: 4.4 ms at
+    // 64, 5.3 ms at 8).
     const uint64_t total = n << shift;
     const uint64_t warps = (uint64_t)p.grid * (uint64_t)(p.block / 32);
     p.range = 32u * std::min(claim, 1024u);
     if (levels && total <= warps * 16u) p.range = 16u;
-    while (levels && p.range < 32768u && total / p.range > 128 * warps) p.range *= 2u;
+    while (levels && p.range < 32768u && total / p.range > (allowed ? 16 : 128) * warps) p.range *= 2u;
     p.cursor = total > warps * p.range;
     if (!p.cursor)  // no more blocks than ranges: few records take one warp of each block
         p.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(p.grid, (total + p.range - 1) / p.range));

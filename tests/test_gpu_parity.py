@@ -483,3 +483,29 @@ def test_split_launch_with_boards_that_end_early():
     assert e.value.code == nq.NQ_EINVAL
     want[7] = 0
     assert np.array_equal(u64(cnt), want)
+
+
+def one_solution(n):
+    """Columns of one solution of an even n >= 8 board, by the even-odd construction."""
+    even, odd = list(range(2, n + 1, 2)), list(range(1, n + 1, 2))
+    if n % 6 == 2:
+        odd = [3, 1] + odd[3:] + [5]
+    return [c - 1 for c in even + odd]
+
+
+@pytest.mark.parametrize("n,k", [(1, 1), (4, 1), (8, 8), (8, 1), (12, 1), (14, 2), (16, 4), (18, 7),
+                                 (20, 9), (22, 12), (24, 13), (26, 15)])
+def test_constrained_whole_board_split(orc, n, k):
+    """Partial boards of every width the row field allows (N <= 26), counted as one
+    split record under row masks: few and many given queens, boards that end in the
+    split levels, given queens in the first, middle and last rows."""
+    cols = one_solution(n) if n >= 8 else [1, 3, 0, 2] if n == 4 else [0]
+    top = [(r, cols[r]) for r in range(k)]  # (the oracle places rows from the top)
+    want = orc.count_constrained(n, top)[0]
+    for qs in (top, [(n - 1 - r, c) for r, c in top], [(c, r) for r, c in top],
+               [(c, n - 1 - r) for r, c in top[::-1]]):
+        assert nq.count_constrained(n, qs) == want, qs  # the board's symmetries
+    if n <= 12:
+        g = synth_inputs.SplitMix64(7000 + 32 * n + k)
+        qs = [(r, cols[r]) for r in synth_inputs.sample_ranks(g.next_u64(), n, k)]
+        assert nq.count_constrained(n, qs) == orc.count_constrained(n, qs)[0], qs
