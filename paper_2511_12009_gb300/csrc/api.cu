@@ -108,6 +108,23 @@ struct CallCtx {
     }
 };
 
+// The three timing events of a synchronous call.
+struct CallEvents {
+    cudaEvent_t e[3] = {};
+    int init() {
+        for (auto &x : e)
+            if (cudaEventCreate(&x) != cudaSuccess) {
+                x = nullptr;
+                return NQ_ECUDA;
+            }
+        return NQ_OK;
+    }
+    ~CallEvents() {
+        for (auto &x : e)
+            if (x) cudaEventDestroy(x);
+    }
+};
+
 // Enqueue one search over device-resident prefixes (shared by nq_count*,
 // nq_total_ex, nq_count_constrained and nq_count_split). n_tags > 0: the
 // records are split subproblems whose counts and nodes are added into entry
@@ -245,7 +262,82 @@ extern "C" int nq_sync(void *stream) {
     return take_status(status, s);
 }
 
-// nq_total_ex streams large prefix sets: below this many subproblems the set
+namespace {
+
+// nq_total_ex in the default form: the launch splits subtrees by itself
+// (plan_records), so only the prefixes of the first kTotalRows rows are made and
+// copied, some 10^4 records, and the depth-d set is only counted, beside
+// the search, for the caller who asks. Before, the host wrote all of it (N = 18:
+// 7.4 M records, 2.8 ms of host work and 118 MB beside the search).
+// kTotalRows: rows 0 and 1 hold the symmetry rules; two more leave the launch two
+// levels less to split at next to no host work (N = 14: search of 0.081, 0.082,
+// 0.064, 0.091 ms from 2, 3, 4, 5 rows; N = 17: 3.45, 3.58, 3.26, 3.15 ms).
+constexpr int kTotalRows = 4;
+
+int total_split(int N, int d, const nq_config *cfg, uint64_t *total_out, nq_timing *timing) {
+    const auto t_start = Clock::now();
+    const int b = std::min(d, kTotalRows);
+    uint64_t n = 0;
+    int rc = nq_enumerate_prefixes(N, b, nullptr, 0, &n);
+    if (rc) return rc;
+    // one block: [0] work cursor, [1] status, [2..33] totals, then the records
+    constexpr size_t kHead = 34 * sizeof(uint64_t);
+    static_assert(kHead % sizeof(nq_prefix) == 0, "the records are 16-byte aligned");
+    const size_t bytes = kHead + n * sizeof(nq_prefix);
+    unsigned char *stage = static_cast<unsigned char *>(t_stage.get(bytes));
+    if (!stage) return NQ_ENOMEM;
+    std::memset(stage, 0, kHead);
+    if (n && (rc = nq_enumerate_prefixes(N, b, reinterpret_cast<nq_prefix *>(stage + kHead), n, &n)))
+        return rc;
+    const double enum_ms = ms_since(t_start);
+    CallCtx ctx;
+    if ((rc = ctx.init())) return rc;
+    unsigned char *dev = nullptr;
+    if ((rc = ctx.alloc(&dev, bytes))) return rc;
+    auto *d_head = reinterpret_cast<uint64_t *>(dev);
+    CallEvents ev;
+    if (timing && (rc = ev.init())) return rc;
+    if (timing) cudaEventRecord(ev.e[0], ctx.s);
+    rc = cuda_rc(cudaMemcpyAsync(dev, stage, bytes, cudaMemcpyHostToDevice, ctx.s));
+    if (timing) cudaEventRecord(ev.e[1], ctx.s);
+    Plan p{};
+    if (!rc)
+        rc = enqueue_search(reinterpret_cast<nq_prefix *>(dev + kHead), n, N, b, N, nullptr, nullptr,
+                            d_head + 2, cfg, nullptr, ctx.s, &p, reinterpret_cast<int *>(d_head + 1),
+                            0, reinterpret_cast<unsigned long long *>(d_head));
+    if (timing) cudaEventRecord(ev.e[2], ctx.s);
+    // (the staging block's head takes the results: its records are on the device
+    // before the copy back runs)
+    if (!rc)
+        rc = cuda_rc(cudaMemcpyAsync(stage, dev, kHead, cudaMemcpyDeviceToHost, ctx.s));
+    uint64_t prefixes = n;
+    if (!rc && timing && d > b) rc = nq_enumerate_prefixes(N, d, nullptr, 0, &prefixes);
+    if (cudaStreamSynchronize(ctx.s) != cudaSuccess) return NQ_ECUDA;
+    if (rc) return rc;
+    const auto *head = reinterpret_cast<const uint64_t *>(stage);
+    const int st = *reinterpret_cast<const int *>(head + 1);
+    if (st) return st;
+    *total_out = head[2 + N];
+    if (timing) {
+        float up = 0, kern = 0;
+        cudaEventElapsedTime(&up, ev.e[0], ev.e[1]);
+        cudaEventElapsedTime(&kern, ev.e[1], ev.e[2]);
+        timing->enumerate_ms = enum_ms;
+        timing->upload_ms = up;
+        timing->kernel_ms = kern;
+        timing->prefixes = prefixes;
+        timing->d = d;
+        timing->layout = p.layout;
+        timing->block = p.block;
+        timing->grid = p.grid;
+        timing->total_ms = ms_since(t_start);
+    }
+    return NQ_OK;
+}
+
+}  // namespace
+
+// The other forms stream large prefix sets: below this many subproblems the set
 // is written, copied and searched in one go.
 constexpr uint64_t kStreamMin = 1ull << 20;
 constexpr int kStreamPieces = 8;
@@ -259,6 +351,9 @@ extern "C" int nq_total_ex(int N, const nq_config *cfg, uint64_t *total_out, uin
     cfg = &cfg_eff;
     const int d = cfg->d > 0 ? cfg->d : nq_default_depth(N);
     if (d < 0 || d > N) return NQ_EINVAL;
+
+    const int lay = cfg->layout ? cfg->layout : NQ_LAYOUT_DEFAULT_SEARCH;
+    if (lay == NQ_LAYOUT_REGP && !nodes_out) return total_split(N, d, cfg, total_out, timing);
 
     // a1 (counting pass): the set cut at its depth-3 nodes, the size of each part
     const auto t_enum = Clock::now();
@@ -336,9 +431,8 @@ extern "C" int nq_total_ex(int N, const nq_config *cfg, uint64_t *total_out, uin
         cs = nullptr;
         return NQ_ECUDA;
     }
-    // streamed input needs a register-stack layout (the default); any other
-    // layout searches once every piece is in
-    const int lay = cfg->layout ? cfg->layout : NQ_LAYOUT_DEFAULT_SEARCH;
+    // streamed input needs a register-stack layout; any other layout searches
+    // once every piece is in
     const bool stream_in = npieces > 1 && layout_register_top(lay);
     cudaEventRecord(ev[0], ctx.s);
     rc = cuda_rc(cudaMemsetAsync(d_tot, 0, 32 * sizeof(uint64_t), ctx.s));
@@ -432,23 +526,6 @@ extern "C" int nq_total(int N, uint64_t *total_out) {
     return nq_total_ex(N, nullptr, total_out, nullptr, nullptr);
 }
 
-// The three timing events of a split call.
-struct SplitEvents {
-    cudaEvent_t e[3] = {};
-    int init() {
-        for (auto &x : e)
-            if (cudaEventCreate(&x) != cudaSuccess) {
-                x = nullptr;
-                return NQ_ECUDA;
-            }
-        return NQ_OK;
-    }
-    ~SplitEvents() {
-        for (auto &x : e)
-            if (x) cudaEventDestroy(x);
-    }
-};
-
 // ---------------------------------------------------------------------------
 // Host-side split: few heavy subproblems (fewer than the grid has lanes) are
 // extended a few rows deeper on the host, every child carrying its parent's
@@ -522,7 +599,7 @@ extern "C" int nq_count_split(const nq_prefix *h_prefixes, uint64_t n, int rows,
         uint64_t *d_out = nullptr;  // [0..31] totals, [32] status, then the counts
         if ((rc = ctx.alloc(&d_pre, n * sizeof(nq_prefix)))) return rc;
         if ((rc = ctx.alloc(&d_out, (34 + n) * sizeof(uint64_t)))) return rc;
-        SplitEvents ev;
+        CallEvents ev;
         if ((rc = ev.init())) return rc;
         cudaEventRecord(ev.e[0], ctx.s);
         rc = cuda_rc(cudaMemcpyAsync(d_pre, h_prefixes, n * sizeof(nq_prefix),
@@ -581,7 +658,7 @@ extern "C" int nq_count_split(const nq_prefix *h_prefixes, uint64_t n, int rows,
     if (diag && (rc = ctx.alloc(&d_nodes, n * sizeof(uint64_t)))) return rc;
     if ((rc = ctx.alloc(&d_tot, 32 * sizeof(uint64_t) + 16))) return rc;
     int *d_status = reinterpret_cast<int *>(d_tot + 32);
-    SplitEvents evs;
+    CallEvents evs;
     if ((rc = evs.init())) return rc;
     cudaEvent_t *ev = evs.e;
     cudaEventRecord(ev[0], ctx.s);

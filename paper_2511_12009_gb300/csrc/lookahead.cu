@@ -30,9 +30,6 @@ namespace nqi {
 namespace {
 
 constexpr int kLookSteps = 31;  // steps between bookkeeping points
-// Idle lanes for which a warp of a split launch takes a new range (before that
-// they take frames of the warp's own busy lanes).
-constexpr int kRefill = 8;
 
 // The sentinel frame, in slot 0 of every stack: whatever candidate bit p is
 // taken, cols + p, L + 2p and R + p/2 together cover all 32 bits (each of the
@@ -234,7 +231,7 @@ __device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint32_t
 // Units that cannot hold anything are passed over in one go: the warp's
 // position moves on by the last asking lane's skip.
 // MASKED (split only): one table of row masks for the launch, above the stacks.
-template <bool STREAM, bool SPLIT, bool MASKED>
+template <bool SPLIT, bool MASKED>
 __device__ __forceinline__ void look_body(const SearchArgs &a) {
     static_assert(SPLIT || !MASKED, "masked searches are split");
     constexpr uint32_t kSC = MASKED ? kSentMaskedC : kSentC, kSL = MASKED ? 0u : kSentL,
@@ -278,7 +275,6 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     uint64_t next = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * range;
     uint32_t rem = next < total ? (uint32_t)(total - next < range ? total - next : range) : 0u;
     bool exhausted = a.cursor == nullptr;
-    uint32_t waits = 0;
 
     auto finish = [&](uint64_t i, uint64_t s, uint32_t w_n) {
         if (SPLIT) {
@@ -315,7 +311,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
         unsigned need_mask = __ballot_sync(~0u, need);
         while (need_mask) {
             if (rem == 0u) {
-                if (exhausted || (SPLIT && __popc(need_mask) < kRefill)) break;
+                if (exhausted || (SPLIT && __popc(need_mask) < a.refill)) break;
                 unsigned long long f = 0;
                 if (lane == 0) f = atomicAdd(a.cursor, (unsigned long long)range);
                 next = __shfl_sync(~0u, f, 0) + warps * range;
@@ -325,16 +321,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                 }
                 rem = total - next < range ? (uint32_t)(total - next) : range;
             }
-            uint32_t ready = rem;
-            if (STREAM) {  // streamed input: only what has been published may be read
-                unsigned long long v = 0;
-                if (lane == 0)
-                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v)
-                                 : "l"(a.published) : "memory");
-                v = __shfl_sync(~0u, v, 0);
-                ready = v <= next ? 0u : v - next < rem ? (uint32_t)(v - next) : rem;
-                if (ready == 0u) break;
-            }
+            const uint32_t ready = rem;
             const uint32_t rank = __popc(need_mask & lt_mask);
             uint32_t skip = 1u;
             if (need && rank < ready) {
@@ -345,14 +332,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                     at >>= a.split_shift;
                 }
                 const uint64_t pi = a.order ? a.n - 1 - at : at;
-                uint4 P;
-                if (STREAM)  // (a line may have been cached before its copy arrived)
-                    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(P.x), "=r"(P.y), "=r"(P.z), "=r"(P.w)
-                                 : "l"(a.pre + pi)
-                                 : "memory");
-                else
-                    P = __ldg(reinterpret_cast<const uint4 *>(a.pre) + pi);
+                const uint4 P = __ldg(reinterpret_cast<const uint4 *>(a.pre) + pi);
                 const uint32_t n = (P.w >> 2) & 31u, d = (P.w >> 7) & 31u, w = P.w & 3u;
                 const uint32_t last = (n >= 1u) ? (0xFFFFFFFFu >> (32u - n)) : 0u;
                 const bool ok = n >= 1u && (a.expect_n == 0 || (int)n == a.expect_n) &&
@@ -414,16 +394,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
             rem -= taken;
             need_mask = __ballot_sync(~0u, need);
         }
-        if (need_mask == ~0u) {  // the whole warp is idle
-            if (!STREAM || (exhausted && rem == 0u)) break;
-            // bounded wait for the host to publish more
-            if (++waits > kMaxPublishWaits) {
-                look_error(a.status, NQ_ETIMEOUT);
-                break;
-            }
-            __nanosleep(256);
-            continue;
-        }
+        if (need_mask == ~0u) break;  // the whole warp is idle, and nothing is left
 
         if (SPLIT && need_mask && rem == 0u) {
             // Each idle lane takes the shallowest saved frame of a busy lane of
@@ -490,26 +461,20 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     }
 }
 
-__global__ void __maxnreg__(48) look_kernel(const SearchArgs a) {
-    look_body<false, false, false>(a);
-}
-__global__ void __maxnreg__(48) look_kernel_stream(const SearchArgs a) {
-    look_body<true, false, false>(a);
-}
+__global__ void __maxnreg__(48) look_kernel(const SearchArgs a) { look_body<false, false>(a); }
 __global__ void __maxnreg__(48) look_kernel_split(const SearchArgs a) {
-    look_body<false, true, false>(a);
+    look_body<true, false>(a);
 }
 __global__ void __maxnreg__(48) look_kernel_masked(const SearchArgs a) {
-    look_body<false, true, true>(a);
+    look_body<true, true>(a);
 }
 
 }  // namespace
 
-void *look_kernel_ptr(bool stream, bool split, bool masked) {
-    return stream   ? reinterpret_cast<void *>(&look_kernel_stream)
-           : masked ? reinterpret_cast<void *>(&look_kernel_masked)
-           : split  ? reinterpret_cast<void *>(&look_kernel_split)
-                    : reinterpret_cast<void *>(&look_kernel);
+void *look_kernel_ptr(bool split, bool masked) {
+    return masked  ? reinterpret_cast<void *>(&look_kernel_masked)
+           : split ? reinterpret_cast<void *>(&look_kernel_split)
+                   : reinterpret_cast<void *>(&look_kernel);
 }
 
 }  // namespace nqi

@@ -76,6 +76,7 @@ struct SearchArgs {
     int levels;
     int split_shift;
     uint32_t digits;
+    int refill;         // idle lanes for which a warp takes a new range of units
 };
 // Bookkeeping rounds a lane may wait for an unpublished index (each round is
 // one chunk of idle steps, plus a short sleep once the whole warp waits):
@@ -191,9 +192,9 @@ struct ServeArgs {
     int *status;                     // the server's error word (device)
 };
 
-// The production kernel of layout REGP (lookahead.cu): plain, for streamed
-// input, with the records' subtrees split, or split and under row masks.
-void *look_kernel_ptr(bool stream, bool split, bool masked);
+// The production kernel of layout REGP (lookahead.cu): plain, with the records'
+// subtrees split, or split and under row masks.
+void *look_kernel_ptr(bool split, bool masked);
 
 int launch_serve(const ServeArgs &a, int grid, int block, size_t smem, cudaStream_t s);
 int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *smem,
@@ -211,7 +212,7 @@ struct Plan {
     bool stream;    // the kernel variant for streamed input (SearchArgs::published)
     // layout REGP's production kernel (SearchArgs has the same names)
     bool look;
-    int rows, levels, split_shift;
+    int rows, levels, split_shift, refill;
     uint32_t digits, range;
     bool cursor;    // the launch takes more than every warp's first range
 };

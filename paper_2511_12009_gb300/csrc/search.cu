@@ -1359,14 +1359,14 @@ void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
     if (stream) {
         switch (layout) {
             case NQ_LAYOUT_REGM: return stream_ptr<NQ_LAYOUT_REGM>(diag);
-            case NQ_LAYOUT_REGP:
-                return diag ? stream_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(true, false, false);
+            case NQ_LAYOUT_REGP:  // (the production build takes no streamed input)
+                return diag ? stream_ptr<NQ_LAYOUT_REGP, true>() : nullptr;
             case NQ_LAYOUT_REGZ: return stream_ptr<NQ_LAYOUT_REGZ>(diag);
             case NQ_LAYOUT_REGPZ: return stream_ptr<NQ_LAYOUT_REGPZ>(diag);
             default: return stream_ptr<NQ_LAYOUT_REG>(diag);
         }
     }
-    if (constrained) return look_kernel_ptr(false, true, true);
+    if (constrained) return look_kernel_ptr(true, true);
     if (donate && layout == NQ_LAYOUT_REGM)
         return diag ? kernel_ptr<NQ_LAYOUT_REGM, true, true>()
                     : kernel_ptr<NQ_LAYOUT_REGM, false, true>();
@@ -1381,7 +1381,7 @@ void *pick_kernel(int layout, bool diag, bool constrained, bool donate = false,
         case NQ_LAYOUT_WTM: return plain_ptr<NQ_LAYOUT_WTM>(diag);
         case NQ_LAYOUT_REGM: return plain_ptr<NQ_LAYOUT_REGM>(diag);
         case NQ_LAYOUT_REGP:
-            return diag ? kernel_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(false, split, false);
+            return diag ? kernel_ptr<NQ_LAYOUT_REGP, true>() : look_kernel_ptr(split, false);
         case NQ_LAYOUT_REGZ: return plain_ptr<NQ_LAYOUT_REGZ>(diag);
         case NQ_LAYOUT_REGPZ: return plain_ptr<NQ_LAYOUT_REGPZ>(diag);
         case NQ_LAYOUT_AVAIL: return plain_ptr<NQ_LAYOUT_AVAIL>(diag);
@@ -1436,7 +1436,7 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
     }
     p.donate = donate && (p.layout == NQ_LAYOUT_REG || p.layout == NQ_LAYOUT_REGM) && !constrained;
     p.stream = stream && !p.donate && !constrained && layout_register_top(p.layout);
-    if (stream && !p.stream) return NQ_EINVAL;
+    if (stream && (!p.stream || p.look)) return NQ_EINVAL;
     void *k = pick_kernel(p.layout, diag, constrained, p.donate, p.stream, p.levels > 0);
     if (!(cfg && cfg->block) && !layout_split_words(p.layout)) {
         // No block size asked for: the one that keeps the most threads resident
@@ -1496,6 +1496,7 @@ double subtree_steps(int n, int rows) {
 struct Cut {
     int levels = 0, shift = 0;  // rows that the units fix, bits of a unit's index
     uint32_t digits = 0;        // bits of each level's digit, a nibble each
+    double live = 0.0;          // units that hold something, about
 };
 
 // cap[j]: the most columns that row j below a record could have free (rows
@@ -1542,7 +1543,7 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, bo
         }
         if (c.shift > 31 || n > (1ull << (62 - c.shift))) break;
         cut = c;
-        live = lv;
+        cut.live = live = lv;
         unit = un;
     }
     return cut;
@@ -1577,6 +1578,12 @@ int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t
     }
     p.split_shift = shift;
     p.digits = digits;
+    // The end of a range idles lanes one by one. With many units to come the
+    // warp takes the next range at once; with few, its idle lanes first take
+    // frames of its busy ones, so that the units go round (Q(19): at 1 idle lane
+    // 147.3 ms, at 8 151.2 ms, at 16 154.6 ms; N = 15 from d = 3: 0.219, 0.214,
+    // 0.172 ms).
+    p.refill = cut.live > 8.0 * lanes ? 1 : 16;
     // A warp takes 32 indices x claim at once. Of split work: half of that
     // where the first ranges cover everything (other warps get the rest and
     // each one's lanes share), and more where the empty units among them are
@@ -1608,6 +1615,7 @@ int launch_search(const SearchArgs &a, const Plan &p, bool diag, bool constraine
     args.levels = p.levels;
     args.split_shift = p.split_shift;
     args.digits = p.digits;
+    args.refill = p.refill;
     if (p.look && !p.cursor) args.cursor = nullptr;
     void *params[] = {&args};
     const cudaError_t e = cudaLaunchKernel(k, dim3(p.grid), dim3(p.block), params, p.smem, s);
