@@ -30,6 +30,9 @@
  *     streams share one overflow word. A status nq_sync has not collected
  *     stays with the stream handle, also for a later stream that reuses it.
  *   - N is in 1..NQ_MAX_N (bit b of a mask is column b, so N <= 31).
+ *   - Between calls the library keeps, per device context, up to 64 MB of device
+ *     memory in a pool of its own, up to 8 idle streams, and the launch shapes
+ *     it has planned; nq_count_host_noalloc uses none of the pool.
  *   - Thread safety: calls on different streams may run concurrently, and an
  *     error found by one stream's work is reported only by that stream's
  *     nq_sync.

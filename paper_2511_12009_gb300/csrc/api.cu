@@ -4,6 +4,8 @@
 #include <cstdlib>
 #include <cstring>
 #include <memory>
+#include <mutex>
+#include <unordered_map>
 #include <vector>
 
 #include "nq_internal.h"
@@ -85,23 +87,97 @@ struct PinnedBuf {
 };
 thread_local PinnedBuf t_stage;
 
+// What synchronous calls keep between them, per device context: a memory pool
+// of the library's own that holds on to kPoolKeep bytes when a stream
+// synchronises (the device's default pool gives everything back to the driver
+// then, so that each call mapped its few kilobytes anew: most of the 290 us
+// that nq_total(8) took), and up to kStreamsKept idle streams. A stream is
+// kept only once its work is done, and by one call at a time.
+constexpr uint64_t kPoolKeep = 64ull << 20;  // (a pool grows by 32 MB at a time)
+constexpr size_t kStreamsKept = 8;
+
+struct Kept {
+    cudaMemPool_t pool = nullptr;
+    std::vector<cudaStream_t> streams;
+};
+std::mutex g_kept_mu;
+
+// The current context's entry (NULL if there is no context). Caller holds the lock.
+Kept *kept_locked() {
+    static std::unordered_map<unsigned long long, Kept> *kept =
+        new std::unordered_map<unsigned long long, Kept>();  // (calls may outlive static teardown)
+    unsigned long long ctx = 0;
+    return current_context_id(&ctx) == NQ_OK ? &(*kept)[ctx] : nullptr;
+}
+
+// The library's memory pool on the current device.
+int memory_pool(cudaMemPool_t *out) {
+    std::lock_guard<std::mutex> g(g_kept_mu);
+    Kept *k = kept_locked();
+    if (!k) return NQ_ECUDA;
+    if (!k->pool) {
+        int dev = 0;
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        if (cudaGetDevice(&dev) != cudaSuccess) return NQ_ECUDA;
+        props.location.id = dev;
+        if (cudaMemPoolCreate(&k->pool, &props) != cudaSuccess) {
+            k->pool = nullptr;
+            return NQ_ENOMEM;
+        }
+        uint64_t keep = kPoolKeep;
+        cudaMemPoolSetAttribute(k->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    *out = k->pool;
+    return NQ_OK;
+}
+
+int pool_alloc(void **out, size_t bytes, cudaStream_t s) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess ||
+        capture != cudaStreamCaptureStatusNone)  // (the graph owns its allocation)
+        return cudaMallocAsync(out, bytes, s) == cudaSuccess ? NQ_OK : NQ_ENOMEM;
+    cudaMemPool_t pool = nullptr;
+    const int rc = memory_pool(&pool);
+    if (rc) return rc;
+    return cudaMallocFromPoolAsync(out, bytes, pool, s) == cudaSuccess ? NQ_OK : NQ_ENOMEM;
+}
+
 // Owns a non-blocking stream and the stream-ordered device allocations of one
 // synchronous call.
 struct CallCtx {
     cudaStream_t s = nullptr;
     std::vector<void *> bufs;
     ~CallCtx() {
-        if (s) {
-            for (void *b : bufs) cudaFreeAsync(b, s);
-            cudaStreamSynchronize(s);
-            cudaStreamDestroy(s);
+        if (!s) return;
+        for (void *b : bufs) cudaFreeAsync(b, s);
+        if (cudaStreamSynchronize(s) == cudaSuccess) {
+            std::lock_guard<std::mutex> g(g_kept_mu);
+            Kept *k = kept_locked();
+            if (k && k->streams.size() < kStreamsKept) {
+                k->streams.push_back(s);
+                return;
+            }
         }
+        cudaStreamDestroy(s);
     }
-    int init() { return cuda_rc(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)); }
+    int init() {
+        {
+            std::lock_guard<std::mutex> g(g_kept_mu);
+            Kept *k = kept_locked();
+            if (k && !k->streams.empty()) {
+                s = k->streams.back();
+                k->streams.pop_back();
+                return NQ_OK;
+            }
+        }
+        return cuda_rc(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    }
     template <typename T>
     int alloc(T **out, size_t bytes) {
         void *p = nullptr;
-        if (cudaMallocAsync(&p, bytes ? bytes : 16, s) != cudaSuccess) return NQ_ENOMEM;
+        if (const int rc = pool_alloc(&p, bytes ? bytes : 16, s)) return rc;
         bufs.push_back(p);
         *out = static_cast<T *>(p);
         return NQ_OK;
@@ -171,8 +247,7 @@ int enqueue_search(const nq_prefix *d_prefixes, uint64_t n, int expect_n, int mi
     const size_t bytes = donate ? head_bytes + kDonateCap * sizeof(DonateItem) : 64;
     const bool own = donate || (!cursor_ext && (!p.look || p.cursor));
     unsigned char *scratch = nullptr;
-    if (own && cudaMallocAsync(reinterpret_cast<void **>(&scratch), bytes, s) != cudaSuccess)
-        return NQ_ENOMEM;
+    if (own && (rc = pool_alloc(reinterpret_cast<void **>(&scratch), bytes, s))) return rc;
     unsigned long long *cursor =  // (NULL: the launch needs none)
         own ? reinterpret_cast<unsigned long long *>(scratch) : cursor_ext;
     if (own) rc = cuda_rc(cudaMemsetAsync(scratch, 0, donate ? bytes : 64, s));
@@ -274,22 +349,24 @@ namespace {
 // 0.064, 0.091 ms from 2, 3, 4, 5 rows; N = 17: 3.45, 3.58, 3.26, 3.15 ms).
 constexpr int kTotalRows = 4;
 
-int total_split(int N, int d, const nq_config *cfg, uint64_t *total_out, nq_timing *timing) {
-    const auto t_start = Clock::now();
-    const int b = std::min(d, kTotalRows);
-    uint64_t n = 0;
-    int rc = nq_enumerate_prefixes(N, b, nullptr, 0, &n);
-    if (rc) return rc;
-    // one block: [0] work cursor, [1] status, [2..33] totals, then the records
-    constexpr size_t kHead = 34 * sizeof(uint64_t);
-    static_assert(kHead % sizeof(nq_prefix) == 0, "the records are 16-byte aligned");
+// The records behind a block's head, and the head itself: [0] work cursor, [1]
+// status, [2..33] totals. One copy takes both to the device and one brings the
+// head back.
+constexpr size_t kHead = 34 * sizeof(uint64_t);
+static_assert(kHead % sizeof(nq_prefix) == 0, "the records are 16-byte aligned");
+nq_prefix *staged_records(unsigned char *stage) {
+    return reinterpret_cast<nq_prefix *>(stage + kHead);
+}
+
+// Count the n records staged behind `stage` (pinned), every one an N x N board
+// with at least d rows placed (allowed: under row masks), and their weighted
+// total. beside(): host work done while the search runs.
+template <typename F>
+int search_staged(int N, int d, unsigned char *stage, uint64_t n, const nq_config *cfg,
+                  const uint32_t *allowed, uint64_t *total_out, nq_timing *timing, F beside) {
     const size_t bytes = kHead + n * sizeof(nq_prefix);
-    unsigned char *stage = static_cast<unsigned char *>(t_stage.get(bytes));
-    if (!stage) return NQ_ENOMEM;
     std::memset(stage, 0, kHead);
-    if (n && (rc = nq_enumerate_prefixes(N, b, reinterpret_cast<nq_prefix *>(stage + kHead), n, &n)))
-        return rc;
-    const double enum_ms = ms_since(t_start);
+    int rc;
     CallCtx ctx;
     if ((rc = ctx.init())) return rc;
     unsigned char *dev = nullptr;
@@ -302,34 +379,50 @@ int total_split(int N, int d, const nq_config *cfg, uint64_t *total_out, nq_timi
     if (timing) cudaEventRecord(ev.e[1], ctx.s);
     Plan p{};
     if (!rc)
-        rc = enqueue_search(reinterpret_cast<nq_prefix *>(dev + kHead), n, N, b, N, nullptr, nullptr,
-                            d_head + 2, cfg, nullptr, ctx.s, &p, reinterpret_cast<int *>(d_head + 1),
-                            0, reinterpret_cast<unsigned long long *>(d_head));
+        rc = enqueue_search(staged_records(dev), n, N, d, N, nullptr, nullptr, d_head + 2, cfg,
+                            allowed, ctx.s, &p, reinterpret_cast<int *>(d_head + 1), 0,
+                            reinterpret_cast<unsigned long long *>(d_head));
     if (timing) cudaEventRecord(ev.e[2], ctx.s);
-    // (the staging block's head takes the results: its records are on the device
-    // before the copy back runs)
-    if (!rc)
-        rc = cuda_rc(cudaMemcpyAsync(stage, dev, kHead, cudaMemcpyDeviceToHost, ctx.s));
-    uint64_t prefixes = n;
-    if (!rc && timing && d > b) rc = nq_enumerate_prefixes(N, d, nullptr, 0, &prefixes);
+    if (!rc) rc = cuda_rc(cudaMemcpyAsync(stage, dev, kHead, cudaMemcpyDeviceToHost, ctx.s));
+    const int brc = rc ? NQ_OK : beside();
     if (cudaStreamSynchronize(ctx.s) != cudaSuccess) return NQ_ECUDA;
-    if (rc) return rc;
+    if (rc || brc) return rc ? rc : brc;
     const auto *head = reinterpret_cast<const uint64_t *>(stage);
-    const int st = *reinterpret_cast<const int *>(head + 1);
-    if (st) return st;
+    if (const int st = *reinterpret_cast<const int *>(head + 1)) return st;
     *total_out = head[2 + N];
     if (timing) {
         float up = 0, kern = 0;
         cudaEventElapsedTime(&up, ev.e[0], ev.e[1]);
         cudaEventElapsedTime(&kern, ev.e[1], ev.e[2]);
-        timing->enumerate_ms = enum_ms;
         timing->upload_ms = up;
         timing->kernel_ms = kern;
-        timing->prefixes = prefixes;
-        timing->d = d;
         timing->layout = p.layout;
         timing->block = p.block;
         timing->grid = p.grid;
+    }
+    return NQ_OK;
+}
+
+int total_split(int N, int d, const nq_config *cfg, uint64_t *total_out, nq_timing *timing) {
+    const auto t_start = Clock::now();
+    const int b = std::min(d, kTotalRows);
+    uint64_t n = 0;
+    int rc = nq_enumerate_prefixes(N, b, nullptr, 0, &n);
+    if (rc) return rc;
+    unsigned char *stage =
+        static_cast<unsigned char *>(t_stage.get(kHead + n * sizeof(nq_prefix)));
+    if (!stage) return NQ_ENOMEM;
+    if (n && (rc = nq_enumerate_prefixes(N, b, staged_records(stage), n, &n))) return rc;
+    const double enum_ms = ms_since(t_start);
+    uint64_t prefixes = n;
+    rc = search_staged(N, b, stage, n, cfg, nullptr, total_out, timing, [&]() -> int {
+        return timing && d > b ? nq_enumerate_prefixes(N, d, nullptr, 0, &prefixes) : NQ_OK;
+    });
+    if (rc) return rc;
+    if (timing) {
+        timing->enumerate_ms = enum_ms;
+        timing->prefixes = prefixes;
+        timing->d = d;
         timing->total_ms = ms_since(t_start);
     }
     return NQ_OK;
@@ -727,28 +820,8 @@ extern "C" int nq_count_constrained(int N, const nq_queen *q, int k, uint64_t *c
         }
     // The whole board as one record; the launch splits it (plan_records).
     const nq_prefix root{0, 0, 0, NQ_META(1, N, 0, 0)};
-    CallCtx ctx;
-    int rc = ctx.init();
-    if (rc) return rc;
-    nq_prefix *d_pre = nullptr;
-    uint64_t *d_tot = nullptr;
-    if ((rc = ctx.alloc(&d_pre, sizeof(nq_prefix)))) return rc;
-    if ((rc = ctx.alloc(&d_tot, 32 * sizeof(uint64_t) + 16))) return rc;
-    int *d_status = reinterpret_cast<int *>(d_tot + 32);
-    rc = cuda_rc(
-        cudaMemcpyAsync(d_pre, &root, sizeof(root), cudaMemcpyHostToDevice, ctx.s));
-    if (!rc) rc = cuda_rc(cudaMemsetAsync(d_tot, 0, 32 * sizeof(uint64_t) + 16, ctx.s));
-    if (!rc)
-        rc = enqueue_search(d_pre, 1, N, 0, N, nullptr, nullptr, d_tot, nullptr, allowed, ctx.s,
-                            nullptr, d_status);
-    uint64_t tot = 0;
-    if (!rc)
-        rc = cuda_rc(cudaMemcpyAsync(&tot, d_tot + N, sizeof(uint64_t), cudaMemcpyDeviceToHost,
-                                     ctx.s));
-    if (cudaStreamSynchronize(ctx.s) != cudaSuccess) return NQ_ECUDA;
-    if (rc) return rc;
-    const int st = take_status(d_status, ctx.s);
-    if (st) return st;
-    *count_out = tot;
-    return NQ_OK;
+    unsigned char *stage = static_cast<unsigned char *>(t_stage.get(kHead + sizeof(root)));
+    if (!stage) return NQ_ENOMEM;
+    *staged_records(stage) = root;
+    return search_staged(N, 0, stage, 1, nullptr, allowed, count_out, nullptr, [] { return NQ_OK; });
 }

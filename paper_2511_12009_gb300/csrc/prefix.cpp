@@ -202,9 +202,12 @@ class Pool {
     unsigned active_ = 0, gen_ = 0;
 };
 
-// Run fn(i) for i in [0, n) on the host's cores, pulling indices dynamically.
+// Run fn(i) for i in [0, n) on the host's cores, pulling indices dynamically;
+// on the calling thread alone where the whole work, n x `each` visits, is less
+// than waking the others costs (about 150 us).
+constexpr double kSerialVisits = 20000.0;
 template <typename F>
-void parallel_for(size_t n, F fn) {
+void parallel_for(size_t n, F fn, double each = 1e9) {
     std::atomic<size_t> next{0};
     const std::function<void()> work = [&]() {
         for (;;) {
@@ -213,7 +216,7 @@ void parallel_for(size_t n, F fn) {
             fn(i);
         }
     };
-    if (n <= 64) {
+    if (n <= 64 || (double)n * each <= kSerialVisits) {
         work();
         return;
     }
@@ -242,6 +245,13 @@ extern "C" int nq_default_depth(int N) {
 
 namespace nqi {
 
+// Nodes that a walk `rows` rows below a node of an N x N board visits, at most.
+static double visits_below(int N, int rows) {
+    double v = 1.0;
+    for (int j = 0; j < rows; ++j) v *= N;
+    return v;
+}
+
 // The set is split at depth t = min(3, d): every depth-t node counts the
 // prefixes below it (in parallel), and then writes its own contiguous slice.
 // The slices follow the nodes' canonical order, so the result is the same
@@ -257,7 +267,7 @@ int cut_prefixes(int N, int d, PrefixCut *cut) {
     parallel_for(cut->nodes.size(), [&](size_t i) {
         const Node &v = cut->nodes[i];
         cut->first[i + 1] = count_below(N, d, cut->t, v.cols, v.ld, v.rd, v.col0);
-    });
+    }, visits_below(N, d - 1 - cut->t));
     for (size_t i = 0; i < cut->nodes.size(); ++i) cut->first[i + 1] += cut->first[i];
     return NQ_OK;
 }
@@ -272,7 +282,7 @@ void write_prefix_nodes(const PrefixCut &cut, size_t lo, size_t hi, nq_prefix *o
         const Node &v = cut.nodes[i];
         Walker w{cut.n, cut.d, mask_n(cut.n), true, 0, out + cut.first[i], cap - cut.first[i], 0};
         w.rec(cut.t, v.cols, v.ld, v.rd, v.col0);
-    });
+    }, visits_below(cut.n, cut.d - cut.t));
 }
 
 }  // namespace nqi

@@ -43,6 +43,7 @@
 #include <cstdio>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <unordered_map>
 #include <utility>
 
@@ -1403,16 +1404,93 @@ int slots_needed(int layout, int max_n, int min_d) {
     return s < 1 ? 1 : s;
 }
 
+namespace {
+
+// What planning asks the runtime, kept per device context (a reset or a new
+// context has another id): some dozen queries, about 10 us, on every call
+// otherwise. One entry per device, and per kernel, block size asked for and
+// stack footprint -- a few hundred at most.
+int device_shape(unsigned long long ctx, int *sms, int *max_smem) {
+    static std::mutex mu;
+    static std::unordered_map<unsigned long long, std::pair<int, int>> shapes;
+    std::lock_guard<std::mutex> g(mu);
+    auto it = shapes.find(ctx);
+    if (it == shapes.end()) {
+        int dev = 0, n = 0, m = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&m, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+                cudaSuccess)
+            return NQ_ECUDA;
+        it = shapes.emplace(ctx, std::make_pair(n, m)).first;
+    }
+    *sms = it->second.first;
+    *max_smem = it->second.second;
+    return NQ_OK;
+}
+
+// Blocks of kernel k that fit an SM, for *block threads or (any_block) the size
+// of 256..128 that keeps the most threads resident under this stack footprint
+// (ties: the larger block): a frame more per thread can cost a whole block per
+// SM at 256 threads and none at 192 or 224. Raises the kernel's dynamic
+// shared-memory limit, one attribute per kernel, to what the launch needs, and
+// never lowers it: plans made earlier may still be launched.
+int resident_blocks(unsigned long long ctx, void *k, bool any_block, size_t per_thread,
+                    size_t extra, int max_smem, int *block, int *blocks) {
+    static std::mutex mu;
+    static std::map<std::tuple<unsigned long long, void *, int, size_t, size_t>,
+                    std::pair<int, int>> known;
+    const auto key = std::make_tuple(ctx, k, any_block ? -*block : *block, per_thread, extra);
+    std::lock_guard<std::mutex> g(mu);
+    const auto it = known.find(key);
+    if (it != known.end()) {
+        *block = it->second.first;
+        *blocks = it->second.second;
+        return NQ_OK;
+    }
+    int best = *block;
+    if (any_block) {
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) !=
+            cudaSuccess)
+            return NQ_ECUDA;
+        int best_threads = 0;
+        for (int b : {256, 224, 192, 160, 128}) {
+            const size_t sm = (size_t)b * per_thread + extra;
+            if (sm > (size_t)max_smem) continue;
+            int nb = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, b, sm) != cudaSuccess)
+                return NQ_ECUDA;
+            if (nb * b > best_threads) {
+                best = b;
+                best_threads = nb * b;
+            }
+        }
+    }
+    const size_t smem = (size_t)best * per_thread + extra;
+    cudaFuncAttributes fa{};
+    if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return NQ_ECUDA;
+    if (fa.maxDynamicSharedSizeBytes < (int)smem &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess)
+        return NQ_ECUDA;
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, best, smem) != cudaSuccess)
+        return NQ_ECUDA;
+    known.emplace(key, std::make_pair(best, nb));
+    *block = best;
+    *blocks = nb;
+    return NQ_OK;
+}
+
+}  // namespace
+
 int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config *cfg,
               Plan *plan, bool donate, bool stream, int levels) {
     if (max_n < 1 || max_n > NQ_MAX_N || min_d < 0 || min_d > max_n) return NQ_EINVAL;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return NQ_ECUDA;
+    unsigned long long ctx = 0;
+    if (const int rc = current_context_id(&ctx)) return rc;
     int sms = 0, max_smem = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-            cudaSuccess)
-        return NQ_ECUDA;
+    if (const int rc = device_shape(ctx, &sms, &max_smem)) return rc;
     Plan p{};
     p.layout = (cfg && cfg->layout) ? cfg->layout : NQ_LAYOUT_DEFAULT_SEARCH;
     if (p.layout < NQ_LAYOUT_PAPER || p.layout > NQ_LAYOUT_LAST) return NQ_EINVAL;
@@ -1438,41 +1516,11 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
     p.stream = stream && !p.donate && !constrained && layout_register_top(p.layout);
     if (stream && (!p.stream || p.look)) return NQ_EINVAL;
     void *k = pick_kernel(p.layout, diag, constrained, p.donate, p.stream, p.levels > 0);
-    if (!(cfg && cfg->block) && !layout_split_words(p.layout)) {
-        // No block size asked for: the one that keeps the most threads resident
-        // per SM under this stack footprint (ties: the larger block). A frame
-        // more per thread (deeper boards, REGP) can cost a whole block per SM
-        // at 256 threads and none at 192 or 224.
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) !=
-            cudaSuccess)
-            return NQ_ECUDA;
-        int best = 0, best_threads = 0;
-        for (int b : {256, 224, 192, 160, 128}) {
-            const size_t sm = (size_t)b * per_thread + extra;
-            if (sm > (size_t)max_smem) continue;
-            int nb = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, b, sm) != cudaSuccess)
-                return NQ_ECUDA;
-            if (nb * b > best_threads) {
-                best = b;
-                best_threads = nb * b;
-            }
-        }
-        if (best) p.block = best;
-    }
-    p.smem = (size_t)p.block * per_thread + extra;
-    // The kernel's dynamic shared-memory limit is one attribute per kernel, and
-    // plans made earlier (a batch's per-board plans, other callers) may still
-    // be launched: raise it when this plan needs more, never lower it.
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return NQ_ECUDA;
-    if (fa.maxDynamicSharedSizeBytes < (int)p.smem &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) !=
-            cudaSuccess)
-        return NQ_ECUDA;
+    const bool any_block = !(cfg && cfg->block) && !layout_split_words(p.layout);
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, p.block, p.smem) != cudaSuccess)
-        return NQ_ECUDA;
+    if (const int rc = resident_blocks(ctx, k, any_block, per_thread, extra, max_smem, &p.block, &nb))
+        return rc;
+    p.smem = (size_t)p.block * per_thread + extra;
     if (nb < 1) return NQ_ESTACK;
     if (cfg && cfg->blocks_per_sm > 0 && cfg->blocks_per_sm < nb) nb = cfg->blocks_per_sm;
     p.sms = sms;

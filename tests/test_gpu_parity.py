@@ -509,3 +509,37 @@ def test_constrained_whole_board_split(orc, n, k):
         g = synth_inputs.SplitMix64(7000 + 32 * n + k)
         qs = [(r, cols[r]) for r in synth_inputs.sample_ranks(g.next_u64(), n, k)]
         assert nq.count_constrained(n, qs) == orc.count_constrained(n, qs)[0], qs
+
+
+def test_synchronous_calls_from_many_threads(orc):
+    """Synchronous calls share the library's streams, memory pool and planned launch
+    shapes: twelve threads, each with its own boards, queries and stream, all exact."""
+    import threading
+    pre = nq.enumerate_prefixes(13, 4)
+    want = run(pre, 4, 13, "reg")[0]
+    q = orc.count_constrained(11, [(2, 3)])[0]
+    errors = []
+
+    def work(i):
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                dp = nq.to_device(pre)
+                cnt = torch.zeros(len(pre), dtype=torch.int64, device="cuda")
+                for k in range(6):
+                    n = 5 + (i + 3 * k) % 10
+                    assert nq.total(n) == Q[n]
+                    assert nq.count_constrained(11, [(2, 3)]) == q
+                    nq.count(13, 4, dp, cnt, stream=s)
+                    nq.sync(s)
+                    assert np.array_equal(u64(cnt), want)
+                    cnt.zero_()
+        except Exception as e:  # noqa: BLE001 (reported by the main thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(12)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
