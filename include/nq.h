@@ -339,8 +339,10 @@ typedef struct nq_server nq_server;
 typedef struct nq_server_config {
     int32_t max_n;          /* largest board accepted (<= 26; 0: 20) */
     int32_t request_slots;  /* requests in flight at once (<= 256; 0: 64) */
-    int32_t stack_slots;    /* stack frames per lane (0: 13). Admission by footprint: a
-                               request's prefix depth d is raised until N-1-d frames fit */
+    int32_t stack_slots;    /* stack frames per lane (0: 13). Admission by footprint: the
+                               depth d that a request's searches start at (its prefix rows
+                               and the rows that the kernel splits below them) is raised
+                               until N-1-d frames fit */
     int32_t block;          /* threads per block (0: 256) */
     uint64_t ring_records;  /* subproblem ring capacity, a power of two >= 1024 (0: 2^25) */
     uint32_t idle_ms;       /* the kernel exits once every warp has had nothing to do for

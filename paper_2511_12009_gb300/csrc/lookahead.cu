@@ -106,13 +106,16 @@ __device__ __forceinline__ void look_step(uint32_t &c, uint32_t &L, uint32_t &R,
 // The same step under per-row masks (partial-board queries): the row rides in
 // bits 27..31 of c, already counted up for the child (c = columns | (row + 1)
 // << 27), so entering a child adds the next row where look_step moves a
-// register. The masks of the child's row and of the row after it come as one
-// 8-byte load whose address depends on the frame alone; rows at or below the
-// last have mask 0 after them, so a last-row child is counted and not entered.
+// register. The masks of the child's row and of the row after it are loaded from
+// a table whose address depends on the frame alone: 8 bytes a row holding both
+// (ROW = 8, one load), or 33 words (ROW = 4, two loads, half the table: the
+// server keeps one for each request). Rows at or below the last have mask 0
+// after them, so a last-row child is counted and not entered.
 // The last row is a compare of the row field, no population count.
 // Six queries of two queens at N = 16: 98 ms with the host enumerating the
 // subproblems on one core, 1.8 ms as one split record (of which 1.2 ms are the
 // six calls' own cost).
+template <uint32_t ROW>
 __device__ __forceinline__ void look_step_masked(uint32_t &c, uint32_t &L, uint32_t &R,
                                                  uint32_t &av, uint32_t &top,
                                                  const uint32_t stride, const uint32_t table,
@@ -120,10 +123,14 @@ __device__ __forceinline__ void look_step_masked(uint32_t &c, uint32_t &L, uint3
                                                  const uint32_t m1, const uint32_t m2,
                                                  const uint32_t mneg) {
     uint32_t A1, A2;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
-                 : "=r"(A1), "=r"(A2)
-                 : "r"(((c >> kRowShift) << 3) + table)
-                 : "memory");
+    const uint32_t at = (c >> kRowShift) * ROW + table;
+    if constexpr (ROW == 8u)
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(A1), "=r"(A2) : "r"(at) : "memory");
+    else
+        asm volatile("ld.shared.u32 %0, [%2];\n\tld.shared.u32 %1, [%2+4];"
+                     : "=&r"(A1), "=r"(A2)
+                     : "r"(at)
+                     : "memory");
     const uint32_t p = av & (av * mneg);
     const uint32_t ar = p * mneg + av;
     const uint32_t c2 = p * m1 + c;
@@ -170,19 +177,21 @@ __device__ __forceinline__ void look_step_masked(uint32_t &c, uint32_t &L, uint3
 //   returns  0: nothing here, 1: search from (c, l, r) with candidates av
 //            (l, r as they reach this row), 2: *found solutions and no search
 //   skip     units to the next one that may hold something
-// MASKED: row `row` takes only the columns of its mask (table: 8 bytes a row),
-// and the board ends after `rows` rows; c holds no pre-set columns.
-template <bool MASKED>
-__device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint32_t digits,
+// ROW > 0: row `row` takes only the columns of its mask (a table of ROW bytes a
+// row), and the board ends after `rows` rows; c holds no pre-set columns.
+template <uint32_t ROW>
+__device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint64_t digits,
                                           int shift, uint32_t &c, uint32_t &l, uint32_t &r,
                                           uint32_t &av, uint32_t &found, uint32_t &skip,
                                           const uint32_t table, uint32_t row, uint32_t rows) {
+    constexpr bool MASKED = ROW > 0u;
     skip = 1u;
     for (int j = 0; j < levels; ++j, digits >>= 4, ++row) {
-        const uint32_t bits = digits & 15u;
+        const uint32_t bits = (uint32_t)digits & 15u;
         const uint32_t here = s & ((1u << shift) - 1u);  // this level's digit and those below
         shift -= (int)bits;
-        if (MASKED ? row == rows : c == ~0u) {  // every row is placed: the solution belongs to the unit of zeros
+        if (MASKED ? row == rows : c == ~0u) {
+            // every row is placed: the solution belongs to the unit of zeros
             skip = (1u << (shift + (int)bits)) - here;
             found = here == 0u ? 1u : 0u;
             return 2;
@@ -190,7 +199,7 @@ __device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint32_t
         uint32_t x = ~(c | l | r);
         if (MASKED) {
             uint32_t mask;
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mask) : "r"(table + 8u * row) : "memory");
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mask) : "r"(table + ROW * row) : "memory");
             x &= mask;
         }
         for (uint32_t t = here >> shift; t && x; --t) x &= x - 1u;
@@ -347,7 +356,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                 } else if (SPLIT) {
                     uint32_t cc = MASKED ? P.x : P.x | ~last;
                     uint32_t ll = P.y, rr = P.z & last, a0 = 0, found = 0;
-                    const int got = split_unit<MASKED>(s, a.levels, a.digits, a.split_shift, cc,
+                    const int got = split_unit<MASKED ? 8u : 0u>(s, a.levels, a.digits, a.split_shift, cc,
                                                        ll, rr, a0, found, skip, table, d, n);
                     if (got == 2) finish(pi, found, w | (n << 2));
                     if (got == 1) {
@@ -436,7 +445,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
 #pragma unroll
         for (int j = 0; j < kLookSteps; ++j) {
             if constexpr (MASKED)
-                look_step_masked(c, L, R, av, top, stride, table, thr, s32, m1, m2, mneg);
+                look_step_masked<8u>(c, L, R, av, top, stride, table, thr, s32, m1, m2, mneg);
             else
                 look_step(c, L, R, av, top, stride, s32, m1, m2, mneg);
         }
@@ -461,6 +470,332 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// Served mode: one persistent launch that keeps taking work of newly admitted
+// requests from a device ring while earlier ones are still being searched
+// (continuous batching). A ring record is a prefix of a request; its tag names
+// the request's slot, which holds the row masks and how the record's subtree is
+// cut into units. A warp takes one record at a time and hands its units to its
+// lanes, whose idle ones first take frames of the warp's busy ones; the masks
+// are cached per block in shared memory and refreshed by generation number.
+//
+// A slot's `remaining` counts what is still held of the request: its records
+// not yet handed out in full, and every lane searching a part of it. Whoever
+// gives back the last publishes the slot's total to mapped host memory.
+//
+// Every wait is bounded: the claim retries a fixed number of times; a warp with
+// nothing to do polls the ring with back-off, counts itself idle after
+// idle_polls rounds, and the grid leaves together once every started warp is
+// idle (or after 64x that many rounds in any case), so the kernel always ends
+// by itself once the host stops feeding it.
+//
+// Records that the host enumerated down to 4 per lane took one core longer than
+// the search (a burst of 32 requests of N = 10..15: 123 ms, of which 2 ms were
+// search); now the host makes at most some records per warp.
+// ---------------------------------------------------------------------------
+constexpr int kServeRefill = 8;  // idle lanes for which a warp takes a new record
+
+__device__ __forceinline__ uint4 ld_cg4(const void *p) {
+    uint4 v;
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_cg1(const void *p) {
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts1(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u32 [%0], %1;" : : "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t lds1(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
+__global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(look_smem);
+    const uint32_t stride = stack_slot_offset(blockDim.x, 0u, 1u, 16u);
+    const uint32_t base = sbase + stack_slot_offset(blockDim.x, threadIdx.x, 0u, 16u);
+    const uint32_t tables = sbase + (uint32_t)a.slots * stride;      // nslots x 33 words
+    const uint32_t gens = tables + (uint32_t)a.nslots * kServeTable;  // nslots words
+    for (int i = threadIdx.x; i < a.nslots; i += blockDim.x) sts1(gens + 4u * i, 0xFFFFFFFFu);
+    for (int i = threadIdx.x; i < a.nslots * (int)(kServeTable / 4u); i += blockDim.x)
+        sts1(tables + 4u * i, 0u);
+    __syncthreads();
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const uint32_t m1 = a.mul[0], m2 = a.mul[1], mneg = a.mul[2];
+
+    uint32_t c = kSentMaskedC, L = 0u, R = 0u, av = kSentAv, top = base, bot = base;
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
+                 :
+                 : "r"(base), "r"(c), "r"(L), "r"(R), "r"(av)
+                 : "memory");
+    int cur_slot = -1;         // the request this lane searches a part of
+    uint32_t cur_w = 1;        // symmetry weight of its record
+    uint32_t table = tables, thr = 0;
+    uint64_t sol = 0;
+    // the record the warp hands out (the same in every lane)
+    uint32_t next = 0, rem = 0, rec_tab = tables;
+    uint4 P = make_uint4(0u, 0u, 0u, 0u);
+    int rec_slot = 0, levels = 0, shift = 0;
+    uint64_t digits = 0;
+    unsigned int idle_polls = 0;
+    bool counted = false;  // warp-uniform: this warp is in *idle_warps
+    if (lane == 0) atomicAdd(a.started_warps, 1u);
+    // Claim back-off (warp-uniform): after a claim that found the ring empty
+    // the warp skips its next `skip` claim rounds, doubling up to 64, so that
+    // lanes still searching are not held up by lookups that find nothing.
+    uint32_t backoff = 0, skip = 0;
+
+    auto give_back = [&](int slot, uint64_t s) {
+        ServeSlot &q = a.slot_info[slot];
+        if (s) atomicAdd(&q.total, (unsigned long long)s);
+        __threadfence();
+        if (atomicSub(&q.remaining, 1u) == 1u) {
+            __threadfence();
+            const unsigned long long tot = atomicAdd(&q.total, 0ull);
+            const unsigned long long seq =
+                *reinterpret_cast<const volatile unsigned long long *>(&q.seq);
+            a.done[slot].total = tot;
+            __threadfence_system();
+            a.done[slot].seq = seq;
+            __threadfence_system();
+        }
+    };
+
+    for (;;) {
+        const bool idle = top == bot;
+        if (idle) {
+            if (cur_slot >= 0) {
+                give_back(cur_slot, sol * cur_w);
+                cur_slot = -1;
+            }
+            bot = top = base;
+            c = kSentMaskedC;
+            L = R = 0u;
+            av = kSentAv;
+        }
+        bool need = idle;
+        unsigned need_mask = __ballot_sync(~0u, need);
+        bool stopping = false, may_claim = true;
+        if (need_mask == ~0u) {  // the mapped stop flag, read only by an all-idle warp
+            int st = 0;
+            if (lane == 0) st = a.ctl->stop;
+            stopping = __shfl_sync(~0u, st, 0) != 0;
+        } else if (skip) {
+            --skip;
+            may_claim = false;
+        }
+        if (__popc(need_mask) >= kServeRefill && rem == 0u && may_claim && !stopping) {
+            unsigned int cl = 0;  // the grid is leaving: claim nothing more
+            if (lane == 0)
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cl) : "l"(a.closing)
+                             : "memory");
+            stopping = __shfl_sync(~0u, cl, 0) != 0;
+        }
+        while (need_mask && !stopping) {
+            if (rem == 0u) {
+                if (!may_claim || __popc(need_mask) < kServeRefill) break;
+                unsigned long long at = 0;
+                int got = 0;
+                if (lane == 0) {
+                    unsigned long long h, cur;
+                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(h) : "l"(a.head)
+                                 : "memory");
+                    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(cur) : "l"(a.cursor)
+                                 : "memory");
+                    for (int t = 0; t < 64 && cur < h; ++t) {
+                        const unsigned long long old = atomicCAS(a.cursor, cur, cur + 1ull);
+                        if (old == cur) {
+                            at = cur;
+                            got = 1;
+                            break;
+                        }
+                        cur = old;
+                    }
+                    __threadfence();  // records published before head are visible
+                }
+                at = __shfl_sync(~0u, at, 0);
+                got = __shfl_sync(~0u, got, 0);
+                if (!got) {
+                    backoff = backoff ? (backoff < 64u ? 2u * backoff : 64u) : 1u;
+                    skip = backoff;
+                    break;
+                }
+                backoff = 0;
+                if (counted) {  // back to work: out of the idle count
+                    if (lane == 0) atomicSub(a.idle_warps, 1u);
+                    counted = false;
+                    idle_polls = 0;
+                }
+                P = ld_cg4(a.ring + (at & a.ring_mask));
+                const uint32_t n = (P.w >> 2) & 31u, d = (P.w >> 7) & 31u, w = P.w & 3u;
+                rec_slot = (int)(P.w >> 12);
+                const uint32_t last = (n >= 1u) ? (0xFFFFFFFFu >> (32u - n)) : 0u;
+                bool ok = rec_slot < a.nslots && n >= 1u && n <= (uint32_t)kMaxConstrainedN &&
+                          (w == 1u || w == 2u) && d <= n && (P.x & ~last) == 0u &&
+                          (uint32_t)__popc(P.x) == d;
+                if (ok) {
+                    const ServeSlot *q = a.slot_info + rec_slot;
+                    levels = (int)ld_cg1(&q->levels);
+                    shift = (int)ld_cg1(&q->split_shift);
+                    digits = (uint64_t)ld_cg1(&q->digits) |
+                             (uint64_t)ld_cg1(reinterpret_cast<const uint32_t *>(&q->digits) + 1) << 32;
+                    const int first = (int)d + levels - 1;  // row that a lane's search starts in
+                    // (stack: the sentinel and the ancestors of rows first..N-2)
+                    ok = levels >= 1 && shift >= 0 && shift < 31 &&
+                         (first + 1 >= (int)n || (int)n - first <= a.slots);
+                }
+                if (!ok) {
+                    if (lane == 0) {
+                        look_error(a.status, NQ_EINVAL);
+                        a.ctl->error = NQ_EINVAL;  // mapped: the next poll reports it
+                        if (rec_slot < a.nslots) give_back(rec_slot, 0);
+                    }
+                    __syncwarp();
+                    continue;
+                }
+                // the slot's masks, cached in this block's shared memory
+                rec_tab = tables + kServeTable * (uint32_t)rec_slot;
+                const uint32_t gen = ld_cg1(&a.slot_info[rec_slot].gen);
+                __threadfence_block();
+                if (__any_sync(~0u, lds1(gens + 4u * (uint32_t)rec_slot) != gen)) {
+                    sts1(rec_tab + 4u * lane, ld_cg1(&a.slot_info[rec_slot].allowed[lane]));
+                    __threadfence_block();
+                    __syncwarp();
+                    if (lane == 0) sts1(gens + 4u * (uint32_t)rec_slot, gen);
+                }
+                __syncwarp();
+                next = 0u;
+                rem = 1u << shift;
+            }
+            const uint32_t n = (P.w >> 2) & 31u, d = (P.w >> 7) & 31u, w = P.w & 3u;
+            const uint32_t last = 0xFFFFFFFFu >> (32u - n);
+            const uint32_t rank = __popc(need_mask & lt_mask);
+            uint32_t past = 1u;
+            bool started = false;
+            if (need && rank < rem) {
+                uint32_t cc = P.x, ll = P.y, rr = P.z & last, a0 = 0, found = 0;
+                const int got = split_unit<4u>(next + rank, levels, digits, shift, cc, ll, rr, a0,
+                                               found, past, rec_tab, d, n);
+                if (got == 2 && found)
+                    atomicAdd(&a.slot_info[rec_slot].total, (unsigned long long)found * w);
+                if (got == 1) {
+                    cur_slot = rec_slot;
+                    cur_w = w;
+                    sol = 0;
+                    table = rec_tab;
+                    thr = (n - 1u) << kRowShift;
+                    c = cc | ((d + (uint32_t)levels) << kRowShift);
+                    L = ll << 1;
+                    R = rr >> 1;
+                    av = a0;
+                    top = base + stride;
+                    need = false;
+                    started = true;
+                }
+            }
+            // the lanes that started hold the request too
+            const unsigned st = __ballot_sync(~0u, started);
+            if (st && lane == 0) atomicAdd(&a.slot_info[rec_slot].remaining, (unsigned)__popc(st));
+            const uint32_t asked = __popc(need_mask);
+            uint32_t taken = asked < rem ? asked : rem;
+            if (asked <= rem) {  // every asker had a unit: pass over empty ones
+                taken += __shfl_sync(~0u, past, 31 - __clz((int)need_mask)) - 1u;
+                taken = taken < rem ? taken : rem;
+            }
+            next += taken;
+            rem -= taken;
+            __threadfence();
+            __syncwarp();
+            if (rem == 0u && lane == 0) give_back(rec_slot, 0);  // the record is handed out
+            __syncwarp();
+            need_mask = __ballot_sync(~0u, need);
+        }
+        if (need_mask && need_mask != ~0u && rem == 0u) {
+            // idle lanes take the shallowest saved frames of busy ones (look_body)
+            const bool giver = !need && top > bot + stride;
+            const unsigned givers = __ballot_sync(~0u, giver);
+            if (givers) {
+                const uint32_t pairs = min(__popc(need_mask), __popc(givers));
+                const uint32_t rank = __popc((need ? need_mask : givers) & lt_mask);
+                const bool taker = need && rank < pairs;
+                const int from = taker ? (int)__fns(givers, 0, (int)rank + 1) : (int)lane;
+                const uint32_t at = __shfl_sync(~0u, bot + stride, from);
+                const int slot = __shfl_sync(~0u, cur_slot, from);
+                const uint32_t w = __shfl_sync(~0u, cur_w, from);
+                const uint32_t tab = __shfl_sync(~0u, table, from);
+                const uint32_t th = __shfl_sync(~0u, thr, from);
+                if (taker) {
+                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(c), "=r"(L), "=r"(R), "=r"(av)
+                                 : "r"(at)
+                                 : "memory");
+                    cur_slot = slot;
+                    cur_w = w;
+                    table = tab;
+                    thr = th;
+                    sol = 0;
+                    top = base + stride;
+                    atomicAdd(&a.slot_info[slot].remaining, 1u);
+                }
+                __threadfence();
+                __syncwarp();
+                if (giver && rank < pairs) {
+                    bot += stride;
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
+                                 :
+                                 : "r"(bot), "r"(kSentMaskedC), "r"(0u), "r"(0u), "r"(kSentAv)
+                                 : "memory");
+                }
+                __syncwarp();
+            }
+        }
+        if (need_mask == ~0u) {
+            // (plain stores to the mapped block: no atomics on host memory)
+            if (stopping) {
+                if (lane == 0) a.ctl->exit_reason = 1;
+                break;
+            }
+            ++idle_polls;
+            if (idle_polls > a.idle_polls && !counted) {
+                if (lane == 0) atomicAdd(a.idle_warps, 1u);
+                counted = true;
+            }
+            if (counted) {
+                int leave = 0;
+                if (lane == 0) {
+                    unsigned int iw, sw;
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(iw)
+                                 : "l"(a.idle_warps) : "memory");
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(sw)
+                                 : "l"(a.started_warps) : "memory");
+                    leave = iw >= sw || (unsigned long long)idle_polls > 64ull * a.idle_polls;
+                    if (leave) {
+                        atomicExch(a.closing, 1u);
+                        a.ctl->exit_reason = 2;
+                    }
+                }
+                if (__shfl_sync(~0u, leave, 0)) break;
+            }
+            __nanosleep(idle_polls < 64 ? 256u : 4096u);
+            continue;
+        }
+        idle_polls = 0;
+        uint32_t s32 = 0;
+#pragma unroll
+        for (int j = 0; j < kLookSteps; ++j)
+            look_step_masked<4u>(c, L, R, av, top, stride, table, thr, s32, m1, m2, mneg);
+        sol += s32;
+    }
+}
+
 __global__ void __maxnreg__(48) look_kernel(const SearchArgs a) { look_body<false, false>(a); }
 __global__ void __maxnreg__(48) look_kernel_split(const SearchArgs a) {
     look_body<true, false>(a);
@@ -476,5 +811,7 @@ void *look_kernel_ptr(bool split, bool masked) {
            : split ? reinterpret_cast<void *>(&look_kernel_split)
                    : reinterpret_cast<void *>(&look_kernel);
 }
+
+void *serve_kernel_ptr() { return reinterpret_cast<void *>(&serve_kernel); }
 
 }  // namespace nqi

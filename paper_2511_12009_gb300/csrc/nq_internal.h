@@ -75,7 +75,7 @@ struct SearchArgs {
     // to a record, level j's digit in the j-th nibble of `digits`, in bits
     int levels;
     int split_shift;
-    uint32_t digits;
+    uint64_t digits;
     int refill;         // idle lanes for which a warp takes a new range of units
 };
 // Bookkeeping rounds a lane may wait for an unpublished index (each round is
@@ -138,14 +138,22 @@ constexpr int kMaxConstrainedN = 26;
 // Served mode: a persistent kernel fed through a device ring.
 // ---------------------------------------------------------------------------
 
-// One request slot's parameters, written by the host before the request's
-// records are published; read by the kernel (bypassing L1) at claim time.
+// One request slot, written by the host before the request's records are
+// published; the parameters are read by the kernel (bypassing L1) as it takes a
+// record.
 struct ServeSlot {
     uint32_t allowed[32];  // columns each row may take (0 for rows >= N)
     uint32_t n;            // board size
     uint32_t gen;          // bumped on every reuse of the slot
     uint64_t seq;          // the request's ticket
+    // how its records are cut into units (as in SearchArgs; levels >= 1)
+    int32_t levels, split_shift;
+    uint64_t digits;
+    unsigned long long total;  // solutions so far
+    uint32_t remaining;        // records not handed out in full, and lanes at work on the request
+    uint32_t pad;
 };
+constexpr uint32_t kServeTable = 33u * 4u;  // bytes of a slot's masks in shared memory
 
 // Host-visible control block (mapped pinned memory).
 struct ServeControl {
@@ -169,9 +177,7 @@ struct ServeArgs {
     unsigned long long ring_mask;
     unsigned long long *cursor;      // next index to claim (device)
     ServeControl *ctl;               // mapped
-    const ServeSlot *slot_info;      // [nslots] (device)
-    unsigned long long *slot_total;  // [nslots] (device)
-    unsigned int *slot_remaining;    // [nslots] (device)
+    ServeSlot *slot_info;            // [nslots] (device)
     ServeDone *done;                 // [nslots] (mapped)
     int nslots;
     int slots;                       // stack slots per lane
@@ -196,6 +202,15 @@ struct ServeArgs {
 // subtrees split, or split and under row masks.
 void *look_kernel_ptr(bool split, bool masked);
 
+void *serve_kernel_ptr();  // (lookahead.cu)
+// How records with d rows placed of a board under row masks are cut into units:
+// n of them, searched by `lanes` lanes with room for `slots` frames (the sentinel
+// among them). NQ_ESTACK: they have to be made deeper first.
+int serve_cut(int N, int d, const uint32_t allowed[32], uint64_t n, double lanes, int slots,
+              ServeSlot *out);
+// Search steps below one such record, to a factor of two or three.
+double masked_steps(int N, int d, const uint32_t allowed[32]);
+
 int launch_serve(const ServeArgs &a, int grid, int block, size_t smem, cudaStream_t s);
 int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *smem,
                int *slots);
@@ -213,7 +228,8 @@ struct Plan {
     // layout REGP's production kernel (SearchArgs has the same names)
     bool look;
     int rows, levels, split_shift, refill;
-    uint32_t digits, range;
+    uint64_t digits;
+    uint32_t range;
     bool cursor;    // the launch takes more than every warp's first range
 };
 

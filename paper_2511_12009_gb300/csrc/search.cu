@@ -28,14 +28,9 @@
 //   - uint64 solution counts per subproblem; weighted totals reduced per warp
 //     with shuffles, one atomicAdd per warp and board size.
 //
-// The default layout REGP's production kernel, and the search under row masks
-// that nq_count_constrained makes, are in lookahead.cu; this file's REGP is its
-// diagnostic build.
-//
-// Served mode (partial-board queries; not in the paper): every row r has a mask allowed[r] of the columns it may take (one
-// column for a row with a given queen; the cells the given queens attack
-// removed elsewhere), the frame's row index rides in bits 27..31 of cols, and
-// the next-row mask is additionally ANDed with allowed[row].
+// The default layout REGP's production kernel, the search under row masks that
+// nq_count_constrained makes and the server's kernel are in lookahead.cu; this
+// file's REGP is its diagnostic build.
 #include <cuda.h>
 
 #include <algorithm>
@@ -60,20 +55,10 @@ __device__ int g_stream_status[kStatusWords];
 
 namespace {
 
-constexpr int kSplitMaxLevels = 8;  // of split work (plan_records); a nibble each
+constexpr int kSplitMaxLevels = 16;  // of split work (plan_records); a nibble each
 constexpr uint64_t kNone = ~0ull;
 constexpr int kChunk = 15;
 static_assert(kChunk < 16, "the sentinel frame holds 16 idle steps (32 for ~0 masks)");
-constexpr uint32_t kRowInc = 1u << kRowShift;
-// Constrained-mode sentinel: row field 30, so the child is row 31 whose allowed
-// mask is 0 -- no push, no count. Its 27 candidate bits lie below the row field
-// and in none of its masks (cols, ld and rd hold no column), so the sums of the
-// multiply-add form stay exact and cols never wraps: 27 idle steps per frame.
-constexpr uint32_t kSentinelC = 30u << kRowShift;
-constexpr uint32_t kSentinelLrC = 0u;
-constexpr uint32_t kSentinelAvC = kRowInc - 1u;
-static_assert(kChunk < kRowShift, "constrained sentinel holds 27 idle steps");
-
 extern __shared__ __align__(16) unsigned char nq_smem[];
 
 __device__ __forceinline__ void record_error(int *status, int code) {
@@ -172,8 +157,7 @@ struct Lane {
     uint32_t stride;   // bytes between a thread's consecutive frames
     uint32_t base;     // shared address of this thread's slot 0 (the sentinel)
     uint32_t limit;    // one past this thread's last slot
-    uint32_t table;    // WT32: bytes per array; constrained mode: address of allowed[]
-    uint32_t thr;      // constrained mode: (N-1) << 27, the last-row threshold
+    uint32_t table;    // WT32: bytes per array
     int *status;       // where this launch records its first error
 };
 
@@ -274,10 +258,6 @@ __device__ __forceinline__ void step_reg(uint32_t &c, uint32_t &l, uint32_t &r, 
     "setp.eq.u32 plast, %6, 31;\n\t"            /* queens in rows 0..N-2 (Algorithm 3) */ \
     "setp.ne.and.u32 pcnt, %7, 0, plast;\n\t"   /* ... and row N-1 has its column free */ \
     "setp.ne.and.u32 ppush, %7, 0, !plast;\n\t" /* a live child above the last row */
-#define NQ_PRED_ROWFIELD \
-    "setp.ge.u32 plast, %9, %6;\n\t"            /* the child is in row N-1 */ \
-    "setp.ne.and.u32 pcnt, %7, 0, plast;\n\t"   /* ... and takes a free, allowed column */ \
-    "setp.ne.and.u32 ppush, %7, 0, !plast;\n\t" /* a live child above the last row */
 #define NQ_PRED_PUSHLAST \
     "setp.eq.u32 pcnt, %9, 0xFFFFFFFF;\n\t"     /* every column holds a queen */ \
     "setp.ne.u32 ppush, %7, 0;\n\t"             /* a live child */
@@ -325,39 +305,12 @@ __device__ __forceinline__ void step_regm(uint32_t &c, uint32_t &l, uint32_t &r,
 #undef NQ_OPERANDS
 }
 
-// One constrained step in the multiply-add form (partial-board queries: the
-// server's kernel and nq_count_constrained): the row index rides in bits
-// 27..31 of cols and is advanced with the placement, the child's row takes
-// only its allowed columns (a shared-memory table of 32 masks at `table`,
-// read at the start of the step: its address depends only on the parent's
-// row), and the child is in the last row when its row field reaches thr =
-// (N-1) << 27 -- one compare where the unconstrained step counts bits.
-// Operand %6 is thr; the rest as in step_regm.
-__device__ __forceinline__ void step_regm_constr(uint32_t &c, uint32_t &l, uint32_t &r,
-                                                 uint32_t &av, uint32_t &top,
-                                                 const uint32_t stride, const uint32_t table,
-                                                 const uint32_t thr, uint32_t &s32,
-                                                 const uint32_t m1, const uint32_t m2,
-                                                 const uint32_t mneg, const uint32_t mhalf) {
-    const uint32_t allowed = lds1(table + ((c >> kRowShift) << 2) + 4u);
-    const uint32_t p = av & (av * mneg);
-    const uint32_t ar = p * mneg + av;
-    const uint32_t c2 = p * m1 + c + kRowInc;
-    const uint32_t l2 = l * m2 + p * m2;
-    const uint32_t r2 = __umulhi(p * m1 + r, mhalf);
-    const uint32_t a2 = ~(c2 | l2 | r2) & allowed;
-    asm volatile(NQ_TAIL(NQ_PRED_ROWFIELD, NQ_SAVE4, NQ_LOAD4)
-                 : "+r"(c), "+r"(l), "+r"(r), "+r"(av), "+r"(top), "+r"(s32)
-                 : "r"(thr), "r"(a2), "r"(ar), "r"(c2), "r"(l2), "r"(r2), "r"(stride)
-                 : "memory");
-}
 #undef NQ_SAVE4
 #undef NQ_LOAD4
 #undef NQ_SAVEZ
 #undef NQ_LOADZ
 #undef NQ_PRED_LASTROW
 #undef NQ_PRED_PUSHLAST
-#undef NQ_PRED_ROWFIELD
 #undef NQ_TAIL
 
 // One step, layout AVAIL (the avail-only stack): one 32-bit word per level,
@@ -1081,241 +1034,6 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
     }
 }
 
-// ---------------------------------------------------------------------------
-// Served mode: one persistent launch that keeps taking subproblems of newly
-// admitted requests from a device ring while earlier ones are still being
-// searched (continuous batching). Each record's tag names its request slot;
-// the slot's allowed-column masks are cached per block in shared memory and
-// refreshed by generation number. The lane that finishes a slot's last
-// subproblem publishes the slot's total to mapped host memory. Every wait is
-// bounded: the claim retries a fixed number of times; a warp with nothing to
-// do polls the ring with back-off, counts itself idle after idle_polls rounds,
-// and the grid leaves together once every started warp is idle (or after 64x
-// that many rounds in any case), so the kernel always ends by itself once the
-// host stops feeding it.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint4 ld_cg4(const void *p) {
-    uint4 v;
-    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p)
-                 : "memory");
-    return v;
-}
-__device__ __forceinline__ uint32_t ld_cg1(const void *p) {
-    uint32_t v;
-    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
-    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(nq_smem);
-    Lane k;
-    k.stride = stack_slot_offset(blockDim.x, 0u, 1u, stack_elem_bytes(false));
-    k.base = sbase + stack_slot_offset(blockDim.x, threadIdx.x, 0u, stack_elem_bytes(false));
-    k.limit = k.base + (uint32_t)a.slots * k.stride;
-    const uint32_t tables = sbase + (uint32_t)a.slots * k.stride;   // nslots x 128 B
-    const uint32_t gens = tables + (uint32_t)a.nslots * 128u;        // nslots x 4 B
-    k.table = tables;
-    k.thr = 0;
-    k.status = a.status;
-    for (int i = threadIdx.x; i < a.nslots; i += blockDim.x) sts1(gens + 4u * i, 0xFFFFFFFFu);
-    for (int i = threadIdx.x; i < a.nslots * 32; i += blockDim.x) sts1(tables + 4u * i, 0u);
-    __syncthreads();
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned lt_mask = (1u << lane) - 1u;
-
-    // two sentinel frames (slots 0 and 1): an idle lane runs whole rounds on them
-    uint32_t c = kSentinelC, l = kSentinelLrC, r = kSentinelLrC, av = kSentinelAvC;
-    uint32_t top = k.base + k.stride;
-    sts4(k.base, make_uint4(kSentinelC, kSentinelLrC, kSentinelLrC, kSentinelAvC));
-    sts4(k.base + k.stride, make_uint4(kSentinelC, kSentinelLrC, kSentinelLrC, kSentinelAvC));
-    int cur_slot = -1;
-    uint32_t cur_w = 1;  // symmetry weight of the record being searched
-    uint64_t sol = 0;
-    unsigned int idle_polls = 0;
-    bool counted = false;  // warp-uniform: this warp is in *idle_warps
-    if (lane == 0) atomicAdd(a.started_warps, 1u);
-    // Claim back-off (warp-uniform): after a claim that found the ring empty
-    // the warp skips its next `skip` claim rounds, doubling up to 64, so that
-    // lanes still searching are not held up by lookups that find nothing.
-    uint32_t backoff = 0, skip = 0;
-
-    auto finish_slot = [&](int slot, uint64_t s) {
-        if (s) atomicAdd(&a.slot_total[slot], (unsigned long long)s);
-        __threadfence();
-        if (atomicSub(&a.slot_remaining[slot], 1u) == 1u) {
-            __threadfence();
-            const unsigned long long tot = atomicAdd(&a.slot_total[slot], 0ull);
-            const unsigned long long seq = *reinterpret_cast<const volatile unsigned long long *>(
-                &a.slot_info[slot].seq);
-            a.done[slot].total = tot;
-            __threadfence_system();
-            a.done[slot].seq = seq;
-            __threadfence_system();
-        }
-    };
-
-    for (;;) {
-        const bool idle = top <= k.base + k.stride;
-        if (idle) {
-            if (cur_slot >= 0) {
-                finish_slot(cur_slot, sol * cur_w);
-                cur_slot = -1;
-            }
-            c = kSentinelC;
-            l = r = kSentinelLrC;
-            av = kSentinelAvC;
-            top = k.base + k.stride;
-        }
-        bool need = idle;
-        unsigned need_mask = __ballot_sync(~0u, need);
-        bool stopping = false;
-        if (need_mask == ~0u) {  // the mapped stop flag, read only by an all-idle warp
-            int st = 0;
-            if (lane == 0) st = a.ctl->stop;
-            stopping = __shfl_sync(~0u, st, 0) != 0;
-        }
-        if (skip && need_mask != ~0u) {
-            --skip;
-            need_mask = 0;
-        }
-        if (need_mask && !stopping) {  // the grid is leaving: claim nothing more
-            unsigned int cl = 0;
-            if (lane == 0)
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cl) : "l"(a.closing)
-                             : "memory");
-            stopping = __shfl_sync(~0u, cl, 0) != 0;
-        }
-        while (need_mask && !stopping) {
-            const int leader = __ffs(need_mask) - 1;
-            unsigned long long first = 0, got = 0;
-            if ((int)lane == leader) {
-                unsigned long long h, cur;
-                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(h) : "l"(a.head)
-                             : "memory");
-                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(cur) : "l"(a.cursor)
-                             : "memory");
-                for (int t = 0; t < 64 && cur < h; ++t) {
-                    const unsigned long long want =
-                        h - cur < (unsigned long long)__popc(need_mask) ? h - cur
-                                                                       : (unsigned long long)__popc(need_mask);
-                    const unsigned long long old = atomicCAS(a.cursor, cur, cur + want);
-                    if (old == cur) {
-                        first = cur;
-                        got = want;
-                        break;
-                    }
-                    cur = old;
-                }
-                __threadfence();  // records published before head are visible
-            }
-            first = __shfl_sync(~0u, first, leader);
-            got = __shfl_sync(~0u, got, leader);
-            if (got == 0) {
-                backoff = backoff ? (backoff < 64u ? 2u * backoff : 64u) : 1u;
-                skip = backoff;
-                break;
-            }
-            backoff = 0;
-            if (counted) {  // back to work: out of the idle count
-                if (lane == 0) atomicSub(a.idle_warps, 1u);
-                counted = false;
-                idle_polls = 0;
-            }
-            const unsigned rank = __popc(need_mask & lt_mask);
-            if (need && rank < got) {
-                const unsigned long long idx = first + rank;
-                const uint4 P = ld_cg4(a.ring + (idx & a.ring_mask));
-                const uint32_t n = (P.w >> 2) & 31u, d = (P.w >> 7) & 31u, w = P.w & 3u;
-                const int slot = (int)(P.w >> 12);
-                const uint32_t last = (n >= 1u) ? (0xFFFFFFFFu >> (32u - n)) : 0u;
-                // (stack: two sentinels + the ancestors of rows d..N-3)
-                const bool ok = slot < a.nslots && n >= 1u && n <= (uint32_t)kMaxConstrainedN &&
-                                (w == 1u || w == 2u) &&
-                                d <= n && (P.x & ~last) == 0u && (uint32_t)__popc(P.x) == d &&
-                                (d + 1u >= n || (int)n - (int)d <= a.slots);
-                if (!ok) {
-                    record_error(k.status, NQ_EINVAL);
-                    a.ctl->error = NQ_EINVAL;  // mapped: the next poll reports it
-                    if (slot < a.nslots) finish_slot(slot, 0);
-                } else {
-                    // the slot's allowed masks, cached in this block's shared memory
-                    const uint32_t gen = ld_cg1(&a.slot_info[slot].gen);
-                    const uint32_t tab = tables + 128u * (uint32_t)slot;
-                    __threadfence_block();
-                    if (lds1(gens + 4u * slot) != gen) {
-                        for (int w = 0; w < 32; ++w)
-                            sts1(tab + 4u * w, ld_cg1(&a.slot_info[slot].allowed[w]));
-                        __threadfence_block();
-                        sts1(gens + 4u * slot, gen);
-                    }
-                    const uint32_t l0 = P.y;
-                    const uint32_t r0 = P.z & last;
-                    const uint32_t c0 = P.x | (d << kRowShift);
-                    const uint32_t a0 = ~(c0 | l0 | r0) & lds1(tab + (d << 2)) & last;
-                    if (d == n) {
-                        finish_slot(slot, w);
-                    } else if (d + 1u == n || a0 == 0u) {
-                        finish_slot(slot, (uint64_t)__popc(a0) * w);
-                    } else {
-                        cur_slot = slot;
-                        cur_w = w;
-                        sol = 0;
-                        k.table = tab;
-                        k.thr = (n - 1u) << kRowShift;
-                        c = c0; l = l0; r = r0; av = a0;
-                        top = k.base + 2u * k.stride;  // above the two sentinels
-                        need = false;
-                    }
-                }
-            }
-            const unsigned asked = __popc(need_mask);
-            need_mask = __ballot_sync(~0u, need);
-            if (got < asked) break;  // the ring is drained for now
-        }
-        if (__all_sync(~0u, top <= k.base + k.stride && cur_slot < 0)) {
-            // (plain stores to the mapped block: no atomics on host memory)
-            if (stopping) {
-                if (lane == 0) a.ctl->exit_reason = 1;
-                break;
-            }
-            ++idle_polls;
-            if (idle_polls > a.idle_polls && !counted) {
-                if (lane == 0) atomicAdd(a.idle_warps, 1u);
-                counted = true;
-            }
-            if (counted) {
-                int leave = 0;
-                if (lane == 0) {
-                    unsigned int iw, sw;
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(iw)
-                                 : "l"(a.idle_warps) : "memory");
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(sw)
-                                 : "l"(a.started_warps) : "memory");
-                    leave = iw >= sw || (unsigned long long)idle_polls > 64ull * a.idle_polls;
-                    if (leave) {
-                        atomicExch(a.closing, 1u);
-                        a.ctl->exit_reason = 2;
-                    }
-                }
-                if (__shfl_sync(~0u, leave, 0)) break;
-            }
-            __nanosleep(idle_polls < 64 ? 256u : 4096u);
-            continue;
-        }
-        idle_polls = 0;
-        uint32_t s32 = 0;
-        const uint32_t m1 = a.mul[0], m2 = a.mul[1], mneg = a.mul[2], mhalf = a.mul[3];
-        // two 27-step sentinels: 31 steps between bookkeeping points
-#pragma unroll
-        for (int j = 0; j < 31; ++j)
-            step_regm_constr(c, l, r, av, top, k.stride, k.table, k.thr, s32, m1, m2, mneg,
-                             mhalf);
-        sol += s32;
-    }
-}
-
 // The production kernel is held to 48 registers (5 resident blocks of 256 at
 // N=18, d=7); the donating variant carries the queue logic and gets 64.
 template <int LAYOUT, bool DIAG>
@@ -1543,9 +1261,22 @@ double subtree_steps(int n, int rows) {
 // How the records' subtrees are cut into units.
 struct Cut {
     int levels = 0, shift = 0;  // rows that the units fix, bits of a unit's index
-    uint32_t digits = 0;        // bits of each level's digit, a nibble each
+    uint64_t digits = 0;        // bits of each level's digit, a nibble each
     double live = 0.0;          // units that hold something, about
 };
+
+// The most columns that each row below a record could have free; returns the
+// size of the free board that the record's searches like: a given queen takes
+// its row and column out.
+int row_caps(int N, int d, const uint32_t *allowed, int *cap) {
+    int board = N;
+    for (int j = 0; j < N - d; ++j) {
+        cap[j] = N - d - j;
+        if (allowed) cap[j] = std::min(cap[j], __builtin_popcount(allowed[d + j]));
+        if (cap[j] <= 1 && j + 1 < N - d && board > 1) --board;
+    }
+    return board;
+}
 
 // cap[j]: the most columns that row j below a record could have free (rows
 // with one are passed through), for `rows` rows; the records lie on boards
@@ -1559,7 +1290,7 @@ struct Cut {
 // 5: 20.3, 18.4, 38.9 ms), a missing one much (2048 records of N = 22, d = 7:
 // 1 level 44 ms, 3 levels 5.5 ms, 4 levels 4.5 ms, 5 levels 6.5 ms, none
 // 326 ms).
-Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, bool at_least_one) {
+Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, int min_levels) {
     int open_rows[NQ_MAX_N + 2] = {};  // rows j.. with a choice
     for (int j = rows - 1; j >= 0; --j) open_rows[j] = open_rows[j + 1] + (cap[j] > 1 ? 1 : 0);
     Cut cut;
@@ -1569,10 +1300,10 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, bo
     while (cut.levels < rows) {
         const bool few = live < lanes / 4.0 && unit > 150.0;
         const bool uneven = unit > std::max(750.0, share / 8.0);
-        if (!few && !uneven && (cut.levels || !at_least_one)) break;
+        if (!few && !uneven && cut.levels >= min_levels) break;
         Cut c;
         c.levels = cut.levels + 1;
-        while (c.levels < rows && cap[c.levels - 1] <= 1) ++c.levels;
+        while (c.levels < rows && c.levels < kSplitMaxLevels && cap[c.levels - 1] <= 1) ++c.levels;
         if (c.levels > kSplitMaxLevels) break;
         double lv = (double)n, un = 0.0;
         for (int j = 0; j < c.levels; ++j) {
@@ -1584,7 +1315,7 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, bo
             if (last) b = std::min(b, 2);
             const double open = std::max(1.0, 0.6 * cap[j]);  // columns free, about
             const double taken = last ? std::min(open, (double)(1 << b)) : open;
-            c.digits |= (uint32_t)b << (4 * j);
+            c.digits |= (uint64_t)b << (4 * j);
             c.shift += b;
             lv *= taken;
             if (last) un = subtree_steps(board, open_rows[j]) / taken;
@@ -1599,6 +1330,28 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, bo
 
 }  // namespace
 
+double masked_steps(int N, int d, const uint32_t allowed[32]) {
+    int cap[NQ_MAX_N + 1] = {}, left = 0;
+    const int board = row_caps(N, d, allowed, cap);
+    for (int j = 0; j < N - d; ++j) left += cap[j] > 1 ? 1 : 0;
+    return subtree_steps(board, left);
+}
+
+int serve_cut(int N, int d, const uint32_t allowed[32], uint64_t n, double lanes, int slots,
+              ServeSlot *out) {
+    int cap[NQ_MAX_N + 1] = {};
+    const int rows = N - d, board = row_caps(N, d, allowed, cap);
+    // a lane's search starts in row d + levels - 1 and needs N less that frames
+    const int need = rows >= 2 ? std::max(1, rows + 1 - slots) : 1;
+    Cut cut = choose_cut(cap, rows, board, n, lanes, need);
+    if (cut.levels < 1 && rows <= 1) cut.levels = 1;  // a solved board or its last row
+    if (cut.levels < need || cut.levels < 1) return NQ_ESTACK;
+    out->levels = cut.levels;
+    out->split_shift = cut.shift;
+    out->digits = cut.digits;
+    return NQ_OK;
+}
+
 int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t n, bool may_split,
                  Plan *plan, const uint32_t *allowed) {
     if (!plan->look) return NQ_OK;
@@ -1607,18 +1360,12 @@ int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t
     const double lanes = (double)p.grid * p.block;
     Cut cut;
     if (may_split && !p.stream && n) {
-        int cap[NQ_MAX_N + 1] = {}, board = max_n;
-        for (int j = 0; j < p.rows; ++j) {
-            cap[j] = p.rows - j;
-            if (allowed) {
-                cap[j] = std::min(cap[j], __builtin_popcount(allowed[min_d + j]));
-                if (cap[j] <= 1 && board > 1) --board;  // a given queen takes its row and column
-            }
-        }
-        cut = choose_cut(cap, p.rows, board, n, lanes, allowed != nullptr);
+        int cap[NQ_MAX_N + 1] = {};
+        const int board = row_caps(max_n, min_d, allowed, cap);
+        cut = choose_cut(cap, p.rows, board, n, lanes, allowed ? 1 : 0);
     }
     const int levels = cut.levels, shift = cut.shift;
-    const uint32_t digits = cut.digits;
+    const uint64_t digits = cut.digits;
     if (levels) {
         const int rc =
             make_plan(max_n, min_d, diag, allowed != nullptr, cfg, &p, false, false, levels);
@@ -1681,10 +1428,10 @@ int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *s
         cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
             cudaSuccess)
         return NQ_ECUDA;
-    const int sl = slots_needed(NQ_LAYOUT_REGM, max_n, min_d);  // two sentinels
-    const size_t bytes = (size_t)sl * 16u * block + (size_t)nslots * 132u;
+    const int sl = std::max(1, max_n - 1 - min_d) + 1;  // a sentinel, and frames down to row N-2
+    const size_t bytes = (size_t)sl * 16u * block + (size_t)nslots * (kServeTable + 4u);
     if (bytes > (size_t)max_smem) return NQ_ESTACK;
-    void *k = reinterpret_cast<void *>(&serve_kernel);
+    void *k = serve_kernel_ptr();
     cudaFuncAttributes fa{};  // (raise only: another server may still relaunch with its size)
     if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return NQ_ECUDA;
     if (fa.maxDynamicSharedSizeBytes < (int)bytes &&
@@ -1704,7 +1451,7 @@ int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *s
 int launch_serve(const ServeArgs &a, int grid, int block, size_t smem, cudaStream_t s) {
     ServeArgs args = a;
     void *params[] = {&args};
-    const cudaError_t e = cudaLaunchKernel(reinterpret_cast<void *>(&serve_kernel), dim3(grid),
+    const cudaError_t e = cudaLaunchKernel(serve_kernel_ptr(), dim3(grid),
                                            dim3(block), params, smem, s);
     return e == cudaSuccess ? NQ_OK : NQ_ECUDA;
 }

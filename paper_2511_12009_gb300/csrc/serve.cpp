@@ -14,10 +14,13 @@
 // so every record below that end has been read -- a later request that
 // completes early does not move it, since a lane may still hold a claimed but
 // unread index of an earlier one), and its stack footprint
-// fits the running kernel's (its prefix depth is raised until N - 1 - d frames
-// fit, and further while it has fewer than four subproblems per resident lane).
+// fits the running kernel's: a record's subtree is cut into units on the device,
+// and its prefix rows and the cut are raised until N - 1 - d frames fit below
+// them (serve_cut). The host makes records until there are eight for every warp
+// that the kernel has resident, or until a record holds little work.
 #include <algorithm>
 #include <atomic>
+#include <cstring>
 #include <deque>
 #include <mutex>
 #include <new>
@@ -39,6 +42,13 @@ constexpr size_t kHeadWord = 16;
 constexpr size_t kExitBytes = 256;
 constexpr size_t kStatusByte = 640;
 
+// Pinned staging of a submission: its slot and, if they fit, its records.
+constexpr uint64_t kStageRecords = 1ull << 16;
+constexpr size_t kStageHead = (sizeof(ServeSlot) + 15) / 16 * 16;
+constexpr size_t kStageBytes = kStageHead + kStageRecords * sizeof(nq_prefix);
+// Search steps below which a record is not worth cutting further on the host.
+constexpr double kRecordSteps = 8000.0;
+
 struct nq_server {
     nq_server_config cfg{};
     int dev = 0;
@@ -51,8 +61,7 @@ struct nq_server {
     nq_prefix *d_ring = nullptr;
     unsigned long long *d_cursor = nullptr;
     ServeSlot *d_slot = nullptr;
-    unsigned long long *d_total = nullptr;
-    unsigned int *d_remaining = nullptr;
+    void *h_stage = nullptr;  // pinned: the slot, then up to kStageRecords records
     ServeControl *h_ctl = nullptr, *d_ctl = nullptr;
     ServeDone *h_done = nullptr, *d_done = nullptr;
     uint64_t head = 0;       // records published
@@ -82,8 +91,7 @@ void release(nq_server *s) {
     if (s->d_ring) cudaFree(s->d_ring);
     if (s->d_cursor) cudaFree(s->d_cursor);
     if (s->d_slot) cudaFree(s->d_slot);
-    if (s->d_total) cudaFree(s->d_total);
-    if (s->d_remaining) cudaFree(s->d_remaining);
+    if (s->h_stage) cudaFreeHost(s->h_stage);
     if (s->h_ctl) cudaFreeHost(s->h_ctl);
     if (s->h_done) cudaFreeHost(s->h_done);
     if (s->kdone) cudaEventDestroy(s->kdone);
@@ -116,8 +124,6 @@ int ensure_running(nq_server *s) {
     a.status = s->status();
     a.ctl = s->d_ctl;
     a.slot_info = s->d_slot;
-    a.slot_total = s->d_total;
-    a.slot_remaining = s->d_remaining;
     a.done = s->d_done;
     a.nslots = s->cfg.request_slots;
     a.slots = s->stack_slots;
@@ -192,10 +198,7 @@ extern "C" int nq_server_create(const nq_server_config *cfg, nq_server **out) {
     if (!rc && (cudaMalloc(&s->d_ring, s->ring * sizeof(nq_prefix)) != cudaSuccess ||
                 cudaMalloc(&s->d_cursor, kCtlBytes) != cudaSuccess ||
                 cudaMalloc(&s->d_slot, c.request_slots * sizeof(ServeSlot)) != cudaSuccess ||
-                cudaMalloc(&s->d_total, c.request_slots * sizeof(unsigned long long)) !=
-                    cudaSuccess ||
-                cudaMalloc(&s->d_remaining, c.request_slots * sizeof(unsigned int)) !=
-                    cudaSuccess ||
+                cudaMallocHost(&s->h_stage, kStageBytes) != cudaSuccess ||
                 cudaHostAlloc(&s->h_ctl, sizeof(ServeControl), cudaHostAllocMapped) !=
                     cudaSuccess ||
                 cudaHostAlloc(&s->h_done, c.request_slots * sizeof(ServeDone),
@@ -250,14 +253,14 @@ extern "C" int nq_server_submit(nq_server *s, int N, const nq_queen *q, int k, u
             break;
         }
     if (slot < 0) return NQ_EBUSY;
-    // The request's depth: at least what fits the kernel's stack (N - 1 - d
-    // frames), then deeper while its subproblems are fewer than four per
-    // resident lane -- a few heavy subtrees would leave most lanes idle while
-    // they finish -- as long as the next depth's records take at most a
-    // quarter of the ring.
-    // (the kernel's stack holds two sentinel frames and N - 2 - d ancestors:
-    // N - d <= s->stack_slots)
-    int d = std::min(N, std::max(N - s->stack_slots, std::min(N - 2 < 0 ? 0 : N - 2, 5)));
+    bool none = false;  // a row that the given queens leave no column
+    for (int r = 0; r < N; ++r) none = none || !allowed[r];
+    // The request's depth: records for the warps to take, eight for each that is
+    // resident unless little work is left below one, and deep enough for the
+    // kernel's stack. (No queen given: at least the rows that the symmetric set's
+    // rules are about.)
+    int d = k == 0 ? std::min(N, 2) : 0;
+    ServeSlot info{};
     {
         auto count_at = [&](int dd) -> uint64_t {
             uint64_t np = 0;
@@ -267,17 +270,24 @@ extern "C" int nq_server_submit(nq_server *s, int N, const nq_queen *q, int k, u
             }
             return nqi::count_constrained_prefixes(N, dd, allowed);
         };
-        const uint64_t lanes = (uint64_t)s->grid * (uint64_t)s->block;
-        uint64_t cnt = count_at(d);
-        while (d + 1 <= N - 2 && cnt < 4 * lanes) {
+        const double lanes = (double)s->grid * (double)s->block;
+        uint64_t cnt = none ? 0 : count_at(d);
+        while (!none && d + 1 <= N - 2 && (double)cnt < lanes / 4.0 &&
+               nqi::masked_steps(N, d, allowed) > kRecordSteps) {
             const uint64_t next = count_at(d + 1);
             if (next > s->ring / 4) break;
             ++d;
             cnt = next;
         }
+        while (!none && nqi::serve_cut(N, d, allowed, cnt, lanes, s->stack_slots, &info)) {
+            if (d >= N) return NQ_ESTACK;
+            cnt = count_at(++d);
+        }
     }
     std::vector<nq_prefix> pre;
-    if (k == 0) {
+    if (none) {
+        // (no record)
+    } else if (k == 0) {
         // no queen given: the symmetric prefix set of Section 1 (weights 1 or 2)
         uint64_t np = 0;
         int erc = nq_enumerate_prefixes(N, d, nullptr, 0, &np);
@@ -299,26 +309,29 @@ extern "C" int nq_server_submit(nq_server *s, int N, const nq_queen *q, int k, u
     }
     if (m > s->ring) return NQ_EOVERFLOW;
     if (s->head + m - s->consumed > s->ring) return NQ_EBUSY;
-    // slot parameters, its counters, then the records (possibly wrapping)
-    ServeSlot info{};
+    // the slot with its counters, then the records (possibly wrapping)
     for (int r = 0; r < 32; ++r) info.allowed[r] = allowed[r];
     info.n = (uint32_t)N;
     info.gen = ++s->gen[slot];
     info.seq = tk;
-    const unsigned long long zero = 0;
-    const unsigned int rem = (unsigned int)m;
-    bool ok = cudaMemcpyAsync(&s->d_slot[slot], &info, sizeof(info), cudaMemcpyHostToDevice,
+    info.remaining = (uint32_t)m;  // one hold for each record
+    info.total = 0;
+    // (the copies of the submission before have ended: it waited for them)
+    unsigned char *stage = static_cast<unsigned char *>(s->h_stage);
+    std::memcpy(stage, &info, sizeof(info));
+    const nq_prefix *rec = pre.data();
+    if (m <= kStageRecords) {
+        std::memcpy(stage + kStageHead, rec, m * sizeof(nq_prefix));
+        rec = reinterpret_cast<const nq_prefix *>(stage + kStageHead);
+    }
+    bool ok = cudaMemcpyAsync(&s->d_slot[slot], stage, sizeof(info), cudaMemcpyHostToDevice,
                               s->cstream) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(&s->d_total[slot], &zero, sizeof(zero), cudaMemcpyHostToDevice,
-                               s->cstream) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(&s->d_remaining[slot], &rem, sizeof(rem), cudaMemcpyHostToDevice,
-                               s->cstream) == cudaSuccess;
     const uint64_t pos = s->head & s->mask;
     const uint64_t first_part = std::min(m, s->ring - pos);
-    ok = ok && cudaMemcpyAsync(s->d_ring + pos, pre.data(), first_part * sizeof(nq_prefix),
+    ok = ok && cudaMemcpyAsync(s->d_ring + pos, rec, first_part * sizeof(nq_prefix),
                                cudaMemcpyHostToDevice, s->cstream) == cudaSuccess;
     if (first_part < m)
-        ok = ok && cudaMemcpyAsync(s->d_ring, pre.data() + first_part,
+        ok = ok && cudaMemcpyAsync(s->d_ring, rec + first_part,
                                    (m - first_part) * sizeof(nq_prefix), cudaMemcpyHostToDevice,
                                    s->cstream) == cudaSuccess;
     // publish: the head's device mirror is copied in after the records, on the

@@ -150,3 +150,24 @@ def test_board_symmetry_served(seed):
     vals = {got[t] for t in tickets}
     assert len(vals) == 1
     assert vals.pop() == nq.count_constrained(n, qs)
+
+
+def test_served_split_edges(orc):
+    """Boards that end within the split levels, rows fixed from the top (more than
+    a level each), full solutions, the widest board, and a small stack that forces
+    deep prefixes, all in one burst; every answer equals the standalone count, and
+    a second burst on the same slots (new generations) too."""
+    from paper_2511_12009_gb300.serve import Server, run_stream
+    sol26 = [c - 1 for c in list(range(2, 27, 2)) + [3, 1, 7, 9, 11, 13, 15, 17, 19, 21, 23, 25, 5]]
+    reqs = [(1, []), (2, []), (3, []), (4, []), (5, [(0, 0)]), (6, []), (8, [(7, 3)]),
+            (26, [(r, sol26[r]) for r in range(26)]), (26, [(r, sol26[r]) for r in range(15)]),
+            (26, [(25 - r, sol26[r]) for r in range(16)]),
+            (13, []), (14, [(6, 6)]), (15, [(0, 7), (14, 2)])]
+    stream = [{"t": 0.0, "n": n, "queens": q} for n, q in reqs]
+    want = [Q[n] if not q else nq.count_constrained(n, q) for n, q in reqs]
+    for slots in (13, 9):
+        with Server(max_n=26, stack_slots=slots, request_slots=8, idle_ms=50) as srv:
+            for _ in range(2):
+                res = run_stream(srv, stream, timeout_s=120)
+                assert [res["answers"][i] for i in range(len(reqs))] == want
+            assert srv.poll() == []
