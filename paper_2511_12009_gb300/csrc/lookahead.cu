@@ -478,6 +478,9 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
 // cut into units. A warp takes one record at a time and hands its units to its
 // lanes, whose idle ones first take frames of the warp's busy ones; the masks
 // are cached per block in shared memory and refreshed by generation number.
+// Records come from the ring to a block in batches, by compare-and-swap on the
+// cursor (which must not pass the published head); one by one for each warp, the
+// 3,648 warps of the grid got a record every 0.7 us between them.
 //
 // A slot's `remaining` counts what is still held of the request: its records
 // not yet handed out in full, and every lane searching a part of it. Whoever
@@ -523,6 +526,13 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
     const uint32_t base = sbase + stack_slot_offset(blockDim.x, threadIdx.x, 0u, 16u);
     const uint32_t tables = sbase + (uint32_t)a.slots * stride;      // nslots x 33 words
     const uint32_t gens = tables + (uint32_t)a.nslots * kServeTable;  // nslots words
+    // the block's batch of ring records: [first, end), taken under `lock`
+    __shared__ unsigned long long batch_first, batch_end;
+    __shared__ int batch_lock;
+    if (threadIdx.x == 0) {
+        batch_first = batch_end = 0ull;
+        batch_lock = 0;
+    }
     for (int i = threadIdx.x; i < a.nslots; i += blockDim.x) sts1(gens + 4u * i, 0xFFFFFFFFu);
     for (int i = threadIdx.x; i < a.nslots * (int)(kServeTable / 4u); i += blockDim.x)
         sts1(tables + 4u * i, 0u);
@@ -584,6 +594,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
         bool need = idle;
         unsigned need_mask = __ballot_sync(~0u, need);
         bool stopping = false, may_claim = true;
+        int closing = 0;
         if (need_mask == ~0u) {  // the mapped stop flag, read only by an all-idle warp
             int st = 0;
             if (lane == 0) st = a.ctl->stop;
@@ -593,39 +604,61 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
             may_claim = false;
         }
         if (__popc(need_mask) >= kServeRefill && rem == 0u && may_claim && !stopping) {
-            unsigned int cl = 0;  // the grid is leaving: claim nothing more
+            unsigned int cl = 0;  // the grid is leaving: nothing more from the ring
             if (lane == 0)
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cl) : "l"(a.closing)
                              : "memory");
-            stopping = __shfl_sync(~0u, cl, 0) != 0;
+            closing = (int)__shfl_sync(~0u, cl, 0);
         }
         while (need_mask && !stopping) {
             if (rem == 0u) {
                 if (!may_claim || __popc(need_mask) < kServeRefill) break;
                 unsigned long long at = 0;
-                int got = 0;
+                int got = 0;  // 1: record `at`, 0: there is none, -1: another warp is looking
                 if (lane == 0) {
-                    unsigned long long h, cur;
-                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(h) : "l"(a.head)
-                                 : "memory");
-                    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(cur) : "l"(a.cursor)
-                                 : "memory");
-                    for (int t = 0; t < 64 && cur < h; ++t) {
-                        const unsigned long long old = atomicCAS(a.cursor, cur, cur + 1ull);
-                        if (old == cur) {
-                            at = cur;
-                            got = 1;
-                            break;
+                    got = -1;
+                    if (atomicCAS(&batch_lock, 0, 1) == 0) {
+                        got = 0;
+                        __threadfence_block();
+                        volatile unsigned long long *first = &batch_first, *end = &batch_end;
+                        unsigned long long f = *first, e = *end;
+                        if (f == e && !closing) {
+                            unsigned long long h, cur;
+                            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(h)
+                                         : "l"(a.head) : "memory");
+                            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(cur)
+                                         : "l"(a.cursor) : "memory");
+                            for (int t = 0; t < 32 && cur < h; ++t) {
+                                unsigned long long g = (h - cur) / (2ull * gridDim.x);
+                                g = g < 1ull ? 1ull : g > 64ull ? 64ull : g;
+                                const unsigned long long old = atomicCAS(a.cursor, cur, cur + g);
+                                if (old == cur) {
+                                    f = cur;
+                                    e = cur + g;
+                                    break;
+                                }
+                                cur = old;
+                            }
+                            __threadfence();  // records published before head are visible
                         }
-                        cur = old;
+                        if (f != e) {
+                            at = f++;
+                            got = 1;
+                        }
+                        *first = f;
+                        *end = e;
+                        __threadfence_block();
+                        atomicExch(&batch_lock, 0);
                     }
-                    __threadfence();  // records published before head are visible
                 }
                 at = __shfl_sync(~0u, at, 0);
                 got = __shfl_sync(~0u, got, 0);
-                if (!got) {
-                    backoff = backoff ? (backoff < 64u ? 2u * backoff : 64u) : 1u;
-                    skip = backoff;
+                if (got <= 0) {
+                    if (got == 0) {
+                        backoff = backoff ? (backoff < 64u ? 2u * backoff : 64u) : 1u;
+                        skip = backoff;
+                        stopping = closing != 0;  // (the block's batch is used up as well)
+                    }
                     break;
                 }
                 backoff = 0;
