@@ -1283,9 +1283,11 @@ int row_caps(int N, int d, const uint32_t *allowed, int *cap) {
 // that search like a free board of size `board`.
 //
 // Split while there is less than a unit for every fourth lane and a unit is not
-// small in itself (setting one up costs some ten steps), or while a unit is
-// more than an eighth of a lane's share of the work (the largest are a few
-// times the mean). A level more or less where the line lies costs little
+// small in itself (setting one up costs some ten steps, less on the first level:
+// 148 records of N = 10, d = 3 take 13.3 us unsplit and 11.3 us with one level;
+// 110 of N = 13, d = 2 27 us down to 80 steps and 40 us down to 50), or while a
+// unit is more than an eighth of a lane's share of the work (the largest are a
+// few times the mean). A level more or less where the line lies costs little
 // (N = 16, d = 5: 1 level 0.60 ms, 2 levels 0.56 ms, none 1.25 ms; N = 18, d =
 // 5: 20.3, 18.4, 38.9 ms), a missing one much (2048 records of N = 22, d = 7:
 // 1 level 44 ms, 3 levels 5.5 ms, 4 levels 4.5 ms, 5 levels 6.5 ms, none
@@ -1298,7 +1300,7 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, in
     double live = (double)n;                              // units that hold something
     double unit = subtree_steps(board, open_rows[0]);     // steps below one
     while (cut.levels < rows) {
-        const bool few = live < lanes / 4.0 && unit > 150.0;
+        const bool few = live < lanes / 4.0 && unit > (cut.levels ? 80.0 : 20.0);
         const bool uneven = unit > std::max(750.0, share / 8.0);
         if (!few && !uneven && cut.levels >= min_levels) break;
         Cut c;
