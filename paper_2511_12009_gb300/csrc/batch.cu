@@ -29,9 +29,12 @@ struct nq_batch {
     bool has_cfg = false;
     nq_prefix *d_pre = nullptr;
     uint64_t *d_counts = nullptr;
-    uint64_t *d_totals = nullptr;
-    unsigned long long *d_cursor = nullptr;  // [0] work cursor; status word at byte 8
-    uint64_t *h_totals = nullptr;  // pinned, 32 entries
+    // [0] work cursor, [1] status word, then the 32 totals: one block, zeroed by
+    // one memset and read back by one copy into h_head (pinned)
+    unsigned long long *d_head = nullptr;
+    uint64_t *h_head = nullptr;
+    cudaEvent_t ev[2] = {};  // around a run
+    uint64_t *d_totals() const { return reinterpret_cast<uint64_t *>(d_head + 2); }
     nqi::Plan plan{};
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -45,9 +48,10 @@ void release(nq_batch *b) {
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->d_pre) cudaFree(b->d_pre);
     if (b->d_counts) cudaFree(b->d_counts);
-    if (b->d_totals) cudaFree(b->d_totals);
-    if (b->d_cursor) cudaFree(b->d_cursor);
-    if (b->h_totals) cudaFreeHost(b->h_totals);
+    if (b->d_head) cudaFree(b->d_head);
+    if (b->h_head) cudaFreeHost(b->h_head);
+    for (cudaEvent_t e : b->ev)
+        if (e) cudaEventDestroy(e);
     delete b;
 }
 
@@ -57,8 +61,8 @@ nqi::SearchArgs args_for(const nq_batch *b, const nq_prefix *pre, uint64_t n, in
     a.pre = pre;
     a.n = n;
     a.counts = b->d_counts + (pre - b->d_pre);
-    a.totals = b->d_totals;
-    a.cursor = b->d_cursor;
+    a.totals = b->d_totals();
+    a.cursor = b->d_head;
     a.expect_n = expect_n;
     a.min_d = min_d;
     a.slots = slots;
@@ -68,13 +72,19 @@ nqi::SearchArgs args_for(const nq_batch *b, const nq_prefix *pre, uint64_t n, in
     a.mul[1] = 2u;
     a.mul[2] = 0xFFFFFFFFu;
     a.mul[3] = 0x80000000u;
-    a.status = reinterpret_cast<int *>(b->d_cursor + 1);
+    a.status = reinterpret_cast<int *>(b->d_head + 1);
     return a;
 }
 
-int fill_totals(const nq_batch *b, uint64_t *totals_out) {
-    if (!totals_out) return NQ_OK;
-    for (int i = 0; i < b->k; ++i) totals_out[i] = b->h_totals[b->ns[i]];
+constexpr size_t kHeadBytes = 34 * sizeof(uint64_t);
+
+// What a finished run left in h_head: its error, or its totals.
+int take_results(const nq_batch *b, float ms, uint64_t *totals_out, float *ms_out) {
+    const int st = *reinterpret_cast<const int *>(b->h_head + 1);
+    if (st) return st;
+    if (ms_out) *ms_out = ms;
+    if (totals_out)
+        for (int i = 0; i < b->k; ++i) totals_out[i] = b->h_head[2 + b->ns[i]];
     return NQ_OK;
 }
 
@@ -147,12 +157,17 @@ extern "C" int nq_batch_create(const int *ns, const int *ds, int k, const nq_con
     }
     if (cudaMalloc(&b->d_pre, (total ? total : 1) * sizeof(nq_prefix)) != cudaSuccess ||
         cudaMalloc(&b->d_counts, (total ? total : 1) * sizeof(uint64_t)) != cudaSuccess ||
-        cudaMalloc(&b->d_totals, 32 * sizeof(uint64_t)) != cudaSuccess ||
-        cudaMalloc(&b->d_cursor, 64) != cudaSuccess ||
-        cudaMallocHost(&b->h_totals, 32 * sizeof(uint64_t)) != cudaSuccess) {
+        cudaMalloc(&b->d_head, kHeadBytes) != cudaSuccess ||
+        cudaMallocHost(&b->h_head, kHeadBytes) != cudaSuccess) {
         release(b);
         return NQ_ENOMEM;
     }
+    for (cudaEvent_t &e : b->ev)
+        if (cudaEventCreate(&e) != cudaSuccess) {
+            e = nullptr;
+            release(b);
+            return NQ_ECUDA;
+        }
     if (total && cudaMemcpy(b->d_pre, host.data(), total * sizeof(nq_prefix),
                             cudaMemcpyHostToDevice) != cudaSuccess) {
         release(b);
@@ -172,13 +187,12 @@ extern "C" int nq_batch_create(const int *ns, const int *ds, int k, const nq_con
     }
     const nqi::SearchArgs a = args_for(b, b->d_pre, b->n, 0, b->min_d, b->plan.slots);
     bool ok = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    ok = ok && cudaMemsetAsync(b->d_cursor, 0, 16, s) == cudaSuccess;  // cursor and status
-    ok = ok && cudaMemsetAsync(b->d_totals, 0, 32 * sizeof(uint64_t), s) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(b->d_head, 0, kHeadBytes, s) == cudaSuccess;
     if (b->plan.levels)  // split work adds into the counts
         ok = ok && cudaMemsetAsync(b->d_counts, 0, total * sizeof(uint64_t), s) == cudaSuccess;
     ok = ok && nqi::launch_search(a, b->plan, false, false, s) == NQ_OK;
-    ok = ok && cudaMemcpyAsync(b->h_totals, b->d_totals, 32 * sizeof(uint64_t),
-                               cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(b->h_head, b->d_head, kHeadBytes, cudaMemcpyDeviceToHost, s) ==
+                   cudaSuccess;
     cudaGraph_t g = nullptr;
     const bool ended = cudaStreamEndCapture(s, &g) == cudaSuccess;
     cudaStreamDestroy(s);
@@ -210,25 +224,12 @@ extern "C" int nq_batch_info(const nq_batch *b, uint64_t *records, int *min_d, i
 extern "C" int nq_batch_run(nq_batch *b, void *stream, uint64_t *totals_out, float *ms_out) {
     if (!b) return NQ_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaEvent_t e0, e1;
-    if (cudaEventCreate(&e0) != cudaSuccess) return NQ_ECUDA;
-    if (cudaEventCreate(&e1) != cudaSuccess) {
-        cudaEventDestroy(e0);
+    if (cudaEventRecord(b->ev[0], s) != cudaSuccess || cudaGraphLaunch(b->exec, s) != cudaSuccess ||
+        cudaEventRecord(b->ev[1], s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
         return NQ_ECUDA;
-    }
-    int rc = NQ_OK;
-    if (cudaEventRecord(e0, s) != cudaSuccess || cudaGraphLaunch(b->exec, s) != cudaSuccess ||
-        cudaEventRecord(e1, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
-        rc = NQ_ECUDA;
     float ms = 0;
-    if (!rc) cudaEventElapsedTime(&ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (rc) return rc;
-    const int st = nqi::take_status(reinterpret_cast<int *>(b->d_cursor + 1), s);
-    if (st) return st;
-    if (ms_out) *ms_out = ms;
-    return fill_totals(b, totals_out);
+    cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]);
+    return take_results(b, ms, totals_out, ms_out);
 }
 
 extern "C" int nq_batch_run_separate(nq_batch *b, void *stream, uint64_t *totals_out,
@@ -245,20 +246,13 @@ extern "C" int nq_batch_run_separate(nq_batch *b, void *stream, uint64_t *totals
                                    b->first[j + 1] - b->first[j], true, &plans[j]);
         if (rc) return rc;
     }
-    cudaEvent_t e0, e1;
-    if (cudaEventCreate(&e0) != cudaSuccess) return NQ_ECUDA;
-    if (cudaEventCreate(&e1) != cudaSuccess) {
-        cudaEventDestroy(e0);
-        return NQ_ECUDA;
-    }
     int rc = NQ_OK;
-    if (cudaEventRecord(e0, s) != cudaSuccess ||
-        cudaMemsetAsync(b->d_totals, 0, 32 * sizeof(uint64_t), s) != cudaSuccess ||
-        cudaMemsetAsync(b->d_cursor + 1, 0, sizeof(int), s) != cudaSuccess)  // status
+    if (cudaEventRecord(b->ev[0], s) != cudaSuccess ||
+        cudaMemsetAsync(b->d_head, 0, kHeadBytes, s) != cudaSuccess)
         rc = NQ_ECUDA;
     for (int j = 0; j < b->k && !rc; ++j) {
         const uint64_t n = b->first[j + 1] - b->first[j];
-        if (cudaMemsetAsync(b->d_cursor, 0, sizeof(unsigned long long), s) != cudaSuccess) {
+        if (cudaMemsetAsync(b->d_head, 0, sizeof(unsigned long long), s) != cudaSuccess) {
             rc = NQ_ECUDA;
             break;
         }
@@ -271,20 +265,15 @@ extern "C" int nq_batch_run_separate(nq_batch *b, void *stream, uint64_t *totals
         }
         rc = nqi::launch_search(a, plans[j], false, false, s);
     }
-    if (!rc && (cudaMemcpyAsync(b->h_totals, b->d_totals, 32 * sizeof(uint64_t),
-                                cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                cudaEventRecord(e1, s) != cudaSuccess))
+    if (!rc && (cudaMemcpyAsync(b->h_head, b->d_head, kHeadBytes, cudaMemcpyDeviceToHost, s) !=
+                    cudaSuccess ||
+                cudaEventRecord(b->ev[1], s) != cudaSuccess))
         rc = NQ_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess && !rc) rc = NQ_ECUDA;
-    float ms = 0;
-    if (!rc) cudaEventElapsedTime(&ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     if (rc) return rc;
-    const int st = nqi::take_status(reinterpret_cast<int *>(b->d_cursor + 1), s);
-    if (st) return st;
-    if (ms_out) *ms_out = ms;
-    return fill_totals(b, totals_out);
+    float ms = 0;
+    cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]);
+    return take_results(b, ms, totals_out, ms_out);
 }
 
 extern "C" int nq_batch_counts(const nq_batch *b, int board, uint64_t *h_counts, uint64_t cap,
