@@ -60,7 +60,7 @@ N22_D7_NODES = 143257329200995
 # DRAM traffic of one production search launch on the default workload (N=18,
 # d=7, default layout), dram__bytes_read.sum + dram__bytes_write.sum from one
 # ncu capture, valid only for the kernel source it was taken on: the sha256 of
-# search.cu and nq_internal.h. Any change to them makes the figure stale, and
+# lookahead.cu and nq_internal.h. Any change to them makes the figure stale, and
 # the roofline then reports traffic as null.
 TRAFFIC_NCU = {"n": 18, "d": 7, "layout": "default", "bytes": 120265472 + 35418368,
                "kernel_sha256": "dfc692036a7ecf9edd96180d51319b24752b3dec0752c3273d9d70dbf7ecda7c"}
@@ -193,7 +193,7 @@ class ClockSampler:
 def kernel_sha256() -> str:
     import hashlib
     h = hashlib.sha256()
-    for name in ("search.cu", "nq_internal.h"):
+    for name in ("lookahead.cu", "nq_internal.h"):
         with open(os.path.join(ROOT, "paper_2511_12009_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
@@ -708,8 +708,13 @@ def main():
             if k:  # the first call warms the pinned staging buffer
                 e2e_times.append(dt)
         e2e_s = max_over_ranks(dist, float(np.mean(e2e_times)), device)
+        # The default form copies the first four rows' prefixes and a 272-byte head (which
+        # comes back); the others the whole depth-d set, and read one total.
+        splits = args.layout in ("default", "regp")
+        records = nq.prefix_count(n, min(d, 4)) if splits else m
         e2e = {"value": nodes_per_step * world / e2e_s, "unit": UNIT,
-               "h2d_bytes_per_step": m * 16, "d2h_bytes_per_step": 8,
+               "h2d_bytes_per_step": records * 16 + (272 if splits else 0),
+               "d2h_bytes_per_step": 272 if splits else 8,
                "solve_ms": 1e3 * e2e_s, "enumerate_ms": r["enumerate_ms"],
                "upload_ms": r["upload_ms"]}
 
@@ -754,6 +759,9 @@ def main():
                            "n": n, "d": d, "subproblems": m, "nodes_per_step": nodes_per_step,
                            "layout": args.layout, "block": args.block, "blocks_per_sm": args.bps,
                            "order": args.order,
+                           "nodes": "queen placements of Algorithm 2's tree below the prefixes "
+                                    "(the oracle's node count); the default form's look-ahead "
+                                    "finds the same solutions in fewer steps",
                            "l2": "flushed between steps (256 MiB write outside the timed events)",
                            "parallelism": f"replicas x{world}"},
                 "solve_ms": ms_per_step, "total": total_q, "wall_s": t_wall,

@@ -1,5 +1,6 @@
-// lookahead.cu -- the default search form's production kernel (layout REGP):
-// Algorithm 2 with a one-row look-ahead.
+// lookahead.cu -- the default search form's production kernels (layout REGP):
+// Algorithm 2 with a one-row look-ahead, on whole records, on records split into
+// units, under row masks (nq_count_constrained), and fed by a ring (the server).
 //
 // A child is entered only if its own row has a free column AND the row after
 // that would still have one under the child's state. Both tests are NORs of
@@ -9,21 +10,23 @@
 // traffic at N = 18 (counted on a sampled tree: 14.8 M steps, 9.4 M entered
 // frames -> 11.9 M, 7.3 M).
 //
-// What bounds it (N = 18, d = 7, 7.4 M subproblems in one launch, 20.0 ms
-// against 26.2 ms for the same search without look-ahead): issue slots 85 %, the ALU pipe 84 % and the shared
-// memory data path 86 % at once, so a step has to lose instructions, ALU work
-// and stack traffic together to get faster. Tried and slower, all on that
-// workload: high-half multiplies in place of the right shifts (22.6 ms), a
+// What bounds it (N = 18, d = 7, 7.4 M subproblems in one launch, 19.4 ms
+// against 26.2 ms for the same search without look-ahead): issue slots 85 %, the
+// ALU pipe 84 % and the shared memory data path 86 % at once, so a step has to
+// lose instructions, ALU work and stack traffic together to get faster. Tried
+// and slower, all on that workload, against 20.0 ms for the step as it is in a
+// bare kernel: high-half multiplies in place of the right shifts (22.6 ms), a
 // compare for the last column in place of the population count (22.4 ms),
 // dropping the candidates that a forced next row rules out (25.7 ms: five more
 // instructions for 16 % fewer steps).
 //
-// Records that are few or heavy are split into units (look_kernel_split) by the
-// digits of the unit's index, so that splitting needs no memory and no launch of
-// its own; the lanes of a warp that has nothing left to take share its last
-// subtrees. Before, one lane searched each record: 2048 records of N = 22, d = 7
-// took 509 ms of which 3.5 ms were work, now 4.3 ms; N = 14 from d = 3 1.97 ms,
-// now 0.07 ms; N = 18 from d = 5 53.6 ms, now 18.5 ms.
+// Records that are few or heavy are split (look_kernel_split) by the digits of an
+// index, so that splitting needs no memory and no launch of its own; a warp's
+// idle lanes take frames of its busy ones when its range is used up. Before, one
+// lane searched each record: 2048 records of N = 22, d = 7 took 509 ms of which
+// 3.5 ms were work, now 4.1 ms; N = 14 from d = 3 1.97 ms, now 0.057 ms (about 8
+// us of work: searches of about 100 steps are as small as pays); N = 18 from d =
+// 5 53.6 ms, now 17.8 ms.
 #include "nq_internal.h"
 
 namespace nqi {
@@ -113,7 +116,7 @@ __device__ __forceinline__ void look_step(uint32_t &c, uint32_t &L, uint32_t &R,
 // after them, so a last-row child is counted and not entered.
 // The last row is a compare of the row field, no population count.
 // Six queries of two queens at N = 16: 98 ms with the host enumerating the
-// subproblems on one core, 1.8 ms as one split record (of which 1.2 ms are the
+// subproblems on one core, 0.50 ms as one split record (of which 0.2 ms are the
 // six calls' own cost).
 template <uint32_t ROW>
 __device__ __forceinline__ void look_step_masked(uint32_t &c, uint32_t &L, uint32_t &R,
@@ -167,63 +170,107 @@ __device__ __forceinline__ void look_step_masked(uint32_t &c, uint32_t &L, uint3
         : "memory");
 }
 
-// One unit of split work: the part of a record's subtree that the digits of s
-// name. Level j (row d + j) has a digit of several bits, the most significant
-// level first. Every level but the last: the t-th free column, or nothing
-// when there are fewer (the digit covers every column the row could have
-// free). The last level: the free columns t, t + R, t + 2R, ... of R = 2^bits,
-// so nothing is left out there with a small digit. The units of a record
+// Split work: the part of a record's subtree that the digits of s name. Level j
+// (row d + j) has a digit of several bits, the most significant level first,
+// which names the t-th free column of its row, or nothing when there are fewer
+// (the digit covers every column the row could have free). The parts of a record
 // partition its solutions.
-//   returns  0: nothing here, 1: search from (c, l, r) with candidates av
-//            (l, r as they reach this row), 2: *found solutions and no search
-//   skip     units to the next one that may hold something
+//
+// Place the first `levels` rows' queens:
+//   returns  0: nothing here, 1: (c, l, r) reach row + levels, with `shift` bits
+//            of s left, 2: the board is complete and *found solutions
+//   skip     values of s to the next one that may hold something
 // ROW > 0: row `row` takes only the columns of its mask (a table of ROW bytes a
 // row), and the board ends after `rows` rows; c holds no pre-set columns.
 template <uint32_t ROW>
-__device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint64_t digits,
-                                          int shift, uint32_t &c, uint32_t &l, uint32_t &r,
-                                          uint32_t &av, uint32_t &found, uint32_t &skip,
-                                          const uint32_t table, uint32_t row, uint32_t rows) {
-    constexpr bool MASKED = ROW > 0u;
+__device__ __forceinline__ uint32_t free_columns(uint32_t c, uint32_t l, uint32_t r,
+                                                 const uint32_t table, uint32_t row) {
+    uint32_t x = ~(c | l | r);
+    if (ROW > 0u) {
+        uint32_t mask;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mask) : "r"(table + ROW * row) : "memory");
+        x &= mask;
+    }
+    return x;
+}
+template <uint32_t ROW>
+__device__ __forceinline__ int descend(uint32_t s, const int levels, uint64_t &digits, int &shift,
+                                       uint32_t &c, uint32_t &l, uint32_t &r, uint32_t &found,
+                                       uint32_t &skip, const uint32_t table, uint32_t row,
+                                       const uint32_t rows) {
     skip = 1u;
-    for (int j = 0; j < levels; ++j, digits >>= 4, ++row) {
-        const uint32_t bits = (uint32_t)digits & 15u;
+    for (int j = 0; j <= levels; ++j, ++row) {
         const uint32_t here = s & ((1u << shift) - 1u);  // this level's digit and those below
-        shift -= (int)bits;
-        if (MASKED ? row == rows : c == ~0u) {
-            // every row is placed: the solution belongs to the unit of zeros
-            skip = (1u << (shift + (int)bits)) - here;
+        if (ROW > 0u ? row == rows : c == ~0u) {  // the solution belongs to the digits of zeros
+            skip = (1u << shift) - here;
             found = here == 0u ? 1u : 0u;
             return 2;
         }
-        uint32_t x = ~(c | l | r);
-        if (MASKED) {
-            uint32_t mask;
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mask) : "r"(table + ROW * row) : "memory");
-            x &= mask;
-        }
+        if (j == levels) return 1;
+        const uint32_t bits = (uint32_t)digits & 15u;
+        digits >>= 4;
+        shift -= (int)bits;
+        uint32_t x = free_columns<ROW>(c, l, r, table, row);
         for (uint32_t t = here >> shift; t && x; --t) x &= x - 1u;
         if (x == 0u) {  // and nothing at any higher value of this digit
             skip = (1u << (shift + (int)bits)) - here;
             return 0;
         }
         const uint32_t p = x & (0u - x);
-        if (j + 1 < levels) {
-            c |= p;
-            l = (l | p) << 1;
-            r = (r | p) >> 1;
-        } else {
-            av = p;
-            for (x ^= p; x;) {
-                for (uint32_t t = (1u << bits) - 1u; t && x; --t) x &= x - 1u;
-                const uint32_t q = x & (0u - x);
-                av |= q;
-                x ^= q;
-            }
-        }
+        c |= p;
+        l = (l | p) << 1;
+        r = (r | p) >> 1;
     }
-    // the last row (the last level's row is row - 1 now): each candidate is a solution
-    if (MASKED ? row == rows : __popc(c) == 31) {
+    return 1;
+}
+
+// A parent: the frame that the digits lead to, in row + levels - 1, whose
+// candidates x are handed out one by one. Returns as descend.
+template <uint32_t ROW>
+__device__ __forceinline__ int split_parent(uint32_t s, const int levels, uint64_t digits,
+                                            int shift, uint32_t &c, uint32_t &l, uint32_t &r,
+                                            uint32_t &x, uint32_t &found, uint32_t &skip,
+                                            const uint32_t table, uint32_t row, uint32_t rows) {
+    const int got = descend<ROW>(s, levels - 1, digits, shift, c, l, r, found, skip, table, row,
+                                 rows);
+    if (got != 1) return got;
+    row += (uint32_t)levels - 1u;
+    x = free_columns<ROW>(c, l, r, table, row);
+    if (x == 0u) return 0;
+    if (ROW > 0u ? row + 1u == rows : __popc(c) == 31) {  // the last row
+        found = (uint32_t)__popc(x);
+        return 2;
+    }
+    return 1;
+}
+
+// A unit (the server's kernel): as a parent, with one more digit of the last
+// row's free columns t, t + R, t + 2R, ... of R = 2^bits, so that a small digit
+// leaves nothing out: search from (c, l, r) with candidates av.
+template <uint32_t ROW>
+__device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint64_t digits,
+                                          int shift, uint32_t &c, uint32_t &l, uint32_t &r,
+                                          uint32_t &av, uint32_t &found, uint32_t &skip,
+                                          const uint32_t table, uint32_t row, uint32_t rows) {
+    const int got = descend<ROW>(s, levels - 1, digits, shift, c, l, r, found, skip, table, row,
+                                 rows);
+    if (got != 1) return got;
+    row += (uint32_t)levels - 1u;
+    const uint32_t here = s & ((1u << shift) - 1u);
+    uint32_t x = free_columns<ROW>(c, l, r, table, row);
+    for (uint32_t t = here; t && x; --t) x &= x - 1u;
+    if (x == 0u) {
+        skip = (1u << shift) - here;
+        return 0;
+    }
+    av = x & (0u - x);
+    for (x ^= av; x;) {
+        for (uint32_t t = (1u << shift) - 1u; t && x; --t) x &= x - 1u;
+        const uint32_t q = x & (0u - x);
+        av |= q;
+        x ^= q;
+    }
+    if (ROW > 0u ? row + 1u == rows : __popc(c) == 31) {  // the last row
         found = (uint32_t)__popc(av);
         return 2;
     }
@@ -235,10 +282,15 @@ __device__ __forceinline__ int split_unit(uint32_t s, const int levels, uint64_t
 // lanes as they become idle. One atomic serves a whole range, and a launch
 // whose records fit the first ranges needs no cursor. Consecutive ranges go to
 // different blocks first, so that few records spread over the SMs.
-// SPLIT: the indices are units (split_unit), 2^split_shift to a record, and a
-// unit's count is added into its record's entry (zeroed before the launch).
-// Units that cannot hold anything are passed over in one go: the warp's
-// position moves on by the last asking lane's skip.
+// SPLIT: the indices are parents (split_parent), 2^split_shift to a record, and
+// what is found below one is added into its record's entry (zeroed before the
+// launch). The warp opens 32 parents at once, every lane one, busy or not, and
+// queues those that hold something in shared memory; idle lanes take the queued
+// parents' candidates one by one. (Each idle lane decoding its own unit, as it
+// became idle, cost some 350 instructions a unit for mostly one lane at a time:
+// 2048 records of N = 22 4.36 ms, 4.12 ms so; 10^5 records of N = 12..17 0.97 and
+// 0.85 ms.) Parents that cannot hold anything are passed over in one go: the
+// warp's position moves on by the last lane's skip.
 // MASKED (split only): one table of row masks for the launch, above the stacks.
 template <bool SPLIT, bool MASKED>
 __device__ __forceinline__ void look_body(const SearchArgs &a) {
@@ -255,7 +307,14 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
     const uint64_t total = SPLIT ? a.n << a.split_shift : a.n;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
 
-    const uint32_t table = sbase + (uint32_t)a.slots * stride;
+    // above the stacks, the warp's queue of 32 opened parents: {c, l, r, candidates},
+    // and {record, weight | N << 2 above its 48 bits}
+    unsigned char *const above = look_smem + (uint32_t)a.slots * stride;
+    uint4 *const q_frame = reinterpret_cast<uint4 *>(above) + (threadIdx.x & ~31u);
+    uint2 *const q_from =
+        reinterpret_cast<uint2 *>(above + 16u * blockDim.x) + (threadIdx.x & ~31u);
+    uint32_t q_at = 0, q_end = 0, q_x = 0;  // entries left, candidates left of entry q_at
+    const uint32_t table = sbase + (uint32_t)a.slots * stride + kSplitQueueBytes * blockDim.x;
     const uint32_t thr = MASKED ? (uint32_t)(a.expect_n - 1) << kRowShift : 0u;
     if (MASKED) {
         if (threadIdx.x < 32u)
@@ -319,6 +378,34 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
         bool need = idle;
         unsigned need_mask = __ballot_sync(~0u, need);
         while (need_mask) {
+            if (SPLIT && q_at < q_end) {  // hand out the candidates of one parent
+                const uint32_t rank = __popc(need_mask & lt_mask);
+                const uint32_t asked = __popc(need_mask), open = __popc(q_x);
+                if (need && rank < open) {
+                    const uint4 f = q_frame[q_at];
+                    const uint2 from = q_from[q_at];
+                    uint32_t x = q_x;
+                    for (uint32_t t = rank; t; --t) x &= x - 1u;
+                    idx = (uint64_t)from.x | (uint64_t)(from.y & 0xFFFFu) << 32;
+                    wn = from.y >> 16;
+                    sol = 0;
+                    busy = true;
+                    c = f.x;
+                    L = f.y << 1;
+                    R = f.z >> 1;
+                    av = x & (0u - x);
+                    top = base + stride;
+                    need = false;
+                }
+                if (asked >= open) {
+                    ++q_at;
+                    if (q_at < q_end) q_x = q_frame[q_at].w;
+                } else {
+                    for (uint32_t t = asked; t; --t) q_x &= q_x - 1u;
+                }
+                need_mask = __ballot_sync(~0u, need);
+                continue;
+            }
             if (rem == 0u) {
                 if (exhausted || (SPLIT && __popc(need_mask) < a.refill)) break;
                 unsigned long long f = 0;
@@ -330,12 +417,15 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                 }
                 rem = total - next < range ? (uint32_t)(total - next) : range;
             }
-            const uint32_t ready = rem;
-            const uint32_t rank = __popc(need_mask & lt_mask);
+            // each idle lane takes a record, or (SPLIT) every lane opens a parent
+            const uint32_t rank = SPLIT ? lane : (uint32_t)__popc(need_mask & lt_mask);
             uint32_t skip = 1u;
-            if (need && rank < ready) {
+            bool open = false;
+            uint4 frame = make_uint4(0u, 0u, 0u, 0u);
+            uint2 from = make_uint2(0u, 0u);
+            if ((SPLIT || need) && rank < rem) {
                 uint64_t at = next + rank;
-                uint32_t s = 0u;  // the unit's digits
+                uint32_t s = 0u;  // the parent's digits
                 if (SPLIT) {
                     s = (uint32_t)at & ((1u << a.split_shift) - 1u);
                     at >>= a.split_shift;
@@ -355,22 +445,15 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                     if (SPLIT) skip = (1u << a.split_shift) - s;
                 } else if (SPLIT) {
                     uint32_t cc = MASKED ? P.x : P.x | ~last;
-                    uint32_t ll = P.y, rr = P.z & last, a0 = 0, found = 0;
-                    const int got = split_unit<MASKED ? 8u : 0u>(s, a.levels, a.digits, a.split_shift, cc,
-                                                       ll, rr, a0, found, skip, table, d, n);
+                    uint32_t ll = P.y, rr = P.z & last, x = 0, found = 0;
+                    const int got =
+                        split_parent<MASKED ? 8u : 0u>(s, a.levels, a.digits, a.split_shift, cc, ll,
+                                                       rr, x, found, skip, table, d, n);
                     if (got == 2) finish(pi, found, w | (n << 2));
-                    if (got == 1) {
-                        idx = pi;
-                        wn = w | (n << 2);
-                        sol = 0;
-                        busy = true;
-                        c = MASKED ? cc | ((d + (uint32_t)a.levels) << kRowShift) : cc;
-                        L = ll << 1;
-                        R = rr >> 1;
-                        av = a0;
-                        top = base + stride;
-                        need = false;
-                    }
+                    open = got == 1;
+                    frame = make_uint4(MASKED ? cc | ((d + (uint32_t)a.levels) << kRowShift) : cc,
+                                       ll, rr, x);
+                    from = make_uint2((uint32_t)pi, (uint32_t)(pi >> 32) | (w | (n << 2)) << 16);
                 } else {
                     const uint32_t c0 = P.x | ~last;
                     const uint32_t l0 = P.y, r0 = P.z & last;
@@ -393,10 +476,23 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
                     }
                 }
             }
-            const uint32_t asked = __popc(need_mask);
-            uint32_t taken = asked < ready ? asked : ready;
-            if (SPLIT && asked <= ready) {  // every asker had a unit: pass over empty ones
-                taken += __shfl_sync(~0u, skip, 31 - __clz((int)need_mask)) - 1u;
+            const uint32_t asked = SPLIT ? 32u : (uint32_t)__popc(need_mask);
+            uint32_t taken = asked < rem ? asked : rem;
+            if (SPLIT) {
+                const unsigned opened = __ballot_sync(~0u, open);
+                __syncwarp();
+                if (open) {
+                    const uint32_t e = (uint32_t)__popc(opened & lt_mask);
+                    q_frame[e] = frame;
+                    q_from[e] = from;
+                }
+                __syncwarp();
+                q_at = 0u;
+                q_end = (uint32_t)__popc(opened);
+                if (q_end) q_x = q_frame[0].w;
+                __syncwarp();
+                // pass over parents that hold nothing
+                taken += __shfl_sync(~0u, skip, (int)taken - 1) - 1u;
                 taken = taken < rem ? taken : rem;
             }
             next += taken;
@@ -405,7 +501,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
         }
         if (need_mask == ~0u) break;  // the whole warp is idle, and nothing is left
 
-        if (SPLIT && need_mask && rem == 0u) {
+        if (SPLIT && need_mask && rem == 0u && q_at == q_end) {
             // Each idle lane takes the shallowest saved frame of a busy lane of
             // its warp, and leaves a sentinel in its place.
             const bool giver = !need && top > bot + stride;
@@ -492,9 +588,9 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
 // idle (or after 64x that many rounds in any case), so the kernel always ends
 // by itself once the host stops feeding it.
 //
-// Records that the host enumerated down to 4 per lane took one core longer than
-// the search (a burst of 32 requests of N = 10..15: 123 ms, of which 2 ms were
-// search); now the host makes at most some records per warp.
+// A burst of 32 requests of N = 10..15 takes 4.8 ms (1.0 ms of it the 32
+// submissions); with the host enumerating subproblems down to four per lane on
+// one core it took 123-190 ms.
 // ---------------------------------------------------------------------------
 constexpr int kServeRefill = 8;  // idle lanes for which a warp takes a new record
 

@@ -71,7 +71,7 @@ struct SearchArgs {
     // Layout REGP's production kernel only (lookahead.cu):
     int rows;           // rows that a record may have left (max_n - min_d)
     uint32_t range;     // indices a warp takes at once
-    // work split below the records (levels 0: not split): 2^split_shift units
+    // work split below the records (levels 0: not split): 2^split_shift parents
     // to a record, level j's digit in the j-th nibble of `digits`, in bits
     int levels;
     int split_shift;
@@ -201,6 +201,7 @@ struct ServeArgs {
 // The production kernel of layout REGP (lookahead.cu): plain, with the records'
 // subtrees split, or split and under row masks.
 void *look_kernel_ptr(bool split, bool masked);
+constexpr uint32_t kSplitQueueBytes = 24u;  // of shared memory a thread, for opened parents
 
 void *serve_kernel_ptr();  // (lookahead.cu)
 // How records with d rows placed of a board under row masks are cut into units:

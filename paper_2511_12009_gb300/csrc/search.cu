@@ -1223,7 +1223,8 @@ int make_plan(int max_n, int min_d, bool diag, bool constrained, const nq_config
     p.rows = max_n - min_d;
     // (a split record's search starts `levels - 1` rows further down)
     p.slots = slots_needed(p.layout, max_n, p.levels ? std::min(max_n, min_d + p.levels - 1) : min_d);
-    const size_t per_thread = (size_t)p.slots * (p.layout == NQ_LAYOUT_AVAIL ? 4u : 16u);
+    const size_t per_thread = (size_t)p.slots * (p.layout == NQ_LAYOUT_AVAIL ? 4u : 16u) +
+                              (p.levels || constrained ? kSplitQueueBytes : 0u);
     const size_t extra = constrained ? 32u * 8u : 0u;  // the masks, two rows to an entry
     if ((size_t)p.block * per_thread + extra > (size_t)max_smem) {
         int fit = (int)(((size_t)max_smem - extra) / per_thread) / 32 * 32;
@@ -1258,9 +1259,10 @@ double subtree_steps(int n, int rows) {
                     0.013134 * n * n);
 }
 
-// How the records' subtrees are cut into units.
+// How the records' subtrees are cut into units, one for each free column of the
+// last level's row.
 struct Cut {
-    int levels = 0, shift = 0;  // rows that the units fix, bits of a unit's index
+    int levels = 0, shift = 0;  // rows that the units fix, bits of the digits
     uint64_t digits = 0;        // bits of each level's digit, a nibble each
     double live = 0.0;          // units that hold something, about
 };
@@ -1283,16 +1285,17 @@ int row_caps(int N, int d, const uint32_t *allowed, int *cap) {
 // that search like a free board of size `board`.
 //
 // Split while there is less than a unit for every fourth lane and a unit is not
-// small in itself (setting one up costs some ten steps, less on the first level:
-// 148 records of N = 10, d = 3 take 13.3 us unsplit and 11.3 us with one level;
-// 110 of N = 13, d = 2 27 us down to 80 steps and 40 us down to 50), or while a
-// unit is more than an eighth of a lane's share of the work (the largest are a
-// few times the mean). A level more or less where the line lies costs little
-// (N = 16, d = 5: 1 level 0.60 ms, 2 levels 0.56 ms, none 1.25 ms; N = 18, d =
-// 5: 20.3, 18.4, 38.9 ms), a missing one much (2048 records of N = 22, d = 7:
-// 1 level 44 ms, 3 levels 5.5 ms, 4 levels 4.5 ms, 5 levels 6.5 ms, none
-// 326 ms).
-Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, int min_levels) {
+// small in itself (148 records of N = 10, d = 3 take 13.3 us unsplit and 11.3 us
+// with one level), or while a unit is more than an eighth of a lane's share of
+// the work (the largest are a few times the mean). A level more or less where
+// the line lies costs little (strided: N = 16, d = 5 1 level 0.60 ms, 2 levels
+// 0.56 ms, none 1.25 ms; N = 18, d = 5 20.3, 18.4, 38.9 ms), a missing one much
+// (2048 records of N = 22, d = 7: 1 level 44 ms, 3 levels 5.5 ms, 4 levels 4.5
+// ms, 5 levels 6.5 ms, none 326 ms).
+// strided: the last level's digit strides over its row's free columns (the
+// server's units); otherwise that row's columns are handed out one by one.
+Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, int min_levels,
+               bool strided) {
     int open_rows[NQ_MAX_N + 2] = {};  // rows j.. with a choice
     for (int j = rows - 1; j >= 0; --j) open_rows[j] = open_rows[j + 1] + (cap[j] > 1 ? 1 : 0);
     Cut cut;
@@ -1309,14 +1312,14 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, in
         if (c.levels > kSplitMaxLevels) break;
         double lv = (double)n, un = 0.0;
         for (int j = 0; j < c.levels; ++j) {
-            // Enough bits for every column that could be free; at most 2 on the
-            // last level, whose digit strides over the free columns.
+            // Enough bits for every column that could be free; on the last level 2
+            // at most (strided), or none.
             const bool last = j + 1 == c.levels;
             int b = 0;
             while ((1 << b) < cap[j]) ++b;
-            if (last) b = std::min(b, 2);
+            if (last) b = strided ? std::min(b, 2) : 0;
             const double open = std::max(1.0, 0.6 * cap[j]);  // columns free, about
-            const double taken = last ? std::min(open, (double)(1 << b)) : open;
+            const double taken = last && strided ? std::min(open, (double)(1 << b)) : open;
             c.digits |= (uint64_t)b << (4 * j);
             c.shift += b;
             lv *= taken;
@@ -1345,7 +1348,7 @@ int serve_cut(int N, int d, const uint32_t allowed[32], uint64_t n, double lanes
     const int rows = N - d, board = row_caps(N, d, allowed, cap);
     // a lane's search starts in row d + levels - 1 and needs N less that frames
     const int need = rows >= 2 ? std::max(1, rows + 1 - slots) : 1;
-    Cut cut = choose_cut(cap, rows, board, n, lanes, need);
+    Cut cut = choose_cut(cap, rows, board, n, lanes, need, true);
     if (cut.levels < 1 && rows <= 1) cut.levels = 1;  // a solved board or its last row
     if (cut.levels < need || cut.levels < 1) return NQ_ESTACK;
     out->levels = cut.levels;
@@ -1364,7 +1367,7 @@ int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t
     if (may_split && !p.stream && n) {
         int cap[NQ_MAX_N + 1] = {};
         const int board = row_caps(max_n, min_d, allowed, cap);
-        cut = choose_cut(cap, p.rows, board, n, lanes, allowed ? 1 : 0);
+        cut = choose_cut(cap, p.rows, board, n, lanes, allowed ? 1 : 0, false);
     }
     const int levels = cut.levels, shift = cut.shift;
     const uint64_t digits = cut.digits;
@@ -1380,19 +1383,24 @@ int plan_records(int max_n, int min_d, bool diag, const nq_config *cfg, uint64_t
     // frames of its busy ones, so that the units go round (Q(19): at 1 idle lane
     // 147.3 ms, at 8 151.2 ms, at 16 154.6 ms; N = 15 from d = 3: 0.219, 0.214,
     // 0.172 ms).
-    p.refill = cut.live > 8.0 * lanes ? 1 : 16;
-    // A warp takes 32 indices x claim at once. Of split work: half of that
-    // where the first ranges cover everything (other warps get the rest and
-    // each one's lanes share), and more where the empty units among them are
-    // many, as long as every warp still takes some 64 ranges -- 8 under row
-    // masks, where one record's units are nearly all empty (six queries at N =
-    // 16: 2.0 ms at 64 ranges, 1.7 ms at 8; 2048 records of N = 22: 4.4 ms at
-    // 64, 5.3 ms at 8).
+    const bool many = cut.live > 8.0 * lanes;
+    p.refill = many ? 1 : 16;
+    // A warp takes 32 indices x claim at once. Of split work fewer, down to 4,
+    // until every warp has a few ranges to take (N = 15 from d = 3: 0.197 ms with
+    // 32 parents, 0.128 ms with 8; many units like more ranges: N = 18 from d = 5
+    // 18.0 and 17.75 ms; a single range for each of few parents needs no cursor),
+    // and more where most parents hold nothing, as long as every warp still takes
+    // some 64 ranges -- 8 under row masks, where one record's parents are nearly
+    // all empty (2048 records of N = 22: 4.0 ms at 64, 4.8 ms at 8).
     const uint64_t total = n << shift;
     const uint64_t warps = (uint64_t)p.grid * (uint64_t)(p.block / 32);
     p.range = 32u * std::min(claim, 1024u);
-    if (levels && total <= warps * 16u) p.range = 16u;
-    while (levels && p.range < 32768u && total / p.range > (allowed ? 16 : 128) * warps) p.range *= 2u;
+    if (levels) {
+        while (p.range > 4u && total < (many && !allowed ? 16u : 2u) * warps * p.range)
+            p.range /= 2u;
+        if (total <= warps) p.range = 1u;
+        while (p.range < 32768u && total / p.range > (allowed ? 16u : 128u) * warps) p.range *= 2u;
+    }
     p.cursor = total > warps * p.range;
     if (!p.cursor)  // no more blocks than ranges: few records take one warp of each block
         p.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(p.grid, (total + p.range - 1) / p.range));

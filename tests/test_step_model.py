@@ -385,7 +385,7 @@ def test_look_ahead_sentinel_holds_32_idle_steps():
         step_look(state, stack, top)
 
 
-# --- work split below a record (layout REGP) ----------------------------------------
+# --- work split below a record (lookahead.cu) -----------------------------------------
 
 def digit_bits(free_columns, last):
     b = 1
@@ -395,7 +395,7 @@ def digit_bits(free_columns, last):
 
 
 def split_unit(s, bits, c, l, r):
-    """(kind, state, candidates, found, skip) of unit s of a record, as the split
+    """(kind, state, candidates, found, skip) of unit s of a record, as the server's
     kernel decodes it: kind 0 nothing, 1 search, 2 solutions found."""
     shift = sum(bits)
     av = 0
@@ -451,6 +451,56 @@ def test_split_units_partition_the_subtree(orc, n, d, levels, rows):
         while s < 1 << sum(bits):
             kind, st, av, found, skip = split_unit(s, bits, *state)
             total += found if kind == 2 else below(*st, av) if kind == 1 else 0
+            assert skip >= 1
+            s += skip
+        assert total == int(want[i])
+
+
+def split_parent(s, bits, c, l, r):
+    """(kind, state, candidates, found, skip) of parent s of a record: its digits'
+    queens placed, the next row's columns open (layout REGP's split launch)."""
+    shift = sum(bits)
+    for j in range(len(bits) + 1):
+        here = s & ((1 << shift) - 1)
+        if c == M:
+            return 2, None, 0, int(here == 0), (1 << shift) - here
+        if j == len(bits):
+            break
+        shift -= bits[j]
+        x = ~(c | l | r) & M
+        for _ in range(here >> shift):
+            x &= x - 1 if x else 0
+        if x == 0:
+            return 0, None, 0, 0, (1 << (shift + bits[j])) - here
+        p = x & -x
+        c, l, r = c | p, ((l | p) << 1) & M, (r | p) >> 1
+    x = ~(c | l | r) & M
+    if x == 0:
+        return 0, None, 0, 0, 1
+    if popc(c) == 31:
+        return 2, None, 0, popc(x), 1
+    return 1, (c, l, r), x, 0, 1
+
+
+@pytest.mark.parametrize("n,d,levels,rows", [(8, 0, 3, 8), (9, 2, 4, 9), (7, 3, 7, 9), (6, 6, 2, 6),
+                                             (6, 5, 3, 4), (10, 4, 1, 6), (9, 1, 2, 8), (5, 1, 6, 20)])
+def test_split_parents_partition_the_subtree(orc, n, d, levels, rows):
+    """The same for the parents that a split launch opens, their candidates handed
+    out one by one."""
+    bits = [digit_bits(max(rows - j, 1), False) for j in range(levels - 1)]
+    pre = nq.enumerate_prefixes(n, d)
+    want, _ = orc.count_prefixes(n, orc.prefixes(n, d)[0])
+    for i in sorted(set([0, len(pre) // 2, len(pre) - 1])):
+        rec, last = pre[i], (1 << n) - 1
+        state = int(rec["cols"]) | (~last & M), int(rec["ld"]), int(rec["rd"])
+        s = total = 0
+        while s < 1 << sum(bits):
+            kind, st, x, found, skip = split_parent(s, bits, *state)
+            if kind == 1:
+                while x:
+                    total += below(*st, x & -x)
+                    x &= x - 1
+            total += found if kind == 2 else 0
             assert skip >= 1
             s += skip
         assert total == int(want[i])
