@@ -690,27 +690,25 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
         bool need = idle;
         unsigned need_mask = __ballot_sync(~0u, need);
         bool stopping = false, may_claim = true;
-        int closing = 0;
-        if (need_mask == ~0u) {  // the mapped stop flag, read only by an all-idle warp
-            int st = 0;
-            if (lane == 0) st = a.ctl->stop;
-            stopping = __shfl_sync(~0u, st, 0) != 0;
+        if (need_mask == ~0u) {
+            // the mapped stop flag: read by an all-idle warp, and by each one only
+            // every 64th poll (3,648 warps reading host memory at every poll made
+            // the polls themselves take 100 us)
+            if (((idle_polls + blockIdx.x) & 63u) == 0u) {
+                int st = 0;
+                if (lane == 0) st = a.ctl->stop;
+                stopping = __shfl_sync(~0u, st, 0) != 0;
+            }
         } else if (skip) {
             --skip;
             may_claim = false;
-        }
-        if (__popc(need_mask) >= kServeRefill && rem == 0u && may_claim && !stopping) {
-            unsigned int cl = 0;  // the grid is leaving: nothing more from the ring
-            if (lane == 0)
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cl) : "l"(a.closing)
-                             : "memory");
-            closing = (int)__shfl_sync(~0u, cl, 0);
         }
         while (need_mask && !stopping) {
             if (rem == 0u) {
                 if (!may_claim || __popc(need_mask) < kServeRefill) break;
                 unsigned long long at = 0;
-                int got = 0;  // 1: record `at`, 0: there is none, -1: another warp is looking
+                // 1: record `at`, 0: there is none, -1: another warp is looking
+                int got = 0, closing = 0;
                 if (lane == 0) {
                     got = -1;
                     if (atomicCAS(&batch_lock, 0, 1) == 0) {
@@ -718,6 +716,9 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                         __threadfence_block();
                         volatile unsigned long long *first = &batch_first, *end = &batch_end;
                         unsigned long long f = *first, e = *end;
+                        if (f == e)  // (1: the grid is leaving, nothing more from the ring)
+                            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(closing)
+                                         : "l"(a.closing) : "memory");
                         if (f == e && !closing) {
                             unsigned long long h, cur;
                             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(h)
@@ -749,6 +750,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                 }
                 at = __shfl_sync(~0u, at, 0);
                 got = __shfl_sync(~0u, got, 0);
+                closing = __shfl_sync(~0u, closing, 0);
                 if (got <= 0) {
                     if (got == 0) {
                         backoff = backoff ? (backoff < 64u ? 2u * backoff : 64u) : 1u;
@@ -897,7 +899,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                 if (lane == 0) atomicAdd(a.idle_warps, 1u);
                 counted = true;
             }
-            if (counted) {
+            if (counted && (idle_polls & 15u) == 0u) {
                 int leave = 0;
                 if (lane == 0) {
                     unsigned int iw, sw;
