@@ -578,9 +578,10 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
 // cursor (which must not pass the published head); one by one for each warp, the
 // 3,648 warps of the grid got a record every 0.7 us between them.
 //
-// A slot's `remaining` counts what is still held of the request: its records
-// not yet handed out in full, and every lane searching a part of it. Whoever
-// gives back the last publishes the slot's total to mapped host memory.
+// A slot's `remaining` counts what is still held of the request: its records not
+// yet searched (a warp gives its own back together), and lanes that hold it by
+// themselves. Whoever gives back the last publishes the slot's total to mapped
+// host memory.
 //
 // Every wait is bounded: the claim retries a fixed number of times; a warp with
 // nothing to do polls the ring with back-off, counts itself idle after
@@ -588,7 +589,7 @@ __device__ __forceinline__ void look_body(const SearchArgs &a) {
 // idle (or after 64x that many rounds in any case), so the kernel always ends
 // by itself once the host stops feeding it.
 //
-// A burst of 32 requests of N = 10..15 takes 4.8 ms (1.0 ms of it the 32
+// A burst of 32 requests of N = 10..15 takes 1.7 ms (0.9 ms of it the 32
 // submissions); with the host enumerating subproblems down to four per lane on
 // one core it took 123-190 ms.
 // ---------------------------------------------------------------------------
@@ -659,11 +660,22 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
     // lanes still searching are not held up by lookups that find nothing.
     uint32_t backoff = 0, skip = 0;
 
-    auto give_back = [&](int slot, uint64_t s) {
+    // The warp holds the records that it took of one request (`held` of them, of
+    // held_slot) until none of its lanes works on them, and adds their solutions
+    // up in its lanes (acc). Only when it turns to another request while lanes
+    // still search the old one do those lanes hold the request each for itself
+    // (own). One atomic per record and lane instead put all of a large request's
+    // traffic on one address: N = 17 alone 13.9 ms, 5.2 ms so.
+    int held_slot = 0;
+    uint32_t held = 0;
+    bool own = false;
+    uint64_t acc = 0;
+
+    auto give_back = [&](int slot, uint64_t s, uint32_t tokens) {
         ServeSlot &q = a.slot_info[slot];
         if (s) atomicAdd(&q.total, (unsigned long long)s);
         __threadfence();
-        if (atomicSub(&q.remaining, 1u) == 1u) {
+        if (atomicSub(&q.remaining, tokens) == tokens) {
             __threadfence();
             const unsigned long long tot = atomicAdd(&q.total, 0ull);
             const unsigned long long seq =
@@ -674,13 +686,31 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
             __threadfence_system();
         }
     };
+    // Give the held records back; lanes still at work on them hold the request.
+    auto let_go = [&]() {
+        const bool works = cur_slot >= 0 && !own;
+        const unsigned at_work = __ballot_sync(~0u, works);
+        uint64_t sum = acc;
+        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(~0u, sum, o);
+        if (lane == 0) {
+            if (at_work)
+                atomicAdd(&a.slot_info[held_slot].remaining, (unsigned)__popc(at_work));
+            give_back(held_slot, sum, held);
+        }
+        own = own || works;
+        acc = 0;
+        held = 0;
+        __syncwarp();
+    };
 
     for (;;) {
         const bool idle = top == bot;
         if (idle) {
             if (cur_slot >= 0) {
-                give_back(cur_slot, sol * cur_w);
+                if (own) give_back(cur_slot, sol * cur_w, 1u);
+                else acc += sol * cur_w;
                 cur_slot = -1;
+                own = false;
             }
             bot = top = base;
             c = kSentMaskedC;
@@ -768,6 +798,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                 P = ld_cg4(a.ring + (at & a.ring_mask));
                 const uint32_t n = (P.w >> 2) & 31u, d = (P.w >> 7) & 31u, w = P.w & 3u;
                 rec_slot = (int)(P.w >> 12);
+                if (held && rec_slot != held_slot) let_go();
                 const uint32_t last = (n >= 1u) ? (0xFFFFFFFFu >> (32u - n)) : 0u;
                 bool ok = rec_slot < a.nslots && n >= 1u && n <= (uint32_t)kMaxConstrainedN &&
                           (w == 1u || w == 2u) && d <= n && (P.x & ~last) == 0u &&
@@ -787,7 +818,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                     if (lane == 0) {
                         look_error(a.status, NQ_EINVAL);
                         a.ctl->error = NQ_EINVAL;  // mapped: the next poll reports it
-                        if (rec_slot < a.nslots) give_back(rec_slot, 0);
+                        if (rec_slot < a.nslots) give_back(rec_slot, 0, 1u);
                     }
                     __syncwarp();
                     continue;
@@ -803,6 +834,8 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                     if (lane == 0) sts1(gens + 4u * (uint32_t)rec_slot, gen);
                 }
                 __syncwarp();
+                held_slot = rec_slot;
+                ++held;
                 next = 0u;
                 rem = 1u << shift;
             }
@@ -810,13 +843,11 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
             const uint32_t last = 0xFFFFFFFFu >> (32u - n);
             const uint32_t rank = __popc(need_mask & lt_mask);
             uint32_t past = 1u;
-            bool started = false;
             if (need && rank < rem) {
                 uint32_t cc = P.x, ll = P.y, rr = P.z & last, a0 = 0, found = 0;
                 const int got = split_unit<4u>(next + rank, levels, digits, shift, cc, ll, rr, a0,
                                                found, past, rec_tab, d, n);
-                if (got == 2 && found)
-                    atomicAdd(&a.slot_info[rec_slot].total, (unsigned long long)found * w);
+                if (got == 2) acc += (uint64_t)found * w;
                 if (got == 1) {
                     cur_slot = rec_slot;
                     cur_w = w;
@@ -829,12 +860,8 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                     av = a0;
                     top = base + stride;
                     need = false;
-                    started = true;
                 }
             }
-            // the lanes that started hold the request too
-            const unsigned st = __ballot_sync(~0u, started);
-            if (st && lane == 0) atomicAdd(&a.slot_info[rec_slot].remaining, (unsigned)__popc(st));
             const uint32_t asked = __popc(need_mask);
             uint32_t taken = asked < rem ? asked : rem;
             if (asked <= rem) {  // every asker had a unit: pass over empty ones
@@ -843,10 +870,6 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
             }
             next += taken;
             rem -= taken;
-            __threadfence();
-            __syncwarp();
-            if (rem == 0u && lane == 0) give_back(rec_slot, 0);  // the record is handed out
-            __syncwarp();
             need_mask = __ballot_sync(~0u, need);
         }
         if (need_mask && need_mask != ~0u && rem == 0u) {
@@ -863,6 +886,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                 const uint32_t w = __shfl_sync(~0u, cur_w, from);
                 const uint32_t tab = __shfl_sync(~0u, table, from);
                 const uint32_t th = __shfl_sync(~0u, thr, from);
+                const bool hold = __shfl_sync(~0u, (int)own, from) != 0;
                 if (taker) {
                     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(c), "=r"(L), "=r"(R), "=r"(av)
@@ -873,8 +897,9 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                     table = tab;
                     thr = th;
                     sol = 0;
+                    own = hold;
                     top = base + stride;
-                    atomicAdd(&a.slot_info[slot].remaining, 1u);
+                    if (hold) atomicAdd(&a.slot_info[slot].remaining, 1u);
                 }
                 __threadfence();
                 __syncwarp();
@@ -888,6 +913,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                 __syncwarp();
             }
         }
+        if (held && rem == 0u && !__any_sync(~0u, cur_slot >= 0 && !own)) let_go();
         if (need_mask == ~0u) {
             // (plain stores to the mapped block: no atomics on host memory)
             if (stopping) {

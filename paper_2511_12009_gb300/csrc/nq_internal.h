@@ -150,7 +150,7 @@ struct ServeSlot {
     int32_t levels, split_shift;
     uint64_t digits;
     unsigned long long total;  // solutions so far
-    uint32_t remaining;        // records not handed out in full, and lanes at work on the request
+    uint32_t remaining;        // records not searched, and lanes that hold the request
     uint32_t pad;
 };
 constexpr uint32_t kServeTable = 33u * 4u;  // bytes of a slot's masks in shared memory
