@@ -1286,8 +1286,10 @@ int row_caps(int N, int d, const uint32_t *allowed, int *cap) {
 //
 // Split while there is less than a unit for every fourth lane and a unit is not
 // small in itself (148 records of N = 10, d = 3 take 13.3 us unsplit and 11.3 us
-// with one level), or while a unit is more than an eighth of a lane's share of
-// the work (the largest are a few times the mean). A level more or less where
+// with one level), or while a unit is more than a thirty-second of a lane's share
+// of the work (the largest are several times the mean: Q(20) 1.27 s at an eighth,
+// 1.20 s at a thirty-second; N = 18 from d = 5 17.7 ms at either, 19.1 ms at a
+// sixty-fourth). A level more or less where
 // the line lies costs little (strided: N = 16, d = 5 1 level 0.60 ms, 2 levels
 // 0.56 ms, none 1.25 ms; N = 18, d = 5 20.3, 18.4, 38.9 ms), a missing one much
 // (2048 records of N = 22, d = 7: 1 level 44 ms, 3 levels 5.5 ms, 4 levels 4.5
@@ -1304,7 +1306,7 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, in
     double unit = subtree_steps(board, open_rows[0]);     // steps below one
     while (cut.levels < rows) {
         const bool few = live < lanes / 4.0 && unit > (cut.levels ? 80.0 : 20.0);
-        const bool uneven = unit > std::max(750.0, share / 8.0);
+        const bool uneven = unit > std::max(750.0, share / 32.0);
         if (!few && !uneven && cut.levels >= min_levels) break;
         Cut c;
         c.levels = cut.levels + 1;
