@@ -1414,6 +1414,7 @@ int launch_search(const SearchArgs &a, const Plan &p, bool diag, bool constraine
                   cudaStream_t s) {
     if (a.n == 0) return NQ_OK;
     if ((a.published != nullptr) != p.stream) return NQ_EINVAL;
+    if (p.look && a.by_tag) return NQ_EINVAL;  // (its records are split on the device instead)
     void *k = pick_kernel(p.layout, diag, constrained, p.donate && a.dq != nullptr, p.stream,
                           p.levels > 0);
     SearchArgs args = a;
