@@ -809,10 +809,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                     shift = (int)ld_cg1(&q->split_shift);
                     digits = (uint64_t)ld_cg1(&q->digits) |
                              (uint64_t)ld_cg1(reinterpret_cast<const uint32_t *>(&q->digits) + 1) << 32;
-                    const int first = (int)d + levels - 1;  // row that a lane's search starts in
-                    // (stack: the sentinel and the ancestors of rows first..N-2)
-                    ok = levels >= 1 && shift >= 0 && shift < 31 &&
-                         (first + 1 >= (int)n || (int)n - first <= a.slots);
+                    ok = serve_accepts((int)n, (int)d, levels, shift, a.slots);
                 }
                 if (!ok) {
                     if (lane == 0) {

@@ -172,6 +172,21 @@ struct ServeDone {
 
 constexpr int kServeMaxSlots = 256;
 
+// Split work (SearchArgs::levels, ServeSlot::levels): an index below a record has
+// at most this many digits, a nibble each in `digits`, and this many bits, so that
+// it and the skips over it are 32-bit numbers.
+constexpr int kMaxSplitLevels = 16;
+constexpr int kMaxSplitBits = 31;
+
+// Whether the server's kernel searches a record with d rows placed of an N x N
+// board that is cut like that, in `slots` frames a lane (the sentinel, and the
+// ancestors of rows d + levels - 1 .. N-2). serve_cut makes no other cuts.
+__host__ __device__ constexpr bool serve_accepts(int n, int d, int levels, int split_bits,
+                                                 int slots) {
+    return levels >= 1 && levels <= kMaxSplitLevels && split_bits >= 0 &&
+           split_bits <= kMaxSplitBits && (d + levels >= n || n - (d + levels - 1) <= slots);
+}
+
 struct ServeArgs {
     const nq_prefix *ring;           // ring_mask + 1 records (device)
     unsigned long long ring_mask;

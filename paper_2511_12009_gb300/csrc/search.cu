@@ -55,7 +55,6 @@ __device__ int g_stream_status[kStatusWords];
 
 namespace {
 
-constexpr int kSplitMaxLevels = 16;  // of split work (plan_records); a nibble each
 constexpr uint64_t kNone = ~0ull;
 constexpr int kChunk = 15;
 static_assert(kChunk < 16, "the sentinel frame holds 16 idle steps (32 for ~0 masks)");
@@ -1310,8 +1309,8 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, in
         if (!few && !uneven && cut.levels >= min_levels) break;
         Cut c;
         c.levels = cut.levels + 1;
-        while (c.levels < rows && c.levels < kSplitMaxLevels && cap[c.levels - 1] <= 1) ++c.levels;
-        if (c.levels > kSplitMaxLevels) break;
+        while (c.levels < rows && c.levels < kMaxSplitLevels && cap[c.levels - 1] <= 1) ++c.levels;
+        if (c.levels > kMaxSplitLevels) break;
         double lv = (double)n, un = 0.0;
         for (int j = 0; j < c.levels; ++j) {
             // Enough bits for every column that could be free; on the last level 2
@@ -1327,7 +1326,7 @@ Cut choose_cut(const int *cap, int rows, int board, uint64_t n, double lanes, in
             lv *= taken;
             if (last) un = subtree_steps(board, open_rows[j]) / taken;
         }
-        if (c.shift > 31 || n > (1ull << (62 - c.shift))) break;
+        if (c.shift > kMaxSplitBits || n > (1ull << (62 - c.shift))) break;
         cut = c;
         cut.live = live = lv;
         unit = un;
@@ -1352,7 +1351,7 @@ int serve_cut(int N, int d, const uint32_t allowed[32], uint64_t n, double lanes
     const int need = rows >= 2 ? std::max(1, rows + 1 - slots) : 1;
     Cut cut = choose_cut(cap, rows, board, n, lanes, need, true);
     if (cut.levels < 1 && rows <= 1) cut.levels = 1;  // a solved board or its last row
-    if (cut.levels < need || cut.levels < 1) return NQ_ESTACK;
+    if (!serve_accepts(N, d, cut.levels, cut.shift, slots)) return NQ_ESTACK;
     out->levels = cut.levels;
     out->split_shift = cut.shift;
     out->digits = cut.digits;

@@ -1,0 +1,164 @@
+// The server's host side without a GPU: libnq's own nq_server_* calls on a device
+// that is faked here (the executable's definitions of the runtime's functions
+// stand before libcudart's). Its kernel takes the published records one by one,
+// asks the function that the real kernel asks whether it searches such a record,
+// and answers a request with the number of its records.
+//
+//   cuts    the cuts that serve_cut makes, over boards, depths, stacks, record
+//           counts and seeded queens, that the kernel would not take or whose digits
+//           do not cover their rows
+//   burst max_n stack_slots N [row col]...    one request: records, answer, errors
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <vector>
+
+#include "nq_internal.h"
+
+using namespace nqi;
+
+extern "C" {
+cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 152 : 232448;
+    return cudaSuccess;
+}
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes *fa, const void *) {
+    std::memset(fa, 0, sizeof(*fa));
+    return cudaSuccess;
+}
+cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *nb, const void *, int block,
+                                                                   size_t smem, unsigned) {
+    const int by_regs = 65536 / (64 * block), by_smem = (int)(233472 / (smem + 1024 + 24));
+    *nb = by_regs < by_smem ? by_regs : by_smem;
+    return cudaSuccess;
+}
+cudaError_t cudaMalloc(void **p, size_t n) { *p = std::calloc(n, 1); return cudaSuccess; }
+cudaError_t cudaMallocHost(void **p, size_t n) { *p = std::calloc(n, 1); return cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { *p = std::calloc(n, 1); return cudaSuccess; }
+cudaError_t cudaHostGetDevicePointer(void **d, void *h, unsigned) { *d = h; return cudaSuccess; }
+cudaError_t cudaFree(void *p) { std::free(p); return cudaSuccess; }
+cudaError_t cudaFreeHost(void *p) { std::free(p); return cudaSuccess; }
+cudaError_t cudaMemset(void *p, int v, size_t n) { std::memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) {
+    std::memset(p, v, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    std::memcpy(d, s, n);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = nullptr; return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { *e = nullptr; return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+
+// serve_kernel: every published record, in order.
+cudaError_t cudaLaunchKernel(const void *, dim3, dim3, void **params, size_t, cudaStream_t) {
+    const ServeArgs &a = *static_cast<const ServeArgs *>(params[0]);
+    for (; *a.cursor < *a.head; ++*a.cursor) {
+        const nq_prefix &P = a.ring[*a.cursor & a.ring_mask];
+        ServeSlot &q = a.slot_info[NQ_META_TAG(P.meta)];
+        if (serve_accepts((int)NQ_META_N(P.meta), (int)NQ_META_D(P.meta), q.levels, q.split_shift,
+                          a.slots)) {
+            ++q.total;
+        } else {
+            a.ctl->error = NQ_EINVAL;
+        }
+        if (--q.remaining == 0) {
+            ServeDone &done = a.done[NQ_META_TAG(P.meta)];
+            done.total = q.total;
+            done.seq = q.seq;
+        }
+    }
+    return cudaSuccess;
+}
+}
+
+namespace {
+
+// Seeded queens, no two attacking each other: the row masks of a partial board.
+bool draw_masks(uint64_t &seed, int n, int k, uint32_t *allowed) {
+    auto next = [&]() {
+        seed = seed * 6364136223846793005ull + 1442695040888963407ull;
+        return (uint32_t)(seed >> 33);
+    };
+    nq_queen q[4];
+    for (int i = 0; i < k; ++i) q[i] = {(int8_t)(next() % n), (int8_t)(next() % n)};
+    bool conflict = false;
+    return constraint_masks(n, q, k, allowed, &conflict) == NQ_OK && !conflict;
+}
+
+int cuts() {
+    long made = 0, wide = 0, refused = 0, short_digit = 0;
+    uint64_t seed = 11;
+    for (int n = 1; n <= kMaxConstrainedN; ++n)
+        for (int k = 0; k <= 4; ++k) {
+            uint32_t allowed[32];
+            if (!draw_masks(seed, n, k, allowed)) continue;
+            for (int d = 0; d <= n; ++d)
+                for (int slots = 2; slots <= 27; ++slots)
+                    for (uint64_t records : {1ull, 700ull, 30000ull, 4000000ull})
+                        for (double lanes : {19456.0, 155648.0}) {
+                            ServeSlot s{};
+                            if (serve_cut(n, d, allowed, records, lanes, slots, &s)) continue;
+                            ++made;
+                            wide += s.split_shift == 31;
+                            refused += !serve_accepts(n, d, s.levels, s.split_shift, slots);
+                            int bits = 0;
+                            for (int j = 0; j < s.levels; ++j) {
+                                const int b = (int)(s.digits >> (4 * j) & 15u);
+                                bits += b;
+                                // (a row's free columns: those of its mask, less the rows above)
+                                if (j + 1 < s.levels && d + j < n) {
+                                    const int m = __builtin_popcount(allowed[d + j]);
+                                    short_digit += (1 << b) < (m < n - d - j ? m : n - d - j);
+                                }
+                            }
+                            short_digit += bits != s.split_shift;
+                        }
+        }
+    std::printf("%ld cuts, %ld of 31 bits, %ld refused, %ld short digits\n", made, wide, refused,
+                short_digit);
+    return 0;
+}
+
+int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
+    nq_server_config cfg{};
+    cfg.max_n = max_n;
+    cfg.stack_slots = stack_slots;
+    nq_server *s = nullptr;
+    uint64_t ticket = 0, published = 0, tickets[4], counts[4];
+    int rc = nq_server_create(&cfg, &s), got = 0;
+    if (!rc) rc = nq_server_submit(s, n, q.data(), (int)q.size(), &ticket);
+    if (rc) {
+        std::printf("refused %d\n", rc);
+        return 0;
+    }
+    nq_server_stats(s, nullptr, nullptr, nullptr, &published);
+    std::printf("%llu records", (unsigned long long)published);
+    for (int i = 0; i < 2; ++i) {
+        rc = nq_server_poll(s, tickets, counts, 4, &got);
+        std::printf(", poll %d:", rc);
+        for (int j = 0; j < got; ++j)
+            std::printf(" %s %llu", tickets[j] == ticket ? "answer" : "stranger",
+                        (unsigned long long)counts[j]);
+    }
+    std::printf("\n");
+    return nq_server_destroy(s);
+}
+
+}  // namespace
+
+int main(int argc, char **argv) {
+    if (argc == 2 && !std::strcmp(argv[1], "cuts")) return cuts();
+    if (argc < 5 || std::strcmp(argv[1], "burst")) return 2;
+    std::vector<nq_queen> q;
+    for (int i = 5; i + 1 < argc; i += 2)
+        q.push_back({(int8_t)std::atoi(argv[i]), (int8_t)std::atoi(argv[i + 1])});
+    return burst(std::atoi(argv[2]), std::atoi(argv[3]), std::atoi(argv[4]), q);
+}

@@ -171,3 +171,14 @@ def test_served_split_edges(orc):
                 res = run_stream(srv, stream, timeout_s=120)
                 assert [res["answers"][i] for i in range(len(reqs))] == want
             assert srv.poll() == []
+
+
+@pytest.mark.parametrize("max_n,stack,queens", [(18, 4, []), (21, 9, [(16, 15), (19, 6)])])
+def test_served_widest_cut(max_n, stack, queens):
+    """A stack so small that a record's units take 31 bits, the most that an index
+    may have: the answer is the board's count."""
+    from paper_2511_12009_gb300.serve import Server, run_stream
+    want = nq.count_constrained(max_n, queens) if queens else Q[max_n]
+    with Server(max_n=max_n, stack_slots=stack, request_slots=4, idle_ms=50) as srv:
+        res = run_stream(srv, [{"t": 0.0, "n": max_n, "queens": queens}], timeout_s=120)
+    assert res["answers"] == {0: want}

@@ -1,0 +1,44 @@
+"""CPU tests of the request server's host side: libnq's own nq_server_* calls on
+a faked device (server_on_host.cpp), whose kernel asks of each record what the
+real one asks."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2511_12009_gb300 import _build, nq
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    nq.lib()  # (built)
+    exe = str(tmp_path_factory.mktemp("host") / "server_on_host")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build.nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", _build.INCLUDE, "-I", _build.CSRC, "-I", cuda,
+                    os.path.join(HERE, "server_on_host.cpp"), _build.LIB,
+                    f"-Wl,-rpath,{_build.OUT_DIR}", "-o", exe], check=True)
+
+    def run(*args):
+        return subprocess.run([exe] + [str(a) for a in args], check=True, capture_output=True,
+                              text=True, timeout=120).stdout.strip()
+    return run
+
+
+def test_every_cut_is_one_the_kernel_takes(host):
+    """serve_cut over all boards, depths and stacks, the widest index (31 bits) among
+    them: the kernel takes each cut, and a digit covers its row's columns."""
+    made, wide, refused, short = (int(x.split()[0]) for x in host("cuts").split(", "))
+    assert made > 100000 and wide > 1000
+    assert refused == 0 and short == 0
+
+
+@pytest.mark.parametrize("max_n,stack,n,queens", [
+    (21, 9, 21, []), (21, 9, 21, [16, 15, 19, 6]), (22, 9, 22, [19, 20, 13, 5, 16, 6]),
+    (26, 0, 26, [15, 18, 14, 1, 2, 10, 20, 4, 17, 14]), (18, 4, 18, []), (20, 0, 20, [])])
+def test_admitted_requests_are_searched(host, max_n, stack, n, queens):
+    """Requests whose records are cut 31 bits wide (all but the last) are admitted
+    with records that the kernel searches, every one."""
+    records, first, second = host("burst", max_n, stack, n, *queens).split(", ")
+    assert first == f"poll 0: answer {records.split()[0]}" and second == "poll 0:"
