@@ -365,11 +365,16 @@ int nq_server_create(const nq_server_config *cfg, nq_server **out);
  */
 int nq_server_submit(nq_server *s, int N, const nq_queen *q, int k, uint64_t *ticket);
 
+/* In place of the count of a request that was not searched whole: the kernel found
+ * one of its records malformed (no count of a board N <= 26 is as large). */
+#define NQ_SERVER_NO_COUNT UINT64_MAX
+
 /*
  * Completed requests since the last poll: up to max (ticket, count) pairs, in
  * completion order; *n_done = how many were written. Also relaunches the kernel
  * if it left on an idle timeout while work was being published, and returns
- * the first error a kernel recorded.
+ * the first error a kernel recorded. A request with a record that the kernel
+ * did not search completes with NQ_SERVER_NO_COUNT.
  */
 int nq_server_poll(nq_server *s, uint64_t *tickets, uint64_t *counts, int max, int *n_done);
 

@@ -681,6 +681,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
             const unsigned long long seq =
                 *reinterpret_cast<const volatile unsigned long long *>(&q.seq);
             a.done[slot].total = tot;
+            a.done[slot].refused = *reinterpret_cast<const volatile uint32_t *>(&q.refused);
             __threadfence_system();
             a.done[slot].seq = seq;
             __threadfence_system();
@@ -815,7 +816,10 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                     if (lane == 0) {
                         look_error(a.status, NQ_EINVAL);
                         a.ctl->error = NQ_EINVAL;  // mapped: the next poll reports it
-                        if (rec_slot < a.nslots) give_back(rec_slot, 0, 1u);
+                        if (rec_slot < a.nslots) {
+                            atomicExch(&a.slot_info[rec_slot].refused, 1u);
+                            give_back(rec_slot, 0, 1u);
+                        }
                     }
                     __syncwarp();
                     continue;

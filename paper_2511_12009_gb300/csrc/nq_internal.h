@@ -151,7 +151,7 @@ struct ServeSlot {
     uint64_t digits;
     unsigned long long total;  // solutions so far
     uint32_t remaining;        // records not searched, and lanes that hold the request
-    uint32_t pad;
+    uint32_t refused;          // kernel: it gave a record back unsearched (total is no count)
 };
 constexpr uint32_t kServeTable = 33u * 4u;  // bytes of a slot's masks in shared memory
 
@@ -168,6 +168,7 @@ struct ServeControl {
 struct ServeDone {
     volatile unsigned long long total;
     volatile unsigned long long seq;
+    volatile unsigned long long refused;  // ServeSlot::refused
 };
 
 constexpr int kServeMaxSlots = 256;

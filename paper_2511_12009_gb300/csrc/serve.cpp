@@ -149,7 +149,8 @@ void collect(nq_server *s) {
         if (!r.active) continue;
         if (s->h_done[i].seq != r.ticket) continue;
         std::atomic_thread_fence(std::memory_order_acquire);
-        s->ready.emplace_back(r.ticket, (uint64_t)s->h_done[i].total);
+        s->ready.emplace_back(r.ticket, s->h_done[i].refused ? NQ_SERVER_NO_COUNT
+                                                             : (uint64_t)s->h_done[i].total);
         s->done_early.insert(r.ticket);
         r.active = false;
         ++s->completed;
@@ -223,6 +224,7 @@ extern "C" int nq_server_create(const nq_server_config *cfg, nq_server **out) {
     for (int i = 0; i < c.request_slots; ++i) {
         s->h_done[i].seq = 0;
         s->h_done[i].total = 0;
+        s->h_done[i].refused = 0;
     }
     s->req.resize(c.request_slots);
     s->gen.assign(c.request_slots, 0);
@@ -316,6 +318,7 @@ extern "C" int nq_server_submit(nq_server *s, int N, const nq_queen *q, int k, u
     info.seq = tk;
     info.remaining = (uint32_t)m;  // one hold for each record
     info.total = 0;
+    info.refused = 0;
     // (the copies of the submission before have ended: it waited for them)
     unsigned char *stage = static_cast<unsigned char *>(s->h_stage);
     std::memcpy(stage, &info, sizeof(info));

@@ -17,6 +17,9 @@ from collections import deque
 from . import nq
 
 
+NO_COUNT = (1 << 64) - 1  # NQ_SERVER_NO_COUNT
+
+
 class ServerConfig(ctypes.Structure):
     _fields_ = [("max_n", ctypes.c_int32), ("request_slots", ctypes.c_int32),
                 ("stack_slots", ctypes.c_int32), ("block", ctypes.c_int32),
@@ -67,11 +70,13 @@ class Server:
         nq._check(rc, "nq_server_submit")
         return int(t.value)
 
-    def poll(self) -> list[tuple[int, int]]:
+    def poll(self) -> list[tuple[int, int | None]]:
+        """Finished (ticket, count) pairs; None for a request that was not searched whole."""
         got = ctypes.c_int()
         nq._check(nq.lib().nq_server_poll(self._h, self._tk, self._ct, self._buf,
                                           ctypes.byref(got)), "nq_server_poll")
-        return [(int(self._tk[i]), int(self._ct[i])) for i in range(got.value)]
+        return [(int(self._tk[i]), None if self._ct[i] == NO_COUNT else int(self._ct[i]))
+                for i in range(got.value)]
 
     def stats(self) -> dict:
         v = [ctypes.c_uint64() for _ in range(4)]

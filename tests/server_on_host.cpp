@@ -8,6 +8,7 @@
 //           counts and seeded queens, that the kernel would not take or whose digits
 //           do not cover their rows
 //   burst max_n stack_slots N [row col]...    one request: records, answer, errors
+//   refuse max_n stack_slots N [row col]...   the same, its last record not searched
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -57,21 +58,26 @@ cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 
+bool refuse_last = false;
+
 // serve_kernel: every published record, in order.
 cudaError_t cudaLaunchKernel(const void *, dim3, dim3, void **params, size_t, cudaStream_t) {
     const ServeArgs &a = *static_cast<const ServeArgs *>(params[0]);
     for (; *a.cursor < *a.head; ++*a.cursor) {
         const nq_prefix &P = a.ring[*a.cursor & a.ring_mask];
         ServeSlot &q = a.slot_info[NQ_META_TAG(P.meta)];
-        if (serve_accepts((int)NQ_META_N(P.meta), (int)NQ_META_D(P.meta), q.levels, q.split_shift,
+        if (!(refuse_last && q.remaining == 1) &&
+            serve_accepts((int)NQ_META_N(P.meta), (int)NQ_META_D(P.meta), q.levels, q.split_shift,
                           a.slots)) {
             ++q.total;
         } else {
+            q.refused = 1;
             a.ctl->error = NQ_EINVAL;
         }
         if (--q.remaining == 0) {
             ServeDone &done = a.done[NQ_META_TAG(P.meta)];
             done.total = q.total;
+            done.refused = q.refused;
             done.seq = q.seq;
         }
     }
@@ -156,7 +162,8 @@ int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
 
 int main(int argc, char **argv) {
     if (argc == 2 && !std::strcmp(argv[1], "cuts")) return cuts();
-    if (argc < 5 || std::strcmp(argv[1], "burst")) return 2;
+    refuse_last = argc > 1 && !std::strcmp(argv[1], "refuse");
+    if (argc < 5 || (!refuse_last && std::strcmp(argv[1], "burst"))) return 2;
     std::vector<nq_queen> q;
     for (int i = 5; i + 1 < argc; i += 2)
         q.push_back({(int8_t)std::atoi(argv[i]), (int8_t)std::atoi(argv[i + 1])});

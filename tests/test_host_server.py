@@ -6,7 +6,7 @@ import subprocess
 
 import pytest
 
-from paper_2511_12009_gb300 import _build, nq
+from paper_2511_12009_gb300 import _build, nq, serve
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -42,3 +42,10 @@ def test_admitted_requests_are_searched(host, max_n, stack, n, queens):
     with records that the kernel searches, every one."""
     records, first, second = host("burst", max_n, stack, n, *queens).split(", ")
     assert first == f"poll 0: answer {records.split()[0]}" and second == "poll 0:"
+
+
+def test_a_request_not_searched_whole_has_no_count(host):
+    """A record that the kernel gives back unsearched is an error, and what the others
+    found is not delivered as the request's count."""
+    _, first, second = host("refuse", 20, 0, 12, 3, 4).split(", ")
+    assert first == f"poll {nq.NQ_EINVAL}: answer {serve.NO_COUNT}" and second == "poll 0:"
