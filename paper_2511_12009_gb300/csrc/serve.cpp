@@ -362,6 +362,7 @@ extern "C" int nq_server_submit(nq_server *s, int N, const nq_queen *q, int k, u
 extern "C" int nq_server_poll(nq_server *s, uint64_t *tickets, uint64_t *counts, int max,
                               int *n_done) {
     if (!s || !n_done || max < 0 || (max && (!tickets || !counts))) return NQ_EINVAL;
+    *n_done = 0;
     std::lock_guard<std::mutex> guard(s->mu);
     collect(s);
     bool pending = false;

@@ -58,6 +58,7 @@ class Server:
         self._buf = 4096
         self._tk = (ctypes.c_uint64 * self._buf)()
         self._ct = (ctypes.c_uint64 * self._buf)()
+        self._held = []  # taken by a poll that then raised
 
     def submit(self, n: int, queens) -> int | None:
         """Ticket of the admitted request, or None if the server is full."""
@@ -71,12 +72,16 @@ class Server:
         return int(t.value)
 
     def poll(self) -> list[tuple[int, int | None]]:
-        """Finished (ticket, count) pairs; None for a request that was not searched whole."""
+        """Finished (ticket, count) pairs; None for a request that was not searched whole.
+        Raises the first error that a kernel found; what finished beside it comes with the
+        next poll."""
         got = ctypes.c_int()
-        nq._check(nq.lib().nq_server_poll(self._h, self._tk, self._ct, self._buf,
-                                          ctypes.byref(got)), "nq_server_poll")
-        return [(int(self._tk[i]), None if self._ct[i] == NO_COUNT else int(self._ct[i]))
-                for i in range(got.value)]
+        rc = nq.lib().nq_server_poll(self._h, self._tk, self._ct, self._buf, ctypes.byref(got))
+        self._held += [(int(self._tk[i]), None if self._ct[i] == NO_COUNT else int(self._ct[i]))
+                       for i in range(got.value)]
+        nq._check(rc, "nq_server_poll")
+        done, self._held = self._held, []
+        return done
 
     def stats(self) -> dict:
         v = [ctypes.c_uint64() for _ in range(4)]

@@ -49,3 +49,28 @@ def test_a_request_not_searched_whole_has_no_count(host):
     found is not delivered as the request's count."""
     _, first, second = host("refuse", 20, 0, 12, 3, 4).split(", ")
     assert first == f"poll {nq.NQ_EINVAL}: answer {serve.NO_COUNT}" and second == "poll 0:"
+
+
+def test_poll_keeps_what_finished_beside_an_error(monkeypatch):
+    """Answers that nq_server_poll hands over together with an error come with the next
+    poll of the Python server."""
+    class Lib:
+        polls = [(nq.NQ_EINVAL, [(1, 10), (2, serve.NO_COUNT)]), (nq.NQ_OK, [(3, 30)])]
+
+        def nq_server_poll(self, h, tickets, counts, size, got):
+            rc, done = self.polls.pop(0)
+            for i, (t, c) in enumerate(done):
+                tickets[i], counts[i] = t, c
+            got._obj.value = len(done)
+            return rc
+
+        nq_server_create = nq_server_destroy = staticmethod(lambda *a: nq.NQ_OK)
+        nq_strerror = nq.lib().nq_strerror
+
+    lib = Lib()
+    monkeypatch.setattr(nq, "lib", lambda: lib)
+    monkeypatch.setattr(serve, "_declare", lambda: lib)
+    srv = serve.Server()
+    with pytest.raises(nq.NQError):
+        srv.poll()
+    assert srv.poll() == [(1, 10), (2, None), (3, 30)]
