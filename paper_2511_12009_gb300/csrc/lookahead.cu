@@ -41,8 +41,9 @@ constexpr int kLookSteps = 31;  // steps between bookkeeping points
 // 32 idle steps: one frame lasts a whole round.
 constexpr uint32_t kSentC = 0x55555555u, kSentL = 0xAAAAAAAAu, kSentR = 0x55555555u;
 constexpr uint32_t kSentAv = 0xFFFFFFFFu;
-// Under masks: the frame above row 31, whose masks are 0, with no diagonals.
-constexpr uint32_t kSentMaskedC = 31u << kRowShift;
+// Under masks: the frame above a row that no board has, whose mask is 0, with no
+// diagonals.
+constexpr uint32_t kSentMaskedC = (uint32_t)kSentinelRow << kRowShift;
 static_assert(kLookSteps < 32, "an idle lane must not use up the sentinel's candidates");
 
 extern __shared__ __align__(16) unsigned char look_smem[];
@@ -111,7 +112,7 @@ __device__ __forceinline__ void look_step(uint32_t &c, uint32_t &L, uint32_t &R,
 // << 27), so entering a child adds the next row where look_step moves a
 // register. The masks of the child's row and of the row after it are loaded from
 // a table whose address depends on the frame alone: 8 bytes a row holding both
-// (ROW = 8, one load), or 33 words (ROW = 4, two loads, half the table: the
+// (ROW = 8, one load), or a word a row (ROW = 4, two loads, half the table: the
 // server keeps one for each request). Rows at or below the last have mask 0
 // after them, so a last-row child is counted and not entered.
 // The last row is a compare of the row field, no population count.
@@ -621,8 +622,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(look_smem);
     const uint32_t stride = stack_slot_offset(blockDim.x, 0u, 1u, 16u);
     const uint32_t base = sbase + stack_slot_offset(blockDim.x, threadIdx.x, 0u, 16u);
-    const uint32_t tables = sbase + (uint32_t)a.slots * stride;      // nslots x 33 words
-    const uint32_t gens = tables + (uint32_t)a.nslots * kServeTable;  // nslots words
+    const uint32_t tables = sbase + (uint32_t)a.slots * stride;  // nslots x kServeTable
     // the block's batch of ring records: [first, end), taken under `lock`
     __shared__ unsigned long long batch_first, batch_end;
     __shared__ int batch_lock;
@@ -630,9 +630,8 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
         batch_first = batch_end = 0ull;
         batch_lock = 0;
     }
-    for (int i = threadIdx.x; i < a.nslots; i += blockDim.x) sts1(gens + 4u * i, 0xFFFFFFFFu);
     for (int i = threadIdx.x; i < a.nslots * (int)(kServeTable / 4u); i += blockDim.x)
-        sts1(tables + 4u * i, 0u);
+        sts1(tables + 4u * i, i % (int)(kServeTable / 4u) == (int)(kServeGen / 4u) ? 0xFFFFFFFFu : 0u);
     __syncthreads();
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -828,11 +827,12 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                 rec_tab = tables + kServeTable * (uint32_t)rec_slot;
                 const uint32_t gen = ld_cg1(&a.slot_info[rec_slot].gen);
                 __threadfence_block();
-                if (__any_sync(~0u, lds1(gens + 4u * (uint32_t)rec_slot) != gen)) {
-                    sts1(rec_tab + 4u * lane, ld_cg1(&a.slot_info[rec_slot].allowed[lane]));
+                if (__any_sync(~0u, lds1(rec_tab + kServeGen) != gen)) {
+                    if (lane <= (unsigned)kSentinelRow)
+                        sts1(rec_tab + 4u * lane, ld_cg1(&a.slot_info[rec_slot].allowed[lane]));
                     __threadfence_block();
                     __syncwarp();
-                    if (lane == 0) sts1(gens + 4u * (uint32_t)rec_slot, gen);
+                    if (lane == 0) sts1(rec_tab + kServeGen, gen);
                 }
                 __syncwarp();
                 held_slot = rec_slot;

@@ -47,7 +47,7 @@ struct SearchArgs {
     int order;                     // 1: claim the last index first
     int claim;                     // consecutive indices a lane claims at once (>= 1)
     // Constrained mode only (partial-board queries): the columns each row may
-    // take; rows >= N and entry 31 must be 0.
+    // take; 0 for rows >= N.
     uint32_t allowed[32];
     // Split subproblems: counts/nodes of record i are added to entry
     // tag(i) = meta >> 12, which must be below n_tags (else NQ_EINVAL).
@@ -153,7 +153,13 @@ struct ServeSlot {
     uint32_t remaining;        // records not searched, and lanes that hold the request
     uint32_t refused;          // kernel: it gave a record back unsearched (total is no count)
 };
-constexpr uint32_t kServeTable = 33u * 4u;  // bytes of a slot's masks in shared memory
+// A slot's part of shared memory: the masks of rows 0..26 (the row after the last of
+// the largest board has none) and of the sentinel's row, then the generation they are
+// of, where the sentinel's second mask would be (what that is does not matter). An
+// odd number of words, so that lanes at different requests meet few bank conflicts.
+constexpr int kSentinelRow = kMaxConstrainedN + 1;
+constexpr uint32_t kServeGen = (kSentinelRow + 1) * 4u;
+constexpr uint32_t kServeTable = kServeGen + 4u;
 
 // Host-visible control block (mapped pinned memory).
 struct ServeControl {

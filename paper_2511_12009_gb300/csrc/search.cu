@@ -1441,7 +1441,7 @@ int serve_plan(int max_n, int min_d, int nslots, int block, int *grid, size_t *s
             cudaSuccess)
         return NQ_ECUDA;
     const int sl = std::max(1, max_n - 1 - min_d) + 1;  // a sentinel, and frames down to row N-2
-    const size_t bytes = (size_t)sl * 16u * block + (size_t)nslots * (kServeTable + 4u);
+    const size_t bytes = (size_t)sl * 16u * block + (size_t)nslots * kServeTable;
     if (bytes > (size_t)max_smem) return NQ_ESTACK;
     void *k = serve_kernel_ptr();
     cudaFuncAttributes fa{};  // (raise only: another server may still relaunch with its size)

@@ -7,6 +7,8 @@
 //   cuts    the cuts that serve_cut makes, over boards, depths, stacks, record
 //           counts and seeded queens, that the kernel would not take or whose digits
 //           do not cover their rows
+//   shapes  launch shapes that fit an SM with 33 words a request slot beside the stacks
+//           and that serve_plan refuses
 //   burst max_n stack_slots N [row col]...    one request: records, answer, errors
 //   refuse max_n stack_slots N [row col]...   the same, its last record not searched
 #include <cstdio>
@@ -31,7 +33,8 @@ cudaError_t cudaFuncGetAttributes(cudaFuncAttributes *fa, const void *) {
 cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *nb, const void *, int block,
                                                                    size_t smem, unsigned) {
-    const int by_regs = 65536 / (64 * block), by_smem = (int)(233472 / (smem + 1024 + 24));
+    // (of shared memory, 1 KB a block and the kernel's own 32 bytes are taken)
+    const int by_regs = 65536 / (64 * block), by_smem = (int)(233472 / (smem + 1024 + 32));
     *nb = by_regs < by_smem ? by_regs : by_smem;
     return cudaSuccess;
 }
@@ -133,6 +136,22 @@ int cuts() {
     return 0;
 }
 
+int shapes() {
+    long fit = 0, refused = 0;
+    for (int block = 32; block <= 1024; block += 32)
+        for (int max_n = 1; max_n <= kMaxConstrainedN; ++max_n)
+            for (int nslots = 1; nslots <= kServeMaxSlots; ++nslots) {
+                const size_t stacks = (size_t)(max_n > 2 ? max_n : 2) * 16 * block;
+                if (stacks + nslots * 132 > 232448) continue;
+                int grid = 0, slots = 0;
+                size_t smem = 0;
+                ++fit;
+                refused += serve_plan(max_n, 0, nslots, block, &grid, &smem, &slots) != NQ_OK;
+            }
+    std::printf("%ld shapes, %ld refused\n", fit, refused);
+    return 0;
+}
+
 int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
     nq_server_config cfg{};
     cfg.max_n = max_n;
@@ -162,6 +181,7 @@ int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
 
 int main(int argc, char **argv) {
     if (argc == 2 && !std::strcmp(argv[1], "cuts")) return cuts();
+    if (argc == 2 && !std::strcmp(argv[1], "shapes")) return shapes();
     refuse_last = argc > 1 && !std::strcmp(argv[1], "refuse");
     if (argc < 5 || (!refuse_last && std::strcmp(argv[1], "burst"))) return 2;
     std::vector<nq_queen> q;

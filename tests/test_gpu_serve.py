@@ -182,3 +182,13 @@ def test_served_widest_cut(max_n, stack, queens):
     with Server(max_n=max_n, stack_slots=stack, request_slots=4, idle_ms=50) as srv:
         res = run_stream(srv, [{"t": 0.0, "n": max_n, "queens": queens}], timeout_s=120)
     assert res["answers"] == {0: want}
+
+
+def test_served_at_the_most_shared_memory():
+    """A block of 1024 threads with 14 frames each and 23 request slots: stacks and row
+    masks take all but a few bytes of an SM's shared memory."""
+    from paper_2511_12009_gb300.serve import Server, run_stream
+    reqs = [{"t": 0.0, "n": 6 + i % 8, "queens": []} for i in range(46)]
+    with Server(max_n=20, stack_slots=13, request_slots=23, block=1024, idle_ms=50) as srv:
+        res = run_stream(srv, reqs, timeout_s=120)
+    assert res["answers"] == {i: Q[r["n"]] for i, r in enumerate(reqs)}

@@ -34,6 +34,12 @@ def test_every_cut_is_one_the_kernel_takes(host):
     assert refused == 0 and short == 0
 
 
+def test_every_shape_that_fits_is_planned(host):
+    """Launch shapes up to the last bytes of an SM's shared memory."""
+    fit, refused = (int(x.split()[0]) for x in host("shapes").split(", "))
+    assert fit > 100000 and refused == 0
+
+
 @pytest.mark.parametrize("max_n,stack,n,queens", [
     (21, 9, 21, []), (21, 9, 21, [16, 15, 19, 6]), (22, 9, 22, [19, 20, 13, 5, 16, 6]),
     (26, 0, 26, [15, 18, 14, 1, 2, 10, 20, 4, 17, 14]), (18, 4, 18, []), (20, 0, 20, [])])
