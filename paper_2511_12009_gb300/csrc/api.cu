@@ -812,7 +812,11 @@ extern "C" int nq_count_constrained(int N, const nq_queen *q, int k, uint64_t *c
         *count_out = 0;
         return NQ_OK;
     }
-    if (k == 0) return nq_total(N, count_out);  // nothing given: the board's symmetries hold
+    if (k == 0) {  // nothing given: the board's symmetries hold
+        nq_config cfg{};  // (of nq_total's, NQ_LAYOUT and NQ_D do not reach this call)
+        cfg.layout = NQ_LAYOUT_REGP;
+        return total_split(N, std::min(N, kTotalRows), &cfg, count_out, nullptr);
+    }
     for (int r = 0; r < N; ++r)
         if (!allowed[r]) {  // a row that the given queens leave no column
             *count_out = 0;

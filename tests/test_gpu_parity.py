@@ -127,6 +127,15 @@ def test_environment_defaults(monkeypatch):
     assert r["d"] == nq.default_depth(16)
 
 
+@pytest.mark.parametrize("name,value", [("NQ_D", "9"), ("NQ_LAYOUT", "paper")])
+def test_constrained_takes_no_depth_or_layout_from_the_environment(monkeypatch, name, value):
+    """NQ_D and NQ_LAYOUT configure whole-board and prefix calls; partial boards, the one
+    with no queen given among them, are counted as without them."""
+    monkeypatch.setenv(name, value)
+    assert nq.count_constrained(8, []) == Q[8]
+    assert nq.count_constrained(8, [(0, 0)]) == 4
+
+
 @pytest.mark.parametrize("layout", LAYOUTS)
 def test_launch_shapes(orc, layout):
     """Block sizes, blocks per SM and claim order do not change any count."""
