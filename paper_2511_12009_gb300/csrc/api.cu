@@ -375,7 +375,10 @@ int search_staged(int N, int d, unsigned char *stage, uint64_t n, const nq_confi
     CallEvents ev;
     if (timing && (rc = ev.init())) return rc;
     if (timing) cudaEventRecord(ev.e[0], ctx.s);
-    rc = cuda_rc(cudaMemcpyAsync(dev, stage, bytes, cudaMemcpyHostToDevice, ctx.s));
+    {
+        Range r("nq.upload");
+        rc = cuda_rc(cudaMemcpyAsync(dev, stage, bytes, cudaMemcpyHostToDevice, ctx.s));
+    }
     if (timing) cudaEventRecord(ev.e[1], ctx.s);
     Plan p{};
     if (!rc)
@@ -406,17 +409,27 @@ int search_staged(int N, int d, unsigned char *stage, uint64_t n, const nq_confi
 int total_split(int N, int d, const nq_config *cfg, uint64_t *total_out, nq_timing *timing) {
     const auto t_start = Clock::now();
     const int b = std::min(d, kTotalRows);
-    uint64_t n = 0;
-    int rc = nq_enumerate_prefixes(N, b, nullptr, 0, &n);
+    PrefixCut cut;
+    int rc;
+    {
+        Range r("nq.enumerate.count");
+        rc = cut_prefixes(N, b, &cut);
+    }
     if (rc) return rc;
+    const uint64_t n = cut.first.back();
     unsigned char *stage =
         static_cast<unsigned char *>(t_stage.get(kHead + n * sizeof(nq_prefix)));
     if (!stage) return NQ_ENOMEM;
-    if (n && (rc = nq_enumerate_prefixes(N, b, staged_records(stage), n, &n))) return rc;
+    {
+        Range r("nq.enumerate.write");
+        write_prefix_nodes(cut, 0, cut.nodes.size(), staged_records(stage), n);
+    }
     const double enum_ms = ms_since(t_start);
     uint64_t prefixes = n;
     rc = search_staged(N, b, stage, n, cfg, nullptr, total_out, timing, [&]() -> int {
-        return timing && d > b ? nq_enumerate_prefixes(N, d, nullptr, 0, &prefixes) : NQ_OK;
+        if (!timing || d <= b) return NQ_OK;
+        Range r("nq.enumerate.count");
+        return nq_enumerate_prefixes(N, d, nullptr, 0, &prefixes);
     });
     if (rc) return rc;
     if (timing) {
