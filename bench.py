@@ -698,7 +698,7 @@ def main():
     e2e = None
     if args.e2e_steps > 0:
         e2e_times = []
-        e2e_cfg = nq.make_config(args.layout, args.block, args.bps, args.order, d)
+        e2e_cfg = nq.make_config(args.layout, args.block, args.bps, args.order, args.d)
         for k in range(args.e2e_steps + 1):
             t0 = time.perf_counter()
             r = nq.total_ex(n, e2e_cfg)
@@ -708,10 +708,11 @@ def main():
             if k:  # the first call warms the pinned staging buffer
                 e2e_times.append(dt)
         e2e_s = max_over_ranks(dist, float(np.mean(e2e_times)), device)
-        # The default form copies the first four rows' prefixes and a 272-byte head (which
-        # comes back); the others the whole depth-d set, and read one total.
+        # The default form copies the first four rows' prefixes (a chosen depth's whole set)
+        # and a 272-byte head, which comes back; the others copy the whole set and read one
+        # total.
         splits = args.layout in ("default", "regp")
-        records = nq.prefix_count(n, min(d, 4)) if splits else m
+        records = nq.prefix_count(n, min(d, 4)) if splits and not args.d else m
         e2e = {"value": nodes_per_step * world / e2e_s, "unit": UNIT,
                "h2d_bytes_per_step": records * 16 + (272 if splits else 0),
                "d2h_bytes_per_step": 272 if splits else 8,

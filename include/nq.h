@@ -137,7 +137,9 @@ typedef struct nq_config {
     int32_t order;         /* claim order: 0 default (last index first: canonical order
                               puts the heavier subtrees late, so they start first),
                               1 index order, 2 last index first */
-    int32_t d;             /* nq_total_ex only: prefix depth 1..N (0 = default) */
+    int32_t d;             /* nq_total_ex only: prefix depth 1..N (0: nq_default_depth(N);
+                              layout REGP's production build then searches the prefixes
+                              of four rows and splits them on the device) */
     int32_t claim;         /* subproblems a lane claims per atomic (work chunk), 1..64 */
     int32_t donate;        /* subtree donation once the queue is empty (register
                               layouts): 0 default (off), 1 off, 2 on */
@@ -146,12 +148,12 @@ typedef struct nq_config {
 
 /* Timing of one nq_total_ex call, host wall clock in milliseconds. */
 typedef struct nq_timing {
-    double enumerate_ms; /* host prefix enumeration */
+    double enumerate_ms; /* host prefix enumeration (of the records that are searched) */
     double upload_ms;    /* host -> device copy of the prefixes */
     double kernel_ms;    /* the search kernel, CUDA events on the call's stream */
     double total_ms;     /* whole call */
-    uint64_t prefixes;   /* number of subproblems */
-    int32_t d;           /* depth used */
+    uint64_t prefixes;   /* number of subproblems of the depth-d set */
+    int32_t d;           /* depth asked for, or nq_default_depth(N) */
     int32_t layout;      /* layout used */
     int32_t block;       /* block size used */
     int32_t grid;        /* blocks launched */
@@ -234,15 +236,17 @@ int nq_sync(void *stream);
 
 /*
  * Q(N), the number of solutions of the N-Queens problem, synchronously:
- * enumerate (default depth), upload, search, sum weight x count. 1 <= N <= 28;
- * N >= 29 returns NQ_EOVERFLOW (the count exceeds 64 bits, Section 4.5).
+ * enumerate (as nq_total_ex with no depth given), upload, search, sum weight x
+ * count. 1 <= N <= 28; N >= 29 returns NQ_EOVERFLOW (the count exceeds 64 bits,
+ * Section 4.5).
  */
 int nq_total(int N, uint64_t *total_out);
 
 /*
  * nq_total with a chosen configuration (cfg == NULL or cfg->d == 0: the
- * default depth). nodes_out (optional) runs the diagnostic kernel build and
- * returns the search nodes below all prefixes (unweighted). timing optional.
+ * default depth, see nq_config.d). nodes_out (optional) runs the diagnostic
+ * kernel build and returns the search nodes below all prefixes (unweighted).
+ * timing optional.
  */
 int nq_total_ex(int N, const nq_config *cfg, uint64_t *total_out, uint64_t *nodes_out,
                 nq_timing *timing);

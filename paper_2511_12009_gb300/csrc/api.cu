@@ -340,10 +340,12 @@ extern "C" int nq_sync(void *stream) {
 namespace {
 
 // nq_total_ex in the default form: the launch splits subtrees by itself
-// (plan_records), so only the prefixes of the first kTotalRows rows are made and
-// copied, some 10^4 records, and the depth-d set is only counted, beside
-// the search, for the caller who asks. Before, the host wrote all of it (N = 18:
-// 7.4 M records, 2.8 ms of host work and 118 MB beside the search).
+// (plan_records), so with no depth given only the prefixes of the first kTotalRows
+// rows are made and copied (2.5 MB at N = 28, the largest), and the default depth's
+// set is only counted, beside the search, for the caller who asks. Before, the host
+// wrote all of it (N = 18: 7.4 M records, 2.8 ms of host work and 118 MB beside the
+// search). A depth that the caller gives is the depth that is searched: N = 18 at
+// d = 7 22.7 ms (20.1 ms with none given), N = 20 at d = 7 1.16 s (1.20 s).
 // kTotalRows: rows 0 and 1 hold the symmetry rules; two more leave the launch two
 // levels less to split at next to no host work (N = 14: search of 0.081, 0.082,
 // 0.064, 0.091 ms from 2, 3, 4, 5 rows; N = 17: 3.45, 3.58, 3.26, 3.15 ms).
@@ -406,9 +408,10 @@ int search_staged(int N, int d, unsigned char *stage, uint64_t n, const nq_confi
     return NQ_OK;
 }
 
-int total_split(int N, int d, const nq_config *cfg, uint64_t *total_out, nq_timing *timing) {
+// Search the set of depth b, report the one of depth d.
+int total_split(int N, int b, int d, const nq_config *cfg, uint64_t *total_out,
+                nq_timing *timing) {
     const auto t_start = Clock::now();
-    const int b = std::min(d, kTotalRows);
     PrefixCut cut;
     int rc;
     {
@@ -427,7 +430,7 @@ int total_split(int N, int d, const nq_config *cfg, uint64_t *total_out, nq_timi
     const double enum_ms = ms_since(t_start);
     uint64_t prefixes = n;
     rc = search_staged(N, b, stage, n, cfg, nullptr, total_out, timing, [&]() -> int {
-        if (!timing || d <= b) return NQ_OK;
+        if (!timing || d == b) return NQ_OK;
         Range r("nq.enumerate.count");
         return nq_enumerate_prefixes(N, d, nullptr, 0, &prefixes);
     });
@@ -459,7 +462,8 @@ extern "C" int nq_total_ex(int N, const nq_config *cfg, uint64_t *total_out, uin
     if (d < 0 || d > N) return NQ_EINVAL;
 
     const int lay = cfg->layout ? cfg->layout : NQ_LAYOUT_DEFAULT_SEARCH;
-    if (lay == NQ_LAYOUT_REGP && !nodes_out) return total_split(N, d, cfg, total_out, timing);
+    if (lay == NQ_LAYOUT_REGP && !nodes_out)
+        return total_split(N, cfg->d > 0 ? d : std::min(d, kTotalRows), d, cfg, total_out, timing);
 
     // a1 (counting pass): the set cut at its depth-3 nodes, the size of each part
     const auto t_enum = Clock::now();
@@ -828,7 +832,8 @@ extern "C" int nq_count_constrained(int N, const nq_queen *q, int k, uint64_t *c
     if (k == 0) {  // nothing given: the board's symmetries hold
         nq_config cfg{};  // (of nq_total's, NQ_LAYOUT and NQ_D do not reach this call)
         cfg.layout = NQ_LAYOUT_REGP;
-        return total_split(N, std::min(N, kTotalRows), &cfg, count_out, nullptr);
+        const int b = std::min(N, kTotalRows);
+        return total_split(N, b, b, &cfg, count_out, nullptr);
     }
     for (int r = 0; r < N; ++r)
         if (!allowed[r]) {  // a row that the given queens leave no column

@@ -1,20 +1,24 @@
-// The server's host side without a GPU: libnq's own nq_server_* calls on a device
-// that is faked here (the executable's definitions of the runtime's functions
-// stand before libcudart's). Its kernel takes the published records one by one,
-// asks the function that the real kernel asks whether it searches such a record,
-// and answers a request with the number of its records.
+// The host side of libnq's calls without a GPU, on a device that is faked here (the
+// executable's definitions of the runtime's functions stand before libcudart's).
+// Its server's kernel takes the published records one by one, asks the function that
+// the real kernel asks whether it searches such a record, and answers a request with
+// the number of its records. Its search kernels answer with the number of theirs.
 //
 //   cuts    the cuts that serve_cut makes, over boards, depths, stacks, record
 //           counts and seeded queens, that the kernel would not take or whose digits
 //           do not cover their rows
 //   shapes  launch shapes that fit an SM with 33 words a request slot beside the stacks
 //           and that serve_plan refuses
+//   total N d    nq_total_ex in the default form (d = 0: no depth given): records
+//           launched and the rows placed in them, records and rows in the timing
 //   burst max_n stack_slots N [row col]...    one request: records, answer, errors
 //   refuse max_n stack_slots N [row col]...   the same, its last record not searched
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <vector>
+
+#include <cuda.h>
 
 #include "nq_internal.h"
 
@@ -58,13 +62,44 @@ cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { *e = nullptr; return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = nullptr; return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 0; return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *c) {
+    *c = cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const cudaMemPoolProps *) {
+    *p = nullptr;
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t) {
+    return cudaMalloc(p, n);
+}
+cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return cudaFree(p); }
+CUresult get_current(CUcontext *c) { *c = reinterpret_cast<CUcontext>(8); return CUDA_SUCCESS; }
+CUresult get_id(CUcontext, unsigned long long *id) { *id = 8; return CUDA_SUCCESS; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult *q) {
+    *f = !std::strcmp(name, "cuCtxGetCurrent") ? reinterpret_cast<void *>(&get_current)
+                                                : reinterpret_cast<void *>(&get_id);
+    *q = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
 cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 
 bool refuse_last = false;
 
-// serve_kernel: every published record, in order.
-cudaError_t cudaLaunchKernel(const void *, dim3, dim3, void **params, size_t, cudaStream_t) {
+// serve_kernel: every published record, in order; the others: what they are given.
+cudaError_t cudaLaunchKernel(const void *k, dim3, dim3, void **params, size_t, cudaStream_t) {
+    if (k != serve_kernel_ptr()) {
+        const SearchArgs &a = *static_cast<const SearchArgs *>(params[0]);
+        std::printf("search %llu records of %u rows, ", (unsigned long long)a.n,
+                    NQ_META_D(a.pre[0].meta));
+        a.totals[a.expect_n] = a.n;
+        return cudaSuccess;
+    }
     const ServeArgs &a = *static_cast<const ServeArgs *>(params[0]);
     for (; *a.cursor < *a.head; ++*a.cursor) {
         const nq_prefix &P = a.ring[*a.cursor & a.ring_mask];
@@ -152,6 +187,17 @@ int shapes() {
     return 0;
 }
 
+int total(int n, int d) {
+    nq_config cfg{};
+    cfg.d = d;
+    nq_timing t{};
+    uint64_t q = 0;
+    const int rc = nq_total_ex(n, d ? &cfg : nullptr, &q, nullptr, &t);
+    std::printf("rc %d, total %llu, timing %llu of %d\n", rc, (unsigned long long)q,
+                (unsigned long long)t.prefixes, t.d);
+    return 0;
+}
+
 int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
     nq_server_config cfg{};
     cfg.max_n = max_n;
@@ -182,6 +228,8 @@ int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
 int main(int argc, char **argv) {
     if (argc == 2 && !std::strcmp(argv[1], "cuts")) return cuts();
     if (argc == 2 && !std::strcmp(argv[1], "shapes")) return shapes();
+    if (argc == 4 && !std::strcmp(argv[1], "total"))
+        return total(std::atoi(argv[2]), std::atoi(argv[3]));
     refuse_last = argc > 1 && !std::strcmp(argv[1], "refuse");
     if (argc < 5 || (!refuse_last && std::strcmp(argv[1], "burst"))) return 2;
     std::vector<nq_queen> q;

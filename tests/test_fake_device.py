@@ -1,6 +1,6 @@
-"""CPU tests of the request server's host side: libnq's own nq_server_* calls on
-a faked device (server_on_host.cpp), whose kernel asks of each record what the
-real one asks."""
+"""CPU tests of the host side of libnq's calls, on a faked device (fake_device.cpp):
+the request server, whose faked kernel asks of each record what the real one
+asks, and what nq_total_ex has searched."""
 import os
 import subprocess
 
@@ -14,10 +14,10 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 @pytest.fixture(scope="module")
 def host(tmp_path_factory):
     nq.lib()  # (built)
-    exe = str(tmp_path_factory.mktemp("host") / "server_on_host")
+    exe = str(tmp_path_factory.mktemp("host") / "fake_device")
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build.nvcc()))), "include")
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", _build.INCLUDE, "-I", _build.CSRC, "-I", cuda,
-                    os.path.join(HERE, "server_on_host.cpp"), _build.LIB,
+                    os.path.join(HERE, "fake_device.cpp"), _build.LIB,
                     f"-Wl,-rpath,{_build.OUT_DIR}", "-o", exe], check=True)
 
     def run(*args):
@@ -80,3 +80,22 @@ def test_poll_keeps_what_finished_beside_an_error(monkeypatch):
     with pytest.raises(nq.NQError):
         srv.poll()
     assert srv.poll() == [(1, 10), (2, None), (3, 30)]
+
+
+@pytest.mark.parametrize("n,d", [(12, 6), (13, 2), (14, 5), (16, 6), (9, 9), (8, 1)])
+def test_total_searches_the_depth_that_is_asked_for(host, n, d):
+    """A chosen depth is the depth of the records that are searched, and the one timed."""
+    m = nq.prefix_count(n, d)
+    assert host("total", n, d) == (f"search {m} records of {d} rows, rc 0, total {m}, "
+                                   f"timing {m} of {d}")
+
+
+@pytest.mark.parametrize("n", [3, 5, 12, 16])
+def test_total_chooses_four_rows(host, n):
+    """With no depth given the default form searches at most four rows' prefixes; the
+    timing is of the default depth's set."""
+    d = nq.default_depth(n)
+    m = nq.prefix_count(n, min(d, 4))
+    want = f"search {m} records of {min(d, 4)} rows, " if m else ""
+    assert host("total", n, 0) == (want + f"rc 0, total {m}, "
+                                   f"timing {nq.prefix_count(n, d)} of {d}")
