@@ -59,9 +59,9 @@ def default_depth(n: int) -> int:
 N22_D7_NODES = 143257329200995
 # DRAM traffic of one production search launch on the default workload (N=18,
 # d=7, default layout), dram__bytes_read.sum + dram__bytes_write.sum from one
-# ncu capture, valid only for the kernel source it was taken on: the sha256 of
-# lookahead.cu and nq_internal.h. Any change to them makes the figure stale, and
-# the roofline then reports traffic as null.
+# ncu capture, valid only for the sources it was taken on: the sha256 of
+# KERNEL_FILES. Any change to them makes the figure stale, and the roofline then
+# reports traffic as null.
 TRAFFIC_NCU = {"n": 18, "d": 7, "layout": "default", "bytes": 119676928 + 29240576,
                "kernel_sha256": "4d2587d70cc41f12c6de225c244fee886545ebdeaab245412e5bc5e02d3e47b1"}
 
@@ -190,10 +190,14 @@ class ClockSampler:
                 "reasons": sorted(reasons)}
 
 
+# the default kernel, its arguments, and the planning of its launch
+KERNEL_FILES = ("lookahead.cu", "nq_internal.h", "search.cu")
+
+
 def kernel_sha256() -> str:
     import hashlib
     h = hashlib.sha256()
-    for name in ("lookahead.cu", "nq_internal.h"):
+    for name in KERNEL_FILES:
         with open(os.path.join(ROOT, "paper_2511_12009_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()

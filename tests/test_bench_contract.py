@@ -80,3 +80,22 @@ def test_served_answer_check_catches_a_wrong_answer():
         wrong = dict(right)
         wrong[i] += 1
         assert not bench.check_served_answers(reqs, wrong, sample=1000, n16=0)["exact"]
+
+
+def test_traffic_figure_holds_for_its_sources_only(tmp_path, monkeypatch):
+    """The measured bytes per launch are reported while the kernel and the planning of
+    its launch are the ones they were measured with."""
+    sys.path.insert(0, ROOT)
+    import shutil
+    import bench
+    csrc = os.path.join("paper_2511_12009_gb300", "csrc")
+    shutil.copytree(os.path.join(ROOT, csrc), tmp_path / csrc)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    monkeypatch.setitem(bench.TRAFFIC_NCU, "kernel_sha256", bench.kernel_sha256())
+    assert bench.measured_traffic(18, 7, "default") == bench.TRAFFIC_NCU["bytes"]
+    for name in ("lookahead.cu", "search.cu", "nq_internal.h"):
+        path = tmp_path / csrc / name
+        text = path.read_text()
+        path.write_text(text + "// changed\n")
+        assert bench.measured_traffic(18, 7, "default") is None, name
+        path.write_text(text)
