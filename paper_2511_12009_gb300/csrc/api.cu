@@ -98,7 +98,8 @@ constexpr size_t kStreamsKept = 8;
 
 struct Kept {
     cudaMemPool_t pool = nullptr;
-    std::vector<cudaStream_t> streams;
+    cudaStream_t streams[kStreamsKept] = {};
+    size_t n_streams = 0;
 };
 std::mutex g_kept_mu;
 
@@ -155,8 +156,8 @@ struct CallCtx {
         if (cudaStreamSynchronize(s) == cudaSuccess) {
             std::lock_guard<std::mutex> g(g_kept_mu);
             Kept *k = kept_locked();
-            if (k && k->streams.size() < kStreamsKept) {
-                k->streams.push_back(s);
+            if (k && k->n_streams < kStreamsKept) {
+                k->streams[k->n_streams++] = s;
                 return;
             }
         }
@@ -166,9 +167,8 @@ struct CallCtx {
         {
             std::lock_guard<std::mutex> g(g_kept_mu);
             Kept *k = kept_locked();
-            if (k && !k->streams.empty()) {
-                s = k->streams.back();
-                k->streams.pop_back();
+            if (k && k->n_streams) {
+                s = k->streams[--k->n_streams];
                 return NQ_OK;
             }
         }

@@ -11,11 +11,14 @@
 //           and that serve_plan refuses
 //   total N d    nq_total_ex in the default form (d = 0: no depth given): records
 //           launched and the rows placed in them, records and rows in the timing
+//   nomem   nq_total(5) with room for no host allocation, for one, for two, ...: the
+//           number of calls until one had enough
 //   burst max_n stack_slots N [row col]...    one request: records, answer, errors
 //   refuse max_n stack_slots N [row col]...   the same, its last record not searched
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <new>
 #include <vector>
 
 #include <cuda.h>
@@ -23,6 +26,20 @@
 #include "nq_internal.h"
 
 using namespace nqi;
+
+// Host allocations left before all fail; -1: none does.
+long allocations_left = -1;
+bool out_of_memory = false;
+
+void *operator new(size_t n) {
+    if (allocations_left == 0) out_of_memory = true;
+    if (allocations_left == 0) throw std::bad_alloc();
+    if (allocations_left > 0) --allocations_left;
+    if (void *p = std::malloc(n)) return p;
+    throw std::bad_alloc();
+}
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, size_t) noexcept { std::free(p); }
 
 extern "C" {
 cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
@@ -57,7 +74,10 @@ cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cu
     std::memcpy(d, s, n);
     return cudaSuccess;
 }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = nullptr; return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
+    *s = reinterpret_cast<cudaStream_t>(16);
+    return cudaSuccess;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { *e = nullptr; return cudaSuccess; }
@@ -198,6 +218,22 @@ int total(int n, int d) {
     return 0;
 }
 
+int nomem() {
+    int calls = 0;
+    do {
+        uint64_t q = 0;
+        out_of_memory = false;
+        allocations_left = calls++;
+        try {
+            nq_total(5, &q);
+        } catch (const std::bad_alloc &) {
+        }
+        allocations_left = -1;
+    } while (out_of_memory);
+    std::printf("%d calls\n", calls);
+    return 0;
+}
+
 int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
     nq_server_config cfg{};
     cfg.max_n = max_n;
@@ -228,6 +264,7 @@ int burst(int max_n, int stack_slots, int n, const std::vector<nq_queen> &q) {
 int main(int argc, char **argv) {
     if (argc == 2 && !std::strcmp(argv[1], "cuts")) return cuts();
     if (argc == 2 && !std::strcmp(argv[1], "shapes")) return shapes();
+    if (argc == 2 && !std::strcmp(argv[1], "nomem")) return nomem();
     if (argc == 4 && !std::strcmp(argv[1], "total"))
         return total(std::atoi(argv[2]), std::atoi(argv[3]));
     refuse_last = argc > 1 && !std::strcmp(argv[1], "refuse");

@@ -99,3 +99,8 @@ def test_total_chooses_four_rows(host, n):
     want = f"search {m} records of {min(d, 4)} rows, " if m else ""
     assert host("total", n, 0) == (want + f"rc 0, total {m}, "
                                    f"timing {nq.prefix_count(n, d)} of {d}")
+
+
+def test_a_failed_host_allocation_does_not_end_the_process(host):
+    """Whichever host allocation of a synchronous call fails, its clean-up does not throw."""
+    assert int(host("nomem").splitlines()[-1].split()[-2]) >= 3
