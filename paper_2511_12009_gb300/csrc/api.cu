@@ -5,6 +5,7 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <new>
 #include <unordered_map>
 #include <vector>
 
@@ -103,19 +104,26 @@ struct Kept {
 };
 std::mutex g_kept_mu;
 
-// The current context's entry (NULL if there is no context). Caller holds the lock.
+// The current context's entry (NULL if there is no context, or no host memory for
+// one). Caller holds the lock.
 Kept *kept_locked() {
-    static std::unordered_map<unsigned long long, Kept> *kept =
-        new std::unordered_map<unsigned long long, Kept>();  // (calls may outlive static teardown)
     unsigned long long ctx = 0;
-    return current_context_id(&ctx) == NQ_OK ? &(*kept)[ctx] : nullptr;
+    if (current_context_id(&ctx) != NQ_OK) return nullptr;
+    try {
+        static std::unordered_map<unsigned long long, Kept> *kept =
+            new std::unordered_map<unsigned long long, Kept>();  // (may outlive static teardown)
+        return &(*kept)[ctx];
+    } catch (const std::bad_alloc &) {
+        return nullptr;
+    }
 }
 
 // The library's memory pool on the current device.
 int memory_pool(cudaMemPool_t *out) {
     std::lock_guard<std::mutex> g(g_kept_mu);
     Kept *k = kept_locked();
-    if (!k) return NQ_ECUDA;
+    unsigned long long ctx = 0;
+    if (!k) return current_context_id(&ctx) == NQ_OK ? NQ_ENOMEM : NQ_ECUDA;
     if (!k->pool) {
         int dev = 0;
         cudaMemPoolProps props{};

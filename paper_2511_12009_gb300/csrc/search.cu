@@ -38,6 +38,7 @@
 #include <cstdio>
 #include <map>
 #include <mutex>
+#include <new>
 #include <tuple>
 #include <unordered_map>
 #include <utility>
@@ -1126,23 +1127,33 @@ namespace {
 // What planning asks the runtime, kept per device context (a reset or a new
 // context has another id): some dozen queries, about 10 us, on every call
 // otherwise. One entry per device, and per kernel, block size asked for and
-// stack footprint -- a few hundred at most.
+// stack footprint -- a few hundred at most. Without host memory for one it is asked
+// again.
+template <typename Map, typename Key, typename Value>
+void keep(Map &map, const Key &key, const Value &value) {
+    try {
+        map.emplace(key, value);
+    } catch (const std::bad_alloc &) {
+    }
+}
+
 int device_shape(unsigned long long ctx, int *sms, int *max_smem) {
     static std::mutex mu;
     static std::unordered_map<unsigned long long, std::pair<int, int>> shapes;
     std::lock_guard<std::mutex> g(mu);
-    auto it = shapes.find(ctx);
-    if (it == shapes.end()) {
-        int dev = 0, n = 0, m = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&m, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-                cudaSuccess)
-            return NQ_ECUDA;
-        it = shapes.emplace(ctx, std::make_pair(n, m)).first;
+    const auto it = shapes.find(ctx);
+    if (it != shapes.end()) {
+        *sms = it->second.first;
+        *max_smem = it->second.second;
+        return NQ_OK;
     }
-    *sms = it->second.first;
-    *max_smem = it->second.second;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+            cudaSuccess)
+        return NQ_ECUDA;
+    keep(shapes, ctx, std::make_pair(*sms, *max_smem));
     return NQ_OK;
 }
 
@@ -1193,7 +1204,7 @@ int resident_blocks(unsigned long long ctx, void *k, bool any_block, size_t per_
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, best, smem) != cudaSuccess)
         return NQ_ECUDA;
-    known.emplace(key, std::make_pair(best, nb));
+    keep(known, key, std::make_pair(best, nb));
     *block = best;
     *blocks = nb;
     return NQ_OK;

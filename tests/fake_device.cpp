@@ -12,7 +12,7 @@
 //   total N d    nq_total_ex in the default form (d = 0: no depth given): records
 //           launched and the rows placed in them, records and rows in the timing
 //   nomem   nq_total(5) with room for no host allocation, for one, for two, ...: the
-//           number of calls until one had enough
+//           number of calls until one had enough; nq_count_ex of new shapes with none
 //   burst max_n stack_slots N [row col]...    one request: records, answer, errors
 //   refuse max_n stack_slots N [row col]...   the same, its last record not searched
 #include <cstdio>
@@ -96,6 +96,7 @@ cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { re
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t) {
     return cudaMalloc(p, n);
 }
+cudaError_t cudaGetSymbolAddress(void **p, const void *) { return cudaMalloc(p, 1 << 20); }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return cudaFree(p); }
 CUresult get_current(CUcontext *c) { *c = reinterpret_cast<CUcontext>(8); return CUDA_SUCCESS; }
 CUresult get_id(CUcontext, unsigned long long *id) { *id = 8; return CUDA_SUCCESS; }
@@ -230,7 +231,22 @@ int nomem() {
         }
         allocations_left = -1;
     } while (out_of_memory);
-    std::printf("%d calls\n", calls);
+    // an asynchronous call's stream is known from its first; then no memory, and shapes
+    // that no call has planned yet
+    const nq_prefix root{0, 0, 0, NQ_META(1, 9, 0, 0)};
+    uint64_t counts[1], totals[32] = {};
+    nq_config cfg{};
+    int rc[3] = {1, 1, 1};  // (1: it threw)
+    for (int i = 0; i < 3; ++i) {
+        cfg.block = 32 + 32 * i;
+        if (i) allocations_left = 0;
+        try {
+            rc[i] = nq_count_ex(&root, 1, 0, 9, counts, nullptr, totals, &cfg, nullptr);
+        } catch (const std::bad_alloc &) {
+        }
+        allocations_left = -1;
+    }
+    std::printf("%d calls, count %d %d %d\n", calls, rc[0], rc[1], rc[2]);
     return 0;
 }
 
