@@ -916,11 +916,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
         }
         if (held && rem == 0u && !__any_sync(~0u, cur_slot >= 0 && !own)) let_go();
         if (need_mask == ~0u) {
-            // (plain stores to the mapped block: no atomics on host memory)
-            if (stopping) {
-                if (lane == 0) a.ctl->exit_reason = 1;
-                break;
-            }
+            if (stopping) break;
             ++idle_polls;
             if (idle_polls > a.idle_polls && !counted) {
                 if (lane == 0) atomicAdd(a.idle_warps, 1u);
@@ -935,10 +931,7 @@ __global__ void __maxnreg__(64) serve_kernel(const ServeArgs a) {
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(sw)
                                  : "l"(a.started_warps) : "memory");
                     leave = iw >= sw || (unsigned long long)idle_polls > 64ull * a.idle_polls;
-                    if (leave) {
-                        atomicExch(a.closing, 1u);
-                        a.ctl->exit_reason = 2;
-                    }
+                    if (leave) atomicExch(a.closing, 1u);
                 }
                 if (__shfl_sync(~0u, leave, 0)) break;
             }

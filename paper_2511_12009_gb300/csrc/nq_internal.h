@@ -165,7 +165,6 @@ constexpr uint32_t kServeTable = kServeGen + 4u;
 struct ServeControl {
     volatile unsigned long long head;   // records published (host writes)
     volatile int stop;                  // host asks the kernel to finish
-    volatile int exit_reason;           // kernel: 1 stopped, 2 idle timeout
     volatile int error;                 // kernel: an error it found (polls report it at once)
 };
 

@@ -108,7 +108,6 @@ int ensure_running(nq_server *s) {
         if (q != cudaSuccess) return NQ_ECUDA;
     }
     s->h_ctl->stop = 0;
-    s->h_ctl->exit_reason = 0;
     std::atomic_thread_fence(std::memory_order_seq_cst);
     nqi::ServeArgs a{};
     a.ring = s->d_ring;
@@ -219,7 +218,6 @@ extern "C" int nq_server_create(const nq_server_config *cfg, nq_server **out) {
     }
     s->h_ctl->head = 0;
     s->h_ctl->stop = 0;
-    s->h_ctl->exit_reason = 0;
     s->h_ctl->error = 0;
     for (int i = 0; i < c.request_slots; ++i) {
         s->h_done[i].seq = 0;
