@@ -469,7 +469,8 @@ def run_probe27(args, device, local):
     want = cnt.cpu().numpy().view(np.uint64).copy()
     stream = torch.cuda.current_stream(device)
     clocks = ClockSampler(local)
-    # one subtree per lane: 4096 heavy subproblems on ~10^5 resident lanes
+    # as device records: 4096 heavy subproblems on ~10^5 resident lanes (the default
+    # form splits them by itself)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     nq.count(n, d0 + extra, pre, cnt, stream)
     nq.sync(stream)
@@ -492,7 +493,7 @@ def run_probe27(args, device, local):
     e1.record(stream)
     nq.sync(stream)
     donate_ms = e0.elapsed_time(e1) / args.steps
-    # host split: each subtree expanded on the host until every lane has work
+    # as host records, through nq_count_split
     split = nq.count_split(host_pre, -1)
     clocks.start()
     runs = [nq.count_split(host_pre, -1) for _ in range(args.steps)]
@@ -735,8 +736,8 @@ def main():
     roofline = roofline_of(nodes_per_step, kern_s_max / args.steps, sms, sm_max)
     roofline["traffic"] = measured_traffic(n, d, args.layout)
 
-    # N = 22: one exact solve through the public call, timed whole (host
-    # enumeration streamed into the running search, upload, search, total back)
+    # N = 22: one exact solve through the public call, timed whole (enumeration,
+    # upload, search, total back)
     n22 = None
     if rank == 0 and not args.no_n22 and args.n == 18:
         n22 = solve_n22(args, sms, sm_max, local)

@@ -243,8 +243,8 @@ int enqueue_search(const nq_prefix *d_prefixes, uint64_t n, int expect_n, int mi
     const bool reg = p.layout == NQ_LAYOUT_REG || p.layout == NQ_LAYOUT_REGM;  // donation forms
     // Donation (its own kernel variant, planned again: its occupancy differs)
     // only when asked for: measured on GB300 it has not paid for its queue
-    // traffic yet, so batches short of work are better split on the host
-    // (nq_count_split).
+    // traffic yet, so batches short of work are better split (on the device in
+    // the default form, by nq_count_split in the others).
     const bool donate = reg && !constrained && !n_tags && !published && cfg && cfg->donate == 2;
     if (donate && (rc = make_plan(max_n, min_d, diag, constrained, cfg, &p, true))) return rc;
     if ((rc = plan_records(max_n, min_d, diag, cfg, n, !n_tags, &p, allowed))) return rc;

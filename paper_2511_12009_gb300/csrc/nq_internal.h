@@ -46,7 +46,7 @@ struct SearchArgs {
     int slots;                     // stack slots (16-byte frames) per thread
     int order;                     // 1: claim the last index first
     int claim;                     // consecutive indices a lane claims at once (>= 1)
-    // Constrained mode only (partial-board queries): the columns each row may
+    // look_kernel_masked only (partial-board queries): the columns each row may
     // take; 0 for rows >= N.
     uint32_t allowed[32];
     // Split subproblems: counts/nodes of record i are added to entry
@@ -130,7 +130,8 @@ __host__ __device__ constexpr bool layout_register_top(int layout) {
     return layout == NQ_LAYOUT_REG || layout_regm_family(layout);
 }
 
-// Constrained mode packs the row index of a frame into bits 27..31 of cols.
+// Searches under row masks pack the row index of a frame's child into bits 27..31
+// of cols.
 constexpr int kRowShift = 27;
 constexpr int kMaxConstrainedN = 26;
 

@@ -170,9 +170,8 @@ extern "C" int nq_server_create(const nq_server_config *cfg, nq_server **out) {
     nq_server_config c = *cfg;
     if (c.max_n == 0) c.max_n = 20;
     if (c.request_slots == 0) c.request_slots = 64;
-    // 13 frames: an unconstrained N = 20 request then needs depth 6 (3.0 M records,
-    // 9 % of the default ring) instead of 7 (22.8 M, 68 %: one such request at a
-    // time), at the same 3 resident blocks of 256 per SM
+    // 13 frames: 3 resident blocks of 256 per SM; an unconstrained N = 20 request makes
+    // 30,880 records of 4 rows
     if (c.stack_slots == 0) c.stack_slots = 13;
     if (c.block == 0) c.block = 256;
     if (c.ring_records == 0) c.ring_records = 1ull << 25;
@@ -187,7 +186,7 @@ extern "C" int nq_server_create(const nq_server_config *cfg, nq_server **out) {
     s->cfg = c;
     s->ring = c.ring_records;
     s->mask = c.ring_records - 1;
-    // stack frames per lane: REG layout needs max_n - 1 - d for depth d
+    // stack frames per lane: a search that starts in row d needs max_n - 1 - d
     s->min_d = std::max(0, c.max_n - 1 - c.stack_slots);
     int rc = cudaGetDevice(&s->dev) == cudaSuccess ? NQ_OK : NQ_ECUDA;
     if (!rc) {

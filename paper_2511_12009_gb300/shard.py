@@ -51,8 +51,9 @@ class CheckpointError(RuntimeError):
 def gpu_counter(device=None, config: nq.Config | None = None,
                 split: bool = False) -> Callable[[np.ndarray], np.ndarray]:
     """Per-prefix solution counts of host records, on this process's GPU.
-    split: count through nq_count_split (each record expanded a few rows on the
-    host so that a piece of few heavy subtrees still fills the GPU)."""
+    split: count through nq_count_split, so that a piece of few heavy subtrees fills
+    the GPU in every layout (the default form splits them on the device either way, the
+    others need each record expanded a few rows on the host)."""
     import torch
     dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
 

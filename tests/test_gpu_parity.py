@@ -98,12 +98,14 @@ def test_total_public_entry(n):
 
 
 @pytest.mark.parametrize("n,d", [(16, 8), (17, 6), (18, 8), (12, 9), (13, 13), (19, 4), (11, 1)])
-def test_total_ex_pieces(n, d):
+@pytest.mark.parametrize("layout", ["default", "regm"])
+def test_total_ex_pieces(n, d, layout):
     """nq_total_ex writes, uploads and searches large prefix sets in pieces
-    (heaviest first, one stream each); small sets in one piece. Every depth,
-    including the deepest (the whole board placed) and one row (odd N: the centre prefix
-    alone has weight 1), gives Q(N)."""
-    r = nq.total_ex(n, nq.make_config(d=d))
+    (heaviest first, the search running meanwhile) in the register-top layouts, and in
+    one go in the default form; small sets in one piece. Every depth, including the
+    deepest (the whole board placed) and one row (odd N: the centre prefix alone has
+    weight 1), gives Q(N)."""
+    r = nq.total_ex(n, nq.make_config(layout, d=d))
     assert r["total"] == Q[n] and r["prefixes"] == nq.prefix_count(n, d)
 
 
@@ -431,7 +433,7 @@ def test_split_word_layouts_need_256_thread_blocks():
 @pytest.mark.parametrize("layout", ["regp", "regz", "regpz"])
 def test_streamed_total_new_layouts(layout):
     """nq_total_ex streams N=18's d=7 set (7.4 M records) into the running search
-    in every register-top layout."""
+    in the register-top layouts, and searches it after its upload in the default form."""
     r = nq.total_ex(18, nq.make_config(layout, d=7))
     assert r["total"] == Q[18] and r["layout"] == nq.LAYOUTS[layout]
 

@@ -154,9 +154,9 @@ def test_board_symmetry_served(seed):
 
 def test_served_split_edges(orc):
     """Boards that end within the split levels, rows fixed from the top (more than
-    a level each), full solutions, the widest board, and a small stack that forces
-    deep prefixes, all in one burst; every answer equals the standalone count, and
-    a second burst on the same slots (new generations) too."""
+    a level each), full solutions and the widest board, at two stack sizes, all in one
+    burst; every answer equals the standalone count, and a second burst on the same
+    slots (new generations) too."""
     from paper_2511_12009_gb300.serve import Server, run_stream
     sol26 = [c - 1 for c in list(range(2, 27, 2)) + [3, 1, 7, 9, 11, 13, 15, 17, 19, 21, 23, 25, 5]]
     reqs = [(1, []), (2, []), (3, []), (4, []), (5, [(0, 0)]), (6, []), (8, [(7, 3)]),

@@ -388,10 +388,12 @@ def test_look_ahead_sentinel_holds_32_idle_steps():
 # --- work split below a record (lookahead.cu) -----------------------------------------
 
 def digit_bits(free_columns, last):
-    b = 1
+    """Bits of a level's digit as the planner gives them: one for every column that could
+    be free, none for a row with one; of the server's last level 2 at most."""
+    b = 0
     while (1 << b) < free_columns:
         b += 1
-    return 2 if last else b
+    return min(b, 2) if last else b
 
 
 def split_unit(s, bits, c, l, r):
